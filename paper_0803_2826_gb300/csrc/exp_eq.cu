@@ -135,7 +135,7 @@ __device__ __forceinline__ void collide_exp(const float m[19], float fx, float f
     for (int k = 16; k < 19; ++k) M[k] = lbd::inv_w(k) * (meq[k] + a.g_even * (m[k] - meq[k]));
     if (NOISE) {
         float g[16];
-        lbd::gaussians16(a.rk, node, a.step, 0u, a.replica, a.mu * (a.noise_rho0 ? a.rho0 : rho), g);
+        lbd::gaussians16(a.rk, node, a.step, 0u, a.replica, sqrtf(a.mu * (a.noise_rho0 ? a.rho0 : rho)), g);
 #pragma unroll
         for (int k = 4; k < 19; ++k) M[k] = fmaf(a.amp[k - 4], g[k - 4], M[k]);
     }
@@ -315,14 +315,14 @@ __device__ __forceinline__ void collide_exp2(const F2 m[19], F2 fx, F2 fy, F2 fz
 #pragma unroll
     for (int k = 16; k < 19; ++k) M[k] = lbp::fma2(lbp::f2s(a.g_even), m[k] - meq[k], meq[k]) * lbd::inv_w(k);
     if (NOISE) {
-        const F2 var = a.noise_rho0 ? lbp::f2s(a.mu * a.rho0) : rho * a.mu;
+        const F2 sd = lbp::noise_sd(a, rho);
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
             const lbd::U4 r0 = lbd::philox10(lbd::U4{node0, a.step, (uint32_t)b, a.replica}, a.rk);
             const lbd::U4 r1 = lbd::philox10(lbd::U4{node0 + 1u, a.step, (uint32_t)b, a.replica}, a.rk);
             F2 g[4];
-            lbp::box_muller2(r0.x, r0.y, r1.x, r1.y, g[0], g[1], var);
-            lbp::box_muller2(r0.z, r0.w, r1.z, r1.w, g[2], g[3], var);
+            lbp::box_muller2(r0.x, r0.y, r1.x, r1.y, g[0], g[1], sd);
+            lbp::box_muller2(r0.z, r0.w, r1.z, r1.w, g[2], g[3], sd);
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const int k = 4 + 4 * b + j;

@@ -183,20 +183,19 @@ __device__ __forceinline__ void backward2(const F2 M[19], F2 n[19])
 // Box-Muller pairs of the two nodes (words (a0, b0) of node x0, (a1, b1) of
 // node x0 + 1): the map of lbd::box_muller -- uniforms (2 (w >> 9) + 1) 2^-24
 // from the mantissa bits, -2 ln v1 from the hardware log2 or the series near
-// 1, the radius sqrt(-2 ln v1 var) as L rsqrt(L), the centred angle -- with
+// 1, the radius sqrt(-2 ln v1) sd as L rsqrt(L) sd, the centred angle -- with
 // the FP32 arithmetic packed and the special functions per half.
 __device__ __forceinline__ void box_muller2(uint32_t a0, uint32_t b0, uint32_t a1, uint32_t b1, F2 &g0, F2 &g1,
-                                            F2 var)
+                                            F2 sd)
 {
     const F2 off = f2s(0.99999994039535522f);
-    const F2 v1 = f2(__uint_as_float(0x3F800000u | (a0 >> 9)), __uint_as_float(0x3F800000u | (a1 >> 9))) - off;
+    const F2 v1 = f2(lbd::one_to_two(a0), lbd::one_to_two(a1)) - off;
     const F2 d1 = f2s(1.0f) - v1;
-    const F2 w = (f2(__uint_as_float(0x3F800000u | (b0 >> 9)), __uint_as_float(0x3F800000u | (b1 >> 9))) - off) -
-                 f2s(0.5f);
+    const F2 w = (f2(lbd::one_to_two(b0), lbd::one_to_two(b1)) - off) - f2s(0.5f);
     float v1l, v1h, d1l, d1h;
     split(v1, v1l, v1h);
     split(d1, d1l, d1h);
-    const F2 lg = f2(__log2f(v1l), __log2f(v1h)) * f2s(-1.3862943611198906f);
+    const F2 lg = f2(lbd::log2_normal(v1l), lbd::log2_normal(v1h)) * f2s(-1.3862943611198906f);
     F2 t = fma2(d1, f2s(1.0f / 6.0f), f2s(0.2f));
     t = fma2(d1, t, f2s(0.25f));
     t = fma2(d1, t, f2s(1.0f / 3.0f));
@@ -206,10 +205,10 @@ __device__ __forceinline__ void box_muller2(uint32_t a0, uint32_t b0, uint32_t a
     float sl, sh, ll, lh;
     split(ser, sl, sh);
     split(lg, ll, lh);
-    const F2 L = f2(d1l < 0.03125f ? sl : ll, d1h < 0.03125f ? sh : lh) * var;
+    const F2 L = f2(d1l < 0.03125f ? sl : ll, d1h < 0.03125f ? sh : lh);
     float Ll, Lh;
     split(L, Ll, Lh);
-    const F2 nr = L * f2(-rsqrtf(Ll), -rsqrtf(Lh));  // -sqrt(L)
+    const F2 nr = L * f2(-lbd::rsqrt_normal(Ll), -lbd::rsqrt_normal(Lh)) * sd;  // -sqrt(L) sd
     const F2 ang = w * f2s(6.283185307179586f);
     float al, ah, s0, c0, s1, c1;
     split(ang, al, ah);
@@ -217,6 +216,15 @@ __device__ __forceinline__ void box_muller2(uint32_t a0, uint32_t b0, uint32_t a
     __sincosf(ah, &s1, &c1);
     g0 = nr * f2(c0, c1);
     g1 = nr * f2(s0, s1);
+}
+
+// sqrt(mu rho) of both nodes (mu rho0 where the amplitude is the reference's).
+__device__ __forceinline__ F2 noise_sd(const lbi::StepArgs &a, F2 rho)
+{
+    if (a.noise_rho0) return f2s(sqrtf(a.mu * a.rho0));
+    float l, h;
+    split(rho * a.mu, l, h);
+    return f2(sqrtf(l), sqrtf(h));
 }
 
 // Where collide_moments2 takes its Philox round keys: ParamKeys reads the
@@ -305,15 +313,15 @@ __device__ __forceinline__ void collide_moments2k(const F2 m[19], F2 fx, F2 fy, 
         // sqrt(mu rho w_k) phi_k r_k / w_k: (phi_k / sqrt(w_k)) times a Gaussian
         // of variance mu rho; the four Gaussians of each Philox block go into
         // their modes at once (r_4 .. r_18 = Gaussians 0 .. 14)
-        const F2 var = a.noise_rho0 ? f2s(a.mu * a.rho0) : rho * a.mu;
+        const F2 sd = noise_sd(a, rho);
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
             lbd::U4 r0, r1;
             keys.pair(lbd::U4{node0, a.step, (uint32_t)b, replica}, lbd::U4{node0 + 1u, a.step, (uint32_t)b, replica},
                       r0, r1);
             F2 g[4];
-            box_muller2(r0.x, r0.y, r1.x, r1.y, g[0], g[1], var);
-            box_muller2(r0.z, r0.w, r1.z, r1.w, g[2], g[3], var);
+            box_muller2(r0.x, r0.y, r1.x, r1.y, g[0], g[1], sd);
+            box_muller2(r0.z, r0.w, r1.z, r1.w, g[2], g[3], sd);
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const int k = 4 + 4 * b + j;

@@ -77,7 +77,7 @@ __device__ __forceinline__ void collide_moments(const float m[19], float fx, flo
         // sqrt(mu rho w_k) phi_k r_k, divided by w_k: (phi_k / sqrt(w_k)) times a
         // Gaussian of variance mu rho (the factor rides in the Box-Muller radius)
         float g[16];
-        lbd::gaussians16(rk, node, a.step, 0u, replica, a.mu * (a.noise_rho0 ? a.rho0 : rho), g);
+        lbd::gaussians16(rk, node, a.step, 0u, replica, sqrtf(a.mu * (a.noise_rho0 ? a.rho0 : rho)), g);
 #pragma unroll
         for (int k = 4; k < 19; ++k) M[k] = fmaf(a.amp[k - 4], g[k - 4], M[k]);
     }
