@@ -63,6 +63,8 @@ StepArgs make_args(const lb_handle *h)
     a.z1 = p.walls ? p.nz - 1 : p.nz;
     a.pitch = h->pitch;
     a.nn = h->n_nodes;
+    a.dnx = h->dnx;
+    a.dny = h->dny;
     a.rho0 = (float)p.rho0;
     a.kT = (float)p.kT;
     a.mu = (float)(p.kT * 3.0);
@@ -315,6 +317,8 @@ lb_status lb_create(const lb_params *p, void *pops_a, void *pops_b, float *force
     h->n_nodes = (size_t)p->nx * p->ny * p->nz;
     h->pitch = lb_plane_pitch(p);
     h->elem = elem_size(p->dtype);
+    h->dnx = make_div((uint32_t)p->nx);
+    h->dny = make_div((uint32_t)p->ny);
     h->pops[0] = pops_a;
     h->pops[1] = pops_b;
     h->cur = 0;

@@ -36,35 +36,6 @@
 namespace lbi {
 namespace {
 
-// Unsigned division by a run-time constant (round-up method of Granlund and
-// Montgomery, "Division by invariant integers using multiplication", 1994).
-struct Div {
-    uint32_t m, s, d;  // d == 1: identity
-};
-
-Div make_div(uint32_t d)
-{
-    Div v;
-    v.d = d;
-    if (d <= 1) {
-        v.m = 0;
-        v.s = 0;
-        return v;
-    }
-    uint32_t l = 0;
-    while ((1ull << l) < d) ++l;
-    v.m = (uint32_t)((((1ull << l) - d) << 32) / d + 1);
-    v.s = l - 1;
-    return v;
-}
-
-__device__ __forceinline__ uint32_t divide(uint32_t n, const Div &v)
-{
-    if (v.d <= 1) return n;
-    const uint32_t t = __umulhi(v.m, n);
-    return (t + ((n - t) >> 1)) >> v.s;
-}
-
 struct BatchDesc {
     int nx, ny, nz;
     uint32_t nodes;
@@ -594,6 +565,8 @@ void replica_view(lb_batch *b, int r, lb_handle &h)
     h.p = b->rep_params[r];
     h.n_nodes = b->desc_h[r].nodes;
     h.pitch = b->desc_h[r].pitch;
+    h.dnx = make_div((uint32_t)h.p.nx);
+    h.dny = make_div((uint32_t)h.p.ny);
     h.elem = b->elem;
     for (int k = 0; k < 2; ++k) h.pops[k] = (char *)b->pops[k] + b->desc_h[r].off * b->elem;
     h.cur = b->cur;

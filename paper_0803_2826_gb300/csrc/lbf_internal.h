@@ -33,6 +33,7 @@ struct lb_handle {
     size_t n_nodes;
     size_t pitch;
     size_t elem;          // bytes per stored population value
+    lbi::Div dnx, dny;    // division by the box edges
     void *pops[2];        // borrowed
     int cur;              // pops[cur] holds the current state
     float *force;         // borrowed, nullable

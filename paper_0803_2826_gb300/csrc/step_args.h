@@ -10,6 +10,30 @@
 
 namespace lbi {
 
+// Unsigned division by a run-time constant (round-up method of Granlund and
+// Montgomery, "Division by invariant integers using multiplication", 1994).
+struct Div {
+    uint32_t m, s, d;  // d <= 1: identity
+};
+
+inline Div make_div(uint32_t d)
+{
+    Div v{0, 0, d};
+    if (d <= 1) return v;
+    uint32_t l = 0;
+    while ((1ull << l) < d) ++l;
+    v.m = (uint32_t)((((1ull << l) - d) << 32) / d + 1);
+    v.s = l - 1;
+    return v;
+}
+
+__device__ __forceinline__ uint32_t divide(uint32_t n, const Div &v)
+{
+    if (v.d <= 1) return n;
+    const uint32_t t = __umulhi(v.m, n);
+    return (t + ((n - t) >> 1)) >> v.s;
+}
+
 // Geometry and physics constants a kernel launch needs, in FP32 where the
 // kernels compute in FP32.
 struct StepArgs {
@@ -17,6 +41,7 @@ struct StepArgs {
     int z0, z1;            // fluid z-range [z0, z1)
     size_t pitch;          // elements per population plane
     size_t nn;             // nodes nx*ny*nz (component stride of caller fields)
+    Div dnx, dny;          // division by nx and ny (node index -> coordinates)
     float rho0;
     float kT;
     float mu;              // kT / c_s^2

@@ -1,9 +1,17 @@
 // stream_collide.cuh -- fused pull-stream + MRT collision + noise + forcing.
 //
-// One thread per fluid node; a block covers BX consecutive x of one (y, z)
-// row, so the 19 plane loads and 19 plane stores of a warp are coalesced
-// (the +-x neighbours of a row are the same 32-byte sectors shifted by one
-// element).  Everything between the loads and the stores stays in registers:
+// Two consecutive nodes per thread in packed FP32 (f32x2.cuh); the 19 plane
+// loads and 19 plane stores of a warp are coalesced (the +-x neighbours of a
+// row are the same 32-byte sectors shifted by one element).  Threads map to
+// the nodes in one of two ways.  Rows whose pairs fill whole blocks (nx a
+// multiple of 256) keep one row per block: no division, y and z from the
+// block index (k_stream_collide2; 256^3 FP32 with noise 383 us a step against
+// 389 us in the linear mapping).  All other boxes run over the linear node
+// index (k_stream_collide_linear), so no lane is idle however short or odd the
+// rows are: 64^3 10.3 us against 12.3 us with a block per row, 200^3 189 us
+// against 248 us, and rows of odd length, which went one node a thread in
+// scalar arithmetic before, 257 x 131 x 129 BF16 between walls 121 us against
+// 170 us.  Everything between the loads and the stores stays in registers:
 //   pull       n_i(r) = n*_i(r - c_i)                       Eq. (LBE)
 //              (link bounce-back at solid z-planes,          Sec. 4.1 Eq. (MBB), u_b = 0)
 //   moments    m_k = sum_i e_ki n_i                          Sec. 3.4 Eq. (forward), Table 1
@@ -21,6 +29,10 @@
 namespace lbi {
 
 constexpr int kBX = 128;  // threads per block along x
+// Threads per block of the linear mapping: small boxes then still spread over
+// the SMs (16^3: 4.1 us a step with 64, 5.6 us with 128; no difference from
+// 64^3 on).
+constexpr int kLinBX = 64;
 
 
 // Collision of one node (Sec. 3.4, 3.5, 3.7) from its pulled populations n
@@ -167,14 +179,11 @@ __device__ __forceinline__ void block_moment_sums_out(const float (*part)[38], f
 }
 
 // The whole update of fluid node (x, y, z): pull, force, collision, store.
-// SUMS: the warp's moment sums go to part (see warp_moment_sums); every
-// lane calls, lanes without a node (valid false) add zeros.
-template <int DT, bool NOISE, bool FIELD, bool WALLS, bool SUMS = false>
+template <int DT, bool NOISE, bool FIELD, bool WALLS>
 __device__ __forceinline__ void update_node(const typename lbd::Store<DT>::T *__restrict__ src,
                                             typename lbd::Store<DT>::T *__restrict__ dst,
                                             const float *__restrict__ ffield, const float *__restrict__ facc,
-                                            const StepArgs &a, int x, int y, int z, bool valid = true,
-                                            float (*part)[38] = nullptr)
+                                            const StepArgs &a, int x, int y, int z)
 {
     using S = lbd::Store<DT>;
     const int nx = a.nx, ny = a.ny, nz = a.nz;
@@ -223,44 +232,10 @@ __device__ __forceinline__ void update_node(const typename lbd::Store<DT>::T *__
     }
     float m[19], out[19];
     lbd::forward(n, m);
-    if (SUMS) {
-        float none[19];
-#pragma unroll
-        for (int k = 0; k < 19; ++k) none[k] = 0.0f;
-        warp_moment_sums(m, none, valid, part);
-    }
-    if (!valid) return;
     collide_moments<NOISE>(m, fx, fy, fz, a, a.rk, self, a.replica, out);
 #pragma unroll
     for (int i = 0; i < 19; ++i)
         if (in_bounds((size_t)i * P + self, 19 * P, a.err)) dst[(size_t)i * P + self] = S::pack(out[i], a.scale);
-}
-
-__device__ __forceinline__ size_t block_linear()
-{
-    return blockIdx.x + (size_t)gridDim.x * (blockIdx.y + (size_t)gridDim.y * blockIdx.z);
-}
-
-// SUMS: the block also writes the moment sums of its nodes (pre-collision,
-// as lb_moments defines them) to partials[block][38].
-template <int DT, bool NOISE, bool FIELD, bool WALLS, bool SUMS>
-__global__ void __launch_bounds__(kBX) k_stream_collide(const typename lbd::Store<DT>::T *__restrict__ src,
-                                                        typename lbd::Store<DT>::T *__restrict__ dst,
-                                                        const float *__restrict__ ffield,
-                                                        const float *__restrict__ facc, const StepArgs a,
-                                                        float *partials)
-{
-    const int x = blockIdx.x * kBX + threadIdx.x;
-    if (SUMS) {
-        __shared__ float part[kBX / 32][38];
-        const bool valid = x < a.nx;  // lanes past the row load node 0 of it and store nothing
-        update_node<DT, NOISE, FIELD, WALLS, true>(src, dst, ffield, facc, a, valid ? x : 0, blockIdx.y,
-                                                   blockIdx.z + a.z0, valid, part);
-        block_moment_sums_out(part, partials + 38 * block_linear());
-    } else {
-        if (x >= a.nx) return;
-        update_node<DT, NOISE, FIELD, WALLS>(src, dst, ffield, facc, a, x, blockIdx.y, blockIdx.z + a.z0);
-    }
 }
 
 // Node k (0 .. span^3 - 1, x fastest) of the block of nodes that an impulse
@@ -559,13 +534,12 @@ template <int DT>
 __device__ __forceinline__ void store_pair(typename lbd::Store<DT>::T *__restrict__ dst, const StepArgs &a,
                                            uint32_t self, const lbp::F2 out[19])
 {
-    const uint32_t P = (uint32_t)a.pitch;
-    const size_t lim = 19 * (size_t)P;
+    const size_t P = a.pitch;
 #pragma unroll
     for (int i = 0; i < 19; ++i) {
         float o0, o1;
         lbp::split(DT == 0 ? out[i] : out[i] * lbp::f2s(a.scale), o0, o1);
-        if (in_bounds((uint32_t)i * P + self + 1, lim, a.err)) Pair<DT>::store(dst + (uint32_t)i * P + self, o0, o1, 1.0f);
+        if (in_bounds((size_t)i * P + self + 1, 19 * P, a.err)) Pair<DT>::store(dst + (size_t)i * P + self, o0, o1, 1.0f);
     }
 }
 
@@ -596,6 +570,14 @@ __device__ __forceinline__ void update_pair(const typename lbd::Store<DT>::T *__
     store_pair<DT>(dst, a, self, out);
 }
 
+// Rows mapped to blocks: block (x, y, z) takes 2 kBX consecutive nodes of row
+// (y, z).  SUMS: the block also writes the moment sums of its nodes
+// (pre-collision, as lb_moments defines them) to partials[block][38].
+__device__ __forceinline__ size_t block_linear()
+{
+    return blockIdx.x + (size_t)gridDim.x * (blockIdx.y + (size_t)gridDim.y * blockIdx.z);
+}
+
 template <int DT, bool NOISE, bool FIELD, bool WALLS, bool SUMS>
 __global__ void __launch_bounds__(kBX) k_stream_collide2(const typename lbd::Store<DT>::T *__restrict__ src,
                                                          typename lbd::Store<DT>::T *__restrict__ dst,
@@ -616,6 +598,225 @@ __global__ void __launch_bounds__(kBX) k_stream_collide2(const typename lbd::Sto
     }
 }
 
+// Two consecutive nodes s, s + 1 (s even) per thread over the fluid's linear
+// index range, for boxes whose rows do not fill whole blocks of pairs: every
+// lane of every warp but the last has its two nodes, whatever nx.  In a row
+// of even length both nodes lie in the same row (load_pair); in one of odd
+// length the pair may straddle two rows, or the wall and the fluid, so each
+// node takes its own addresses and only the store moves the pair as one
+// access.  va / vb: the node lies in the fluid (the first pair of a channel
+// with an odd plane, the last of an odd number of nodes).
+struct PairAt {
+    uint32_t s;
+    int x, y, z;    // node s, or s + 1 where only that one is fluid
+    bool va, vb;
+};
+
+template <bool WALLS>
+__device__ __forceinline__ bool locate_pair(const StepArgs &a, PairAt &p)
+{
+    const uint32_t plane = (uint32_t)a.nx * (uint32_t)a.ny;
+    const uint32_t first = WALLS ? plane : 0u;
+    const uint32_t end = (uint32_t)a.nn - first;
+    p.s = (first & ~1u) + 2u * (blockIdx.x * (uint32_t)kLinBX + threadIdx.x);
+    if (p.s >= end) return false;
+    p.va = !WALLS || p.s >= first;
+    p.vb = p.s + 1u < end;
+    const uint32_t s = p.va ? p.s : p.s + 1u;
+    const uint32_t row = divide(s, a.dnx);
+    const uint32_t z = divide(row, a.dny);
+    p.x = (int)(s - row * (uint32_t)a.nx);
+    p.y = (int)(row - z * (uint32_t)a.ny);
+    p.z = (int)z;
+    return true;
+}
+
+// Pull addresses of one node: row offsets of its neighbours and their x.
+struct PullAt {
+    int x[3];          // x - 1, x, x + 1 (wrapped)
+    uint32_t y[3], z[3];  // row offsets y nx and plane offsets z nx ny, the same way
+    uint32_t self;
+    bool lo, hi;       // next to the lower / upper wall: c_z = +1 / -1 bounce back
+};
+
+template <bool WALLS>
+__device__ __forceinline__ PullAt pull_at(const StepArgs &a, int x, int y, int z)
+{
+    PullAt p;
+    p.x[0] = x == 0 ? a.nx - 1 : x - 1;
+    p.x[1] = x;
+    p.x[2] = x == a.nx - 1 ? 0 : x + 1;
+    const uint32_t nx = (uint32_t)a.nx, pl = nx * (uint32_t)a.ny;
+    p.y[0] = (uint32_t)(y == 0 ? a.ny - 1 : y - 1) * nx;
+    p.y[1] = (uint32_t)y * nx;
+    p.y[2] = (uint32_t)(y == a.ny - 1 ? 0 : y + 1) * nx;
+    if (WALLS) {
+        p.lo = z == a.z0;
+        p.hi = z == a.z1 - 1;
+        p.z[0] = (uint32_t)(z - 1) * pl;
+        p.z[2] = (uint32_t)(z + 1) * pl;
+    } else {
+        p.lo = p.hi = false;
+        p.z[0] = (uint32_t)(z == 0 ? a.nz - 1 : z - 1) * pl;
+        p.z[2] = (uint32_t)(z == a.nz - 1 ? 0 : z + 1) * pl;
+    }
+    p.z[1] = (uint32_t)z * pl;
+    p.self = p.z[1] + p.y[1] + (uint32_t)x;
+    return p;
+}
+
+// Population i as pulled by the node (stored value, FP16 / BF16 still scaled).
+template <int DT, bool WALLS>
+__device__ __forceinline__ float pull_one(const typename lbd::Store<DT>::T *__restrict__ src, const StepArgs &a,
+                                          const PullAt &p, int i)
+{
+    const uint32_t off = p.z[1 - lbd::cz(i)] + p.y[1 - lbd::cy(i)] + (uint32_t)p.x[1 - lbd::cx(i)];
+    const bool bounce = WALLS && ((lbd::cz(i) == 1 && p.lo) || (lbd::cz(i) == -1 && p.hi));
+    const size_t k = WALLS && bounce ? (size_t)lbd::opposite(i) * a.pitch + p.self : (size_t)i * a.pitch + off;
+    return in_bounds(k, 19 * a.pitch, a.err) ? lbd::Store<DT>::load(src + k, 1.0f) : 0.0f;
+}
+
+template <int DT, bool FIELD, bool WALLS>
+__device__ __forceinline__ void load_pair_any(const typename lbd::Store<DT>::T *__restrict__ src,
+                                              const float *__restrict__ ffield, const float *__restrict__ facc,
+                                              const StepArgs &a, const PairAt &at, lbp::F2 n[19], float f0[3],
+                                              float f1[3])
+{
+    int xb = at.x, yb = at.y, zb = at.z;  // node s + 1; the located node where there is only one
+    if (at.va && at.vb) {
+        xb += 1;
+        if (xb == a.nx) {
+            xb = 0;
+            yb += 1;
+            if (yb == a.ny) {
+                yb = 0;
+                zb += 1;
+            }
+        }
+    }
+    const PullAt pa = pull_at<WALLS>(a, at.x, at.y, at.z), pb = pull_at<WALLS>(a, xb, yb, zb);
+#pragma unroll
+    for (int i = 0; i < 19; ++i) {
+        const lbp::F2 v = lbp::f2(pull_one<DT, WALLS>(src, a, pa, i), pull_one<DT, WALLS>(src, a, pb, i));
+        n[i] = DT == 0 ? v : v * lbp::f2s(a.inv_scale);
+    }
+    f0[0] = f1[0] = a.fx;
+    f0[1] = f1[1] = a.fy;
+    f0[2] = f1[2] = a.fz;
+    if (FIELD) {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            if (ffield) {  // caller's field, component stride N
+                f0[d] += __ldg(ffield + d * a.nn + pa.self);
+                f1[d] += __ldg(ffield + d * a.nn + pb.self);
+            }
+            if (facc) {  // library accumulator, component stride = plane pitch
+                f0[d] += __ldg(facc + d * a.pitch + pa.self);
+                f1[d] += __ldg(facc + d * a.pitch + pb.self);
+            }
+        }
+    }
+}
+
+// The store of one node of the pair.
+template <int DT>
+__device__ __forceinline__ void store_one(typename lbd::Store<DT>::T *__restrict__ dst, const StepArgs &a, uint32_t s,
+                                          const lbp::F2 out[19], bool second)
+{
+#pragma unroll
+    for (int i = 0; i < 19; ++i) {
+        const float o = second ? lbp::hi(out[i]) : lbp::lo(out[i]);
+        const size_t k = (size_t)i * a.pitch + s;
+        if (in_bounds(k, 19 * a.pitch, a.err)) dst[k] = lbd::Store<DT>::pack(o, a.scale);
+    }
+}
+
+// The pair's store; a lone node (va or vb false) is stored by itself.
+template <int DT>
+__device__ __forceinline__ void store_pair_any(typename lbd::Store<DT>::T *__restrict__ dst, const StepArgs &a,
+                                               const PairAt &at, const lbp::F2 out[19])
+{
+    if (at.va && at.vb) {
+        store_pair<DT>(dst, a, at.s, out);
+        return;
+    }
+    store_one<DT>(dst, a, at.va ? at.s : at.s + 1u, out, !at.va);
+}
+
+template <int DT, bool FIELD, bool WALLS, bool ODD>
+__device__ __forceinline__ void load_linear(const typename lbd::Store<DT>::T *__restrict__ src,
+                                            const float *__restrict__ ffield, const float *__restrict__ facc,
+                                            const StepArgs &a, const PairAt &at, lbp::F2 n[19], float f0[3],
+                                            float f1[3])
+{
+    if (ODD)
+        load_pair_any<DT, FIELD, WALLS>(src, ffield, facc, a, at, n, f0, f1);
+    else
+        load_pair<DT, FIELD, WALLS>(src, ffield, facc, a, at.x, at.y, at.z, n, f0, f1);
+}
+
+template <int DT, bool NOISE, bool FIELD, bool WALLS, bool ODD>
+__global__ void __launch_bounds__(kLinBX) k_stream_collide_linear(const typename lbd::Store<DT>::T *__restrict__ src,
+                                                               typename lbd::Store<DT>::T *__restrict__ dst,
+                                                               const float *__restrict__ ffield,
+                                                               const float *__restrict__ facc, const StepArgs a)
+{
+    PairAt at;
+    if (!locate_pair<WALLS>(a, at)) return;
+    lbp::F2 n[19], m[19], out[19];
+    float f0[3], f1[3];
+    load_linear<DT, FIELD, WALLS, ODD>(src, ffield, facc, a, at, n, f0, f1);
+    lbp::forward2(n, m);
+    lbp::collide_moments2<NOISE>(m, lbp::f2(f0[0], f1[0]), lbp::f2(f0[1], f1[1]), lbp::f2(f0[2], f1[2]), a, a.rk, at.s,
+                                 a.replica, out);
+    if (ODD)
+        store_pair_any<DT>(dst, a, at, out);
+    else
+        store_pair<DT>(dst, a, at.s, out);
+}
+
+// The step with moment sums on boxes whose pairs cannot move as one access
+// (rows of odd length, or more elements than 32-bit indices reach): rows mapped to blocks
+// as in k_stream_collide2, the pair's addresses and stores one node at a time,
+// the last node of an odd row alone.  The arithmetic is the pair's, so the
+// populations are those of k_stream_collide_linear bit for bit.
+template <int DT, bool NOISE, bool FIELD, bool WALLS>
+__global__ void __launch_bounds__(kBX) k_stream_collide_sums_any(const typename lbd::Store<DT>::T *__restrict__ src,
+                                                                 typename lbd::Store<DT>::T *__restrict__ dst,
+                                                                 const float *__restrict__ ffield,
+                                                                 const float *__restrict__ facc, const StepArgs a,
+                                                                 float *partials)
+{
+    __shared__ float part[kBX / 32][38];
+    const int x0 = 2 * (blockIdx.x * kBX + threadIdx.x);
+    const bool mine = x0 < a.nx;  // lanes past the row load its first nodes and store nothing
+    PairAt at;
+    at.x = mine ? x0 : 0;
+    at.y = blockIdx.y;
+    at.z = blockIdx.z + a.z0;
+    at.s = (uint32_t)((at.z * a.ny + at.y) * a.nx + at.x);
+    at.va = true;
+    at.vb = at.x + 1 < a.nx;
+    lbp::F2 n[19], m[19], out[19];
+    float f0[3], f1[3];
+    load_pair_any<DT, FIELD, WALLS>(src, ffield, facc, a, at, n, f0, f1);
+    lbp::forward2(n, m);
+    float m0[19], m1[19];
+#pragma unroll
+    for (int k = 0; k < 19; ++k) {
+        lbp::split(m[k], m0[k], m1[k]);
+        if (!at.vb) m1[k] = 0.0f;
+    }
+    warp_moment_sums(m0, m1, mine, part);
+    if (mine) {
+        lbp::collide_moments2<NOISE>(m, lbp::f2(f0[0], f1[0]), lbp::f2(f0[1], f1[1]), lbp::f2(f0[2], f1[2]), a, a.rk,
+                                     at.s, a.replica, out);
+        store_one<DT>(dst, a, at.s, out, false);
+        if (at.vb) store_one<DT>(dst, a, at.s + 1u, out, true);
+    }
+    block_moment_sums_out(part, partials + 38 * block_linear());
+}
+
 // Launch geometry of the stream-collide kernels: two nodes per thread when
 // rows pair up and element indices fit 32 bits.
 inline bool sc_paired(const lb_handle *h)
@@ -626,8 +827,7 @@ inline bool sc_paired(const lb_handle *h)
 inline dim3 sc_grid(const lb_handle *h)
 {
     const int nzf = h->p.walls ? h->p.nz - 2 : h->p.nz;
-    const int nxt = sc_paired(h) ? h->p.nx / 2 : h->p.nx;
-    return dim3((nxt + kBX - 1) / kBX, h->p.ny, nzf);
+    return dim3(((h->p.nx + 1) / 2 + kBX - 1) / kBX, h->p.ny, nzf);
 }
 
 // partials != NULL: the launch also writes per-block moment sums
@@ -646,6 +846,10 @@ cudaError_t launch_stream_collide_dt(const lb_handle *h, const void *src, void *
     const bool paired = sc_paired(h);
     const T *s = static_cast<const T *>(src);
     T *d = static_cast<T *>(dst);
+    const bool rows = !partials && paired && (h->p.nx / 2) % kBX == 0;
+    const bool odd = !paired;
+    const uint32_t first = walls ? (uint32_t)(a.nx * a.ny) : 0u;
+    const dim3 linear((unsigned)(((a.nn - first - (first & ~1u) + 1) / 2 + kLinBX - 1) / kLinBX));
 #define LBI_SC(NZ, FL, WL)                                                                                        \
     do {                                                                                                          \
         if (partials) {                                                                                           \
@@ -653,15 +857,17 @@ cudaError_t launch_stream_collide_dt(const lb_handle *h, const void *src, void *
                 k_stream_collide2<DT, NZ, FL, WL, true><<<grid, block, 0, h->stream>>>(s, d, h->force, facc, a,   \
                                                                                         partials);               \
             else                                                                                                  \
-                k_stream_collide<DT, NZ, FL, WL, true><<<grid, block, 0, h->stream>>>(s, d, h->force, facc, a,    \
-                                                                                       partials);                \
+                k_stream_collide_sums_any<DT, NZ, FL, WL><<<grid, block, 0, h->stream>>>(s, d, h->force, facc, a, \
+                                                                                         partials);              \
+        } else if (rows) {                                                                                        \
+            k_stream_collide2<DT, NZ, FL, WL, false><<<grid, block, 0, h->stream>>>(s, d, h->force, facc, a,      \
+                                                                                     nullptr);                   \
+        } else if (odd) {                                                                                         \
+            k_stream_collide_linear<DT, NZ, FL, WL, true><<<linear, kLinBX, 0, h->stream>>>(s, d, h->force, facc,  \
+                                                                                           a);                   \
         } else {                                                                                                  \
-            if (paired)                                                                                           \
-                k_stream_collide2<DT, NZ, FL, WL, false><<<grid, block, 0, h->stream>>>(s, d, h->force, facc, a,  \
-                                                                                         nullptr);               \
-            else                                                                                                  \
-                k_stream_collide<DT, NZ, FL, WL, false><<<grid, block, 0, h->stream>>>(s, d, h->force, facc, a,   \
-                                                                                        nullptr);                \
+            k_stream_collide_linear<DT, NZ, FL, WL, false><<<linear, kLinBX, 0, h->stream>>>(s, d, h->force, facc, \
+                                                                                            a);                  \
         }                                                                                                         \
     } while (0)
     if (noise) {
