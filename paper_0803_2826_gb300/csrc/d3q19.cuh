@@ -19,6 +19,8 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include "chain.cuh"
+
 namespace lbd {
 
 // Weights a^{c_i} (Sec. 3.3) and norms w_k (Table 1).
@@ -350,7 +352,7 @@ struct Store;
 template <>
 struct Store<0> {
     using T = float;
-    static __device__ __forceinline__ float load(const T *p, float /*inv_scale*/) { return __ldg(p); }
+    static __device__ __forceinline__ float load(const T *p, float /*inv_scale*/) { return lbi::ld_f32(p); }
     static __device__ __forceinline__ float cvt(T v, float /*inv_scale*/) { return v; }
     static __device__ __forceinline__ T pack(float x, float /*scale*/) { return x; }
 };
@@ -360,7 +362,7 @@ struct Store<1> {
     using T = __half;
     static __device__ __forceinline__ float load(const T *p, float inv_scale)
     {
-        return __half2float(__ldg(p)) * inv_scale;
+        return __half2float(__ushort_as_half(lbi::ld_u16(p))) * inv_scale;
     }
     static __device__ __forceinline__ float cvt(T v, float inv_scale) { return __half2float(v) * inv_scale; }
     static __device__ __forceinline__ T pack(float x, float scale) { return __float2half_rn(x * scale); }
@@ -371,7 +373,7 @@ struct Store<2> {
     using T = __nv_bfloat16;
     static __device__ __forceinline__ float load(const T *p, float inv_scale)
     {
-        return __bfloat162float(__ldg(p)) * inv_scale;
+        return __bfloat162float(__ushort_as_bfloat16(lbi::ld_u16(p))) * inv_scale;
     }
     static __device__ __forceinline__ float cvt(T v, float inv_scale)
     {

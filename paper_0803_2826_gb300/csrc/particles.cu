@@ -530,6 +530,7 @@ __global__ void __launch_bounds__(kPartThreads) k_build_nlist(const float4 *shad
                                                               const unsigned int *flags, unsigned int *err,
                                                               CoupleArgs c, uint32_t rd)
 {
+    wait_for_previous();
     if (flags[rd] == 0u) return;
     constexpr int kGroups = kPartThreads / kChunks;
     __shared__ int lst[kMaxNb][kGroups];  // column per particle: conflict-free
@@ -872,6 +873,7 @@ template <int SPAN>
 __global__ void k_clear_records_by_particle(float *facc, const int *records, int n, int nsub, StepArgs g)
 {
     const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    wait_for_previous();
     if (t >= (size_t)n * 8) return;
     const int p = (int)(t >> 3), q = (int)(t & 7);
     constexpr int lo = SPAN == 4 ? -1 : 0, nk = SPAN * SPAN * SPAN;
@@ -1100,6 +1102,7 @@ struct PersistArgs {
 __global__ void k_shadow_from_pos(const double *pos, float4 *shadow, int *head, int *next, int *bucket_of,
                                   const unsigned int *flag, unsigned int *err, CoupleArgs c)
 {
+    wait_for_previous();
     if (*flag == 0u) return;
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= c.n) return;
@@ -1907,6 +1910,7 @@ __global__ void __launch_bounds__(kPartThreads) k_couple_free(FreeArgs a)
     const StepArgs &g = c.g;
     const int tid = blockIdx.x * blockDim.x + threadIdx.x;
     const int p = tid / LANES, q = tid % LANES;
+    wait_for_previous();
     if (p >= c.n) return;  // whole groups leave together (LANES divides the block)
     const unsigned gmask = LANES == 1 ? 0xFFFFFFFFu : (0xFFu << (threadIdx.x & 24));
     const T *src = static_cast<const T *>(a.src);
@@ -2095,6 +2099,22 @@ void note_records(Particles *P, int n, size_t count)
     P->n_records += count;
 }
 
+// The list build a persistent launch may need before it (both kernels return
+// at once when the previous call did not ask for it); eight lanes a particle.
+cudaError_t build_list_before(lb_handle *h, const lb_particles *pp, const CoupleArgs &c)
+{
+    Particles *P = h->parts;
+    const unsigned int blocks = (unsigned int)((c.n + kPartThreads - 1) / kPartThreads);
+    const unsigned int gblocks = (unsigned int)(((size_t)c.n * kChunks + kPartThreads - 1) / kPartThreads);
+    cudaError_t e = launch_chained(k_shadow_from_pos, blocks, kPartThreads, h->stream, pp->pos, P->shadow[1], P->head,
+                                   P->next, P->bucket_of, P->flags + 2, h->d_err, c);
+    if (e == cudaSuccess)
+        e = launch_chained(k_build_nlist, gblocks, kPartThreads, h->stream, P->shadow[1], P->head, P->next, P->nlist,
+                           P->ncount, P->ref, P->flags, h->d_err, c, 2u);
+    h->launches += 2;
+    return e;
+}
+
 template <int DT>
 cudaError_t run_substeps(lb_handle *h, const lb_particles *pp, const lb_couple_params *cp)
 {
@@ -2137,9 +2157,11 @@ cudaError_t run_substeps(lb_handle *h, const lb_particles *pp, const lb_couple_p
         fa.err = h->d_err;
         const int lanes = c.kw == 2 ? free_lanes<2>() : free_lanes<3>();
         const unsigned int fblocks = (unsigned int)(((size_t)n * lanes + kPartThreads - 1) / kPartThreads);
-        if (c.kw == 3) k_couple_free<DT, 3><<<fblocks, kPartThreads, 0, h->stream>>>(fa);
-        else if (c.kw == 4) k_couple_free<DT, 4><<<fblocks, kPartThreads, 0, h->stream>>>(fa);
-        else k_couple_free<DT, 2><<<fblocks, kPartThreads, 0, h->stream>>>(fa);
+        const cudaError_t le = launch_chained(c.kw == 3   ? k_couple_free<DT, 3>
+                                              : c.kw == 4 ? k_couple_free<DT, 4>
+                                                          : k_couple_free<DT, 2>,
+                                              fblocks, kPartThreads, h->stream, fa);
+        if (le != cudaSuccess) return le;
         h->launches += 1;
         note_records(P, n, (size_t)n * (size_t)cp->n_substeps);
         P->rec_span = std::max(P->rec_span, c.kw == 3 ? 3 : (c.kw == 4 ? 4 : 2));
@@ -2149,7 +2171,6 @@ cudaError_t run_substeps(lb_handle *h, const lb_particles *pp, const lb_couple_p
     }
 
     // persistent path when every particle group can be resident at once
-    const int gblocks = (int)(((size_t)n * kChunks + kPartThreads - 1) / kPartThreads);  // 8 lanes a particle
     const int pblocks = (n + kPThreads - 1) / kPThreads;                                   // one thread a particle
     int per_sm = 0;
     if (!(cp->flags & LB_COUPLE_PER_SUBSTEP) && c.kw > 2) {
@@ -2177,11 +2198,8 @@ cudaError_t run_substeps(lb_handle *h, const lb_particles *pp, const lb_couple_p
                 h->facc_stale = 0;
             }
             if (need_nlist) {
-                k_shadow_from_pos<<<blocks, kPartThreads, 0, h->stream>>>(pp->pos, P->shadow[1], P->head, P->next,
-                                                                           P->bucket_of, P->flags + 2, h->d_err, c);
-                k_build_nlist<<<gblocks, kPartThreads, 0, h->stream>>>(P->shadow[1], P->head, P->next, P->nlist,
-                                                                       P->ncount, P->ref, P->flags, h->d_err, c, 2u);
-                h->launches += 2;
+                e = build_list_before(h, pp, c);
+                if (e != cudaSuccess) return e;
             }
             PersistArgs a;
             a.c = c;
@@ -2249,11 +2267,8 @@ cudaError_t run_substeps(lb_handle *h, const lb_particles *pp, const lb_couple_p
             h->facc_stale = 0;
         }
         if (need_nlist) {
-            k_shadow_from_pos<<<blocks, kPartThreads, 0, h->stream>>>(pp->pos, P->shadow[1], P->head, P->next,
-                                                                       P->bucket_of, P->flags + 2, h->d_err, c);
-            k_build_nlist<<<gblocks, kPartThreads, 0, h->stream>>>(P->shadow[1], P->head, P->next, P->nlist,
-                                                                   P->ncount, P->ref, P->flags, h->d_err, c, 2u);
-            h->launches += 2;
+            e = build_list_before(h, pp, c);
+            if (e != cudaSuccess) return e;
         }
         PersistArgs a;
         a.c = c;
@@ -2642,12 +2657,11 @@ cudaError_t clear_particle_forces(lb_handle *h)
         if (P->rec_n > 0 && P->n_records % (size_t)P->rec_n == 0) {  // [nsub][n]: skip repeated cells
             const int nsub = (int)(P->n_records / (size_t)P->rec_n);
             const unsigned int blocks = (unsigned int)(((size_t)P->rec_n * 8 + 255) / 256);
-            if (P->rec_span == 4)
-                k_clear_records_by_particle<4><<<blocks, 256, 0, h->stream>>>(h->facc, rec, P->rec_n, nsub, g);
-            else if (P->rec_span == 3)
-                k_clear_records_by_particle<3><<<blocks, 256, 0, h->stream>>>(h->facc, rec, P->rec_n, nsub, g);
-            else
-                k_clear_records_by_particle<2><<<blocks, 256, 0, h->stream>>>(h->facc, rec, P->rec_n, nsub, g);
+            const cudaError_t e = launch_chained(P->rec_span == 4   ? k_clear_records_by_particle<4>
+                                                 : P->rec_span == 3 ? k_clear_records_by_particle<3>
+                                                                    : k_clear_records_by_particle<2>,
+                                                 blocks, 256, h->stream, h->facc, rec, P->rec_n, nsub, g);
+            if (e != cudaSuccess) return e;
         } else {
             int blocks = (int)std::min<size_t>((P->n_records + 255) / 256, (size_t)8 * device_sm_count());
             if (P->rec_span == 4)

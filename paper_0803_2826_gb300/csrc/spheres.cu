@@ -137,6 +137,7 @@ __global__ void k_sph_half(const double *pos, const double *vel, const double *m
                            float *acc, unsigned int *count, StepArgs g, unsigned int *err)
 {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    wait_for_previous();
     if (p == 0) *count = 0u;  // the near-node list of this step
     if (p >= n) return;
     const double m = mass ? mass[p] : mass0;
@@ -165,6 +166,7 @@ __global__ void k_sph_map(int *owner, float *pops, const double *rh, const doubl
     __shared__ Box b;
     const int p = blockIdx.y;
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    wait_for_previous();
     const double c[3] = {rh[3 * p], rh[3 * p + 1], rh[3 * p + 2]};
     box_setup(b, c, a);
     if (p >= n || k >= B * B * B) return;
@@ -235,6 +237,7 @@ __global__ void __launch_bounds__(kSphThreads) k_sph_links(int *owner, const flo
     float v[NV];
 #pragma unroll
     for (int q = 0; q < NV; ++q) v[q] = 0.0f;
+    wait_for_previous();
     const double c[3] = {rh[3 * p], rh[3 * p + 1], rh[3 * p + 2]};
     box_setup(b, c, a);
     bool add = false;  // a near node for the list of the re-update
@@ -433,6 +436,7 @@ __global__ void k_sph_update(double *vel, double *om, const double *mass, double
                              int n, const float *acc, float4 *ut, float4 *uw)
 {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    wait_for_previous();
     if (p >= n) return;
     const double m = mass ? mass[p] : mass0;
     const float *ac = acc + kAcc * p;
@@ -490,6 +494,7 @@ __global__ void k_sph_finish(double *pos, const double *vel, const double *mass,
                              int n, StepArgs g)
 {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    wait_for_previous();
     if (p >= n) return;
     const double m = mass ? mass[p] : mass0;
     if (!(m > 0.0)) return;
@@ -511,10 +516,10 @@ __device__ __forceinline__ float image_f(float d, int L)
 // (Eqs. MBB, NodeVel; c_b = -c_i); far fluid nodes pull without looking at
 // the map.  rot: the spheres rotate (uw, rh are read).
 template <bool NOISE>
-__device__ __forceinline__ void sphere_node(const float *__restrict__ src, float *__restrict__ dst,
-                                            const float *__restrict__ ffield, const int *__restrict__ owner,
-                                            const float4 *__restrict__ ut, const float4 *__restrict__ uw,
-                                            const double *__restrict__ rh, bool rot, const StepArgs &a, int x, int y,
+__device__ __forceinline__ void sphere_node(const float *src, float *dst,
+                                            const float *ffield, const int *owner,
+                                            const float4 *ut, const float4 *uw,
+                                            const double *rh, bool rot, const StepArgs &a, int x, int y,
                                             int z, int own)
 {
     const size_t self = ((size_t)z * a.ny + y) * a.nx + x;
@@ -529,7 +534,7 @@ __device__ __forceinline__ void sphere_node(const float *__restrict__ src, float
             const int sx = lbd::cx(i) == 1 ? xm : (lbd::cx(i) == -1 ? xp : x);
             const int sy = lbd::cy(i) == 1 ? ym : (lbd::cy(i) == -1 ? yp : y);
             const int sz = lbd::cz(i) == 1 ? zm : (lbd::cz(i) == -1 ? zp : z);
-            n[i] = __ldg(src + (size_t)i * P + ((size_t)sz * a.ny + sy) * a.nx + sx);
+            n[i] = ld_f32(src + (size_t)i * P + ((size_t)sz * a.ny + sy) * a.nx + sx);
         }
     } else {
 #pragma unroll
@@ -538,12 +543,12 @@ __device__ __forceinline__ void sphere_node(const float *__restrict__ src, float
             const int sy = lbd::cy(i) == 1 ? ym : (lbd::cy(i) == -1 ? yp : y);
             const int sz = lbd::cz(i) == 1 ? zm : (lbd::cz(i) == -1 ? zp : z);
             const size_t t = ((size_t)sz * a.ny + sy) * a.nx + sx;
-            const int o = i == 0 ? kFar : __ldg(owner + t);
+            const int o = i == 0 ? kFar : owner[t];
             if (o >= 0) {
-                const float4 v = __ldg(ut + o);
+                const float4 v = ut[o];
                 float ub[3] = {v.x, v.y, v.z};
                 if (rot) {
-                    const float4 w = __ldg(uw + o);
+                    const float4 w = uw[o];
                     const float rb[3] = {image_f((float)((double)x - 0.5 * lbd::cx(i) - rh[3 * o]), a.nx),
                                          image_f((float)((double)y - 0.5 * lbd::cy(i) - rh[3 * o + 1]), a.ny),
                                          image_f((float)((double)z - 0.5 * lbd::cz(i) - rh[3 * o + 2]), a.nz)};
@@ -553,17 +558,17 @@ __device__ __forceinline__ void sphere_node(const float *__restrict__ src, float
                     for (int d = 0; d < 3; ++d) ub[d] += wr[d];
                 }
                 const float uc = lbd::cx(i) * ub[0] + lbd::cy(i) * ub[1] + lbd::cz(i) * ub[2];
-                n[i] = __ldg(src + (size_t)lbd::opposite(i) * P + self) + 6.0f * lbd::weight(i) * a.rho0 * uc;
+                n[i] = ld_f32(src + (size_t)lbd::opposite(i) * P + self) + 6.0f * lbd::weight(i) * a.rho0 * uc;
             } else {
-                n[i] = __ldg(src + (size_t)i * P + t);
+                n[i] = ld_f32(src + (size_t)i * P + t);
             }
         }
     }
     float fx = a.fx, fy = a.fy, fz = a.fz;
     if (ffield) {
-        fx += __ldg(ffield + self);
-        fy += __ldg(ffield + a.nn + self);
-        fz += __ldg(ffield + 2 * a.nn + self);
+        fx += ld_f32(ffield + self);
+        fy += ld_f32(ffield + a.nn + self);
+        fz += ld_f32(ffield + 2 * a.nn + self);
     }
     float m[19], out[19];
     lbd::forward(n, m);
@@ -578,14 +583,15 @@ __device__ __forceinline__ void sphere_node(const float *__restrict__ src, float
 // ones are done again here with the moving bounce-back.  Grid-stride over
 // the list.
 template <bool NOISE>
-__global__ void __launch_bounds__(kSphThreads) k_sph_near_nodes(const float *__restrict__ src, float *__restrict__ dst,
-                                                                 const float *__restrict__ ffield,
-                                                                 const int *__restrict__ owner,
-                                                                 const float4 *__restrict__ ut,
-                                                                 const float4 *__restrict__ uw, const double *rh,
+__global__ void __launch_bounds__(kSphThreads) k_sph_near_nodes(const float *src, float *dst,
+                                                                 const float *ffield,
+                                                                 const int *owner,
+                                                                 const float4 *ut,
+                                                                 const float4 *uw, const double *rh,
                                                                  bool rot, const int *list,
                                                                  const unsigned int *count, StepArgs g)
 {
+    wait_for_previous();
     const unsigned int nl = *count;
     for (unsigned int q = blockIdx.x * blockDim.x + threadIdx.x; q < nl; q += gridDim.x * blockDim.x) {
         const int s = list[q];
@@ -754,20 +760,19 @@ lb_status lb_step_spheres(lb_handle *h, const lb_spheres *s)
         const int B = box_edge(s->radius);
         const unsigned pb = (unsigned)((n + kSphThreads - 1) / kSphThreads);
         const dim3 grid((unsigned)((B * B * B + kSphThreads - 1) / kSphThreads), (unsigned)n);
-        k_sph_half<<<pb, kSphThreads, 0, h->stream>>>(s->pos, s->vel, s->mass, s->mass0, n, h->sph_rh, h->sph_acc,
-                                                      h->sph_count, g, h->d_err);
-        k_sph_map<<<grid, kSphThreads, 0, h->stream>>>(h->sph_owner, src, h->sph_rh, s->vel, s->omega, s->radius, B, n,
-                                                       g, h->sph_acc, h->d_err);
-        if (s->omega)
-            k_sph_links<true><<<grid, kSphThreads, 0, h->stream>>>(h->sph_owner, src, h->sph_rh, s->radius, B, n, g,
-                                                                   h->sph_acc, h->sph_list, h->sph_count);
-        else
-            k_sph_links<false><<<grid, kSphThreads, 0, h->stream>>>(h->sph_owner, src, h->sph_rh, s->radius, B, n, g,
-                                                                    h->sph_acc, h->sph_list, h->sph_count);
-        k_sph_update<<<pb, kSphThreads, 0, h->stream>>>(s->vel, s->omega, s->mass, s->mass0, s->radius, s->force, n,
-                                                        h->sph_acc, h->sph_ut, h->sph_uw);
+        e = launch_chained(k_sph_half, pb, kSphThreads, h->stream, s->pos, s->vel, s->mass, s->mass0, n, h->sph_rh,
+                           h->sph_acc, h->sph_count, g, h->d_err);
+        if (e == cudaSuccess)
+            e = launch_chained(k_sph_map, grid, kSphThreads, h->stream, h->sph_owner, src, h->sph_rh, s->vel, s->omega,
+                               s->radius, B, n, g, h->sph_acc, h->d_err);
+        if (e == cudaSuccess)
+            e = launch_chained(s->omega ? k_sph_links<true> : k_sph_links<false>, grid, kSphThreads, h->stream,
+                               h->sph_owner, src, h->sph_rh, s->radius, B, n, g, h->sph_acc, h->sph_list,
+                               h->sph_count);
+        if (e == cudaSuccess)
+            e = launch_chained(k_sph_update, pb, kSphThreads, h->stream, s->vel, s->omega, s->mass, s->mass0, s->radius,
+                               s->force, n, h->sph_acc, h->sph_ut, h->sph_uw);
         h->launches += 4;
-        e = cudaGetLastError();
     }
     if (e == cudaSuccess) {  // every node with the plain update (solid nodes get values nobody reads)
         e = launch_stream_collide_dt<0>(h, src, dst, nullptr, nullptr);
@@ -776,22 +781,15 @@ lb_status lb_step_spheres(lb_handle *h, const lb_spheres *s)
     if (e == cudaSuccess && n > 0) {  // then the near fluid nodes with the moving bounce-back
         const unsigned grid = (unsigned)(4 * device_sm_count());
         const bool rot = s->omega != nullptr;
-        if (g.kT > 0.0f)
-            k_sph_near_nodes<true><<<grid, kSphThreads, 0, h->stream>>>(src, dst, h->force, h->sph_owner, h->sph_ut,
-                                                                        h->sph_uw, h->sph_rh, rot, h->sph_list,
-                                                                        h->sph_count, g);
-        else
-            k_sph_near_nodes<false><<<grid, kSphThreads, 0, h->stream>>>(src, dst, h->force, h->sph_owner, h->sph_ut,
-                                                                         h->sph_uw, h->sph_rh, rot, h->sph_list,
-                                                                         h->sph_count, g);
+        e = launch_chained(g.kT > 0.0f ? k_sph_near_nodes<true> : k_sph_near_nodes<false>, grid, kSphThreads, h->stream,
+                           src, dst, h->force, h->sph_owner, h->sph_ut, h->sph_uw, h->sph_rh, rot, h->sph_list,
+                           h->sph_count, g);
         h->launches += 1;
-        e = cudaGetLastError();
     }
     if (e == cudaSuccess && n > 0) {
-        k_sph_finish<<<(unsigned)((n + kSphThreads - 1) / kSphThreads), kSphThreads, 0, h->stream>>>(
-            s->pos, s->vel, s->mass, s->mass0, h->sph_rh, n, g);
+        e = launch_chained(k_sph_finish, (unsigned)((n + kSphThreads - 1) / kSphThreads), kSphThreads, h->stream, s->pos,
+                           s->vel, s->mass, s->mass0, h->sph_rh, n, g);
         h->launches += 1;
-        e = cudaGetLastError();
     }
     if (e != cudaSuccess) return cuda_fail("lb_step_spheres", e);
     h->cur = 1 - h->cur;

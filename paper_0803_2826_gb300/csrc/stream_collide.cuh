@@ -220,14 +220,14 @@ __device__ __forceinline__ void update_node(const typename lbd::Store<DT>::T *__
     float fx = a.fx, fy = a.fy, fz = a.fz;
     if (FIELD) {
         if (ffield) {  // caller's field, component stride N
-            fx += __ldg(ffield + self);
-            fy += __ldg(ffield + a.nn + self);
-            fz += __ldg(ffield + 2 * a.nn + self);
+            fx += ld_f32(ffield + self);
+            fy += ld_f32(ffield + a.nn + self);
+            fz += ld_f32(ffield + 2 * a.nn + self);
         }
         if (facc) {  // library accumulator, component stride = plane pitch
-            fx += __ldg(facc + self);
-            fy += __ldg(facc + P + self);
-            fz += __ldg(facc + 2 * P + self);
+            fx += ld_f32(facc + self);
+            fy += ld_f32(facc + P + self);
+            fz += ld_f32(facc + 2 * P + self);
         }
     }
     float m[19], out[19];
@@ -281,12 +281,12 @@ __device__ __forceinline__ bool patch_node(int bx, int by, int bz, int k, int sp
 template <int DT, bool NOISE, bool WALLS>
 __global__ void __launch_bounds__(kBX) k_patch_impulse_nodes(const typename lbd::Store<DT>::T *__restrict__ src,
                                                              typename lbd::Store<DT>::T *__restrict__ dst,
-                                                             const float *__restrict__ ffield,
-                                                             float *__restrict__ facc, const int *records,
+                                                             const float *ffield, float *facc, const int *records,
                                                              int n, int nsub, int span, unsigned int *claim,
                                                              unsigned int tag, const StepArgs a)
 {
     const int t = blockIdx.x * kBX + threadIdx.x;
+    wait_for_previous();
     if (t >= n * 8) return;
     const int p = t >> 3, q = t & 7;
     const int nk = span * span * span;
@@ -321,12 +321,13 @@ __global__ void __launch_bounds__(kBX) k_patch_impulse_nodes(const typename lbd:
 // claim makes sure each node is corrected once.  Eight blocks per SM (64 registers, no
 // spills): the launch for the workload's ~1.3e5 threads fits in one wave.
 template <bool WALLS>
-__global__ void __launch_bounds__(kBX, 8) k_patch_impulse_nodes_f32(float *__restrict__ dst, const float *__restrict__ ffield,
-                                                                 float *__restrict__ facc, const int *records, int n,
+__global__ void __launch_bounds__(kBX, 8) k_patch_impulse_nodes_f32(float *dst, const float *ffield, float *facc,
+                                                                 const int *records, int n,
                                                                  int nsub, int span, unsigned int *claim,
                                                                  unsigned int tag, const StepArgs a)
 {
     const int t = blockIdx.x * kBX + threadIdx.x;
+    wait_for_previous();
     if (t >= n * 8) return;
     const int p = t >> 3, q = t & 7;
     const size_t P = a.pitch;
@@ -410,7 +411,7 @@ template <>
 struct Pair<0> {
     static __device__ __forceinline__ void load(const float *p, float inv, float &a, float &b)
     {
-        const float2 v = __ldg(reinterpret_cast<const float2 *>(p));
+        const float2 v = ld_f32x2(p);
         a = v.x;
         b = v.y;
     }
@@ -423,7 +424,8 @@ template <>
 struct Pair<1> {
     static __device__ __forceinline__ void load(const __half *p, float inv, float &a, float &b)
     {
-        const __half2 v = __ldg(reinterpret_cast<const __half2 *>(p));
+        const unsigned int w = ld_u32(p);
+        const __half2 v = *reinterpret_cast<const __half2 *>(&w);
         a = __low2float(v) * inv;
         b = __high2float(v) * inv;
     }
@@ -436,7 +438,8 @@ template <>
 struct Pair<2> {
     static __device__ __forceinline__ void load(const __nv_bfloat16 *p, float inv, float &a, float &b)
     {
-        const __nv_bfloat162 v = __ldg(reinterpret_cast<const __nv_bfloat162 *>(p));
+        const unsigned int w = ld_u32(p);
+        const __nv_bfloat162 v = *reinterpret_cast<const __nv_bfloat162 *>(&w);
         a = __low2float(v) * inv;
         b = __high2float(v) * inv;
     }
@@ -512,8 +515,8 @@ __device__ __forceinline__ void load_pair(const typename lbd::Store<DT>::T *__re
         if (ffield) {  // caller's field, component stride N
 #pragma unroll
             for (int d = 0; d < 3; ++d) {
-                f0[d] += __ldg(ffield + d * a.nn + self);
-                f1[d] += __ldg(ffield + d * a.nn + self + 1);
+                f0[d] += ld_f32(ffield + d * a.nn + self);
+                f1[d] += ld_f32(ffield + d * a.nn + self + 1);
             }
         }
         if (facc) {  // library accumulator, component stride = plane pitch
@@ -586,6 +589,7 @@ __global__ void __launch_bounds__(kBX) k_stream_collide2(const typename lbd::Sto
                                                          float *partials)
 {
     const int x0 = 2 * (blockIdx.x * kBX + threadIdx.x);
+    wait_for_previous();
     if (SUMS) {
         __shared__ float part[kBX / 32][38];
         const bool valid = x0 < a.nx;  // lanes past the row load nodes 0, 1 of it and store nothing
@@ -707,12 +711,12 @@ __device__ __forceinline__ void load_pair_any(const typename lbd::Store<DT>::T *
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
             if (ffield) {  // caller's field, component stride N
-                f0[d] += __ldg(ffield + d * a.nn + pa.self);
-                f1[d] += __ldg(ffield + d * a.nn + pb.self);
+                f0[d] += ld_f32(ffield + d * a.nn + pa.self);
+                f1[d] += ld_f32(ffield + d * a.nn + pb.self);
             }
             if (facc) {  // library accumulator, component stride = plane pitch
-                f0[d] += __ldg(facc + d * a.pitch + pa.self);
-                f1[d] += __ldg(facc + d * a.pitch + pb.self);
+                f0[d] += ld_f32(facc + d * a.pitch + pa.self);
+                f1[d] += ld_f32(facc + d * a.pitch + pb.self);
             }
         }
     }
@@ -762,7 +766,9 @@ __global__ void __launch_bounds__(kLinBX) k_stream_collide_linear(const typename
                                                                const float *__restrict__ facc, const StepArgs a)
 {
     PairAt at;
-    if (!locate_pair<WALLS>(a, at)) return;
+    const bool mine = locate_pair<WALLS>(a, at);
+    wait_for_previous();
+    if (!mine) return;
     lbp::F2 n[19], m[19], out[19];
     float f0[3], f1[3];
     load_linear<DT, FIELD, WALLS, ODD>(src, ffield, facc, a, at, n, f0, f1);
@@ -797,6 +803,7 @@ __global__ void __launch_bounds__(kBX) k_stream_collide_sums_any(const typename 
     at.s = (uint32_t)((at.z * a.ny + at.y) * a.nx + at.x);
     at.va = true;
     at.vb = at.x + 1 < a.nx;
+    wait_for_previous();
     lbp::F2 n[19], m[19], out[19];
     float f0[3], f1[3];
     load_pair_any<DT, FIELD, WALLS>(src, ffield, facc, a, at, n, f0, f1);
@@ -851,40 +858,23 @@ cudaError_t launch_stream_collide_dt(const lb_handle *h, const void *src, void *
     const uint32_t first = walls ? (uint32_t)(a.nx * a.ny) : 0u;
     const dim3 linear((unsigned)(((a.nn - first - (first & ~1u) + 1) / 2 + kLinBX - 1) / kLinBX));
 #define LBI_SC(NZ, FL, WL)                                                                                        \
-    do {                                                                                                          \
-        if (partials) {                                                                                           \
-            if (paired)                                                                                           \
-                k_stream_collide2<DT, NZ, FL, WL, true><<<grid, block, 0, h->stream>>>(s, d, h->force, facc, a,   \
-                                                                                        partials);               \
-            else                                                                                                  \
-                k_stream_collide_sums_any<DT, NZ, FL, WL><<<grid, block, 0, h->stream>>>(s, d, h->force, facc, a, \
-                                                                                         partials);              \
-        } else if (rows) {                                                                                        \
-            k_stream_collide2<DT, NZ, FL, WL, false><<<grid, block, 0, h->stream>>>(s, d, h->force, facc, a,      \
-                                                                                     nullptr);                   \
-        } else if (odd) {                                                                                         \
-            k_stream_collide_linear<DT, NZ, FL, WL, true><<<linear, kLinBX, 0, h->stream>>>(s, d, h->force, facc,  \
-                                                                                           a);                   \
-        } else {                                                                                                  \
-            k_stream_collide_linear<DT, NZ, FL, WL, false><<<linear, kLinBX, 0, h->stream>>>(s, d, h->force, facc, \
-                                                                                            a);                  \
-        }                                                                                                         \
-    } while (0)
+    (partials ? (paired ? launch_chained(k_stream_collide2<DT, NZ, FL, WL, true>, grid, block, h->stream, s, d,     \
+                                         h->force, facc, a, partials)                                             \
+                        : launch_chained(k_stream_collide_sums_any<DT, NZ, FL, WL>, grid, block, h->stream, s, d,   \
+                                         h->force, facc, a, partials))                                            \
+     : rows   ? launch_chained(k_stream_collide2<DT, NZ, FL, WL, false>, grid, block, h->stream, s, d, h->force,    \
+                               facc, a, nullptr)                                                                  \
+     : odd    ? launch_chained(k_stream_collide_linear<DT, NZ, FL, WL, true>, linear, dim3(kLinBX), h->stream, s, d, \
+                               h->force, facc, a)                                                                 \
+              : launch_chained(k_stream_collide_linear<DT, NZ, FL, WL, false>, linear, dim3(kLinBX), h->stream, s,  \
+                               d, h->force, facc, a))
     if (noise) {
-        if (field) {
-            if (walls) LBI_SC(true, true, true); else LBI_SC(true, true, false);
-        } else {
-            if (walls) LBI_SC(true, false, true); else LBI_SC(true, false, false);
-        }
-    } else {
-        if (field) {
-            if (walls) LBI_SC(false, true, true); else LBI_SC(false, true, false);
-        } else {
-            if (walls) LBI_SC(false, false, true); else LBI_SC(false, false, false);
-        }
+        if (field) return walls ? LBI_SC(true, true, true) : LBI_SC(true, true, false);
+        return walls ? LBI_SC(true, false, true) : LBI_SC(true, false, false);
     }
+    if (field) return walls ? LBI_SC(false, true, true) : LBI_SC(false, true, false);
+    return walls ? LBI_SC(false, false, true) : LBI_SC(false, false, false);
 #undef LBI_SC
-    return cudaGetLastError();
 }
 
 template <int DT>
@@ -900,24 +890,17 @@ cudaError_t launch_patch_dt(const lb_handle *h, const void *src, void *dst, floa
     const bool noise = a.kT > 0.0f, walls = h->p.walls != 0;
     if (DT == 0) {  // FP32: correct the stored result in place
         float *d32 = reinterpret_cast<float *>(dst);
-        if (walls)
-            k_patch_impulse_nodes_f32<true><<<blocks, kBX, 0, h->stream>>>(d32, h->force, facc, records, n, nsub, span,
-                                                                          claim, tag, a);
-        else
-            k_patch_impulse_nodes_f32<false><<<blocks, kBX, 0, h->stream>>>(d32, h->force, facc, records, n, nsub,
-                                                                           span, claim, tag, a);
-        return cudaGetLastError();
+        return walls ? launch_chained(k_patch_impulse_nodes_f32<true>, blocks, kBX, h->stream, d32, h->force, facc,
+                                      records, n, nsub, span, claim, tag, a)
+                     : launch_chained(k_patch_impulse_nodes_f32<false>, blocks, kBX, h->stream, d32, h->force, facc,
+                                      records, n, nsub, span, claim, tag, a);
     }
-#define LBI_PATCH(NZ, WL) \
-    k_patch_impulse_nodes<DT, NZ, WL><<<blocks, kBX, 0, h->stream>>>(s, d, h->force, facc, records, n, nsub, span, claim, \
-                                                     tag, a)
-    if (noise) {
-        if (walls) LBI_PATCH(true, true); else LBI_PATCH(true, false);
-    } else {
-        if (walls) LBI_PATCH(false, true); else LBI_PATCH(false, false);
-    }
+#define LBI_PATCH(NZ, WL)                                                                                             \
+    launch_chained(k_patch_impulse_nodes<DT, NZ, WL>, blocks, kBX, h->stream, s, d, h->force, facc, records, n, nsub,   \
+                   span, claim, tag, a)
+    if (noise) return walls ? LBI_PATCH(true, true) : LBI_PATCH(true, false);
+    return walls ? LBI_PATCH(false, true) : LBI_PATCH(false, false);
 #undef LBI_PATCH
-    return cudaGetLastError();
 }
 
 }  // namespace lbi
