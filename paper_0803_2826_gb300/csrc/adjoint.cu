@@ -21,13 +21,13 @@
 #include <cmath>
 #include <vector>
 
-#include "d3q19.cuh"
-#include "lbf_internal.h"
+#include "stream_collide.cuh"
 
 namespace lbi {
 
-template <int DT>
-cudaError_t launch_stream_collide_dt(const lb_handle *h, const void *src, void *dst, const float *facc, float *partials);
+extern template cudaError_t launch_stream_collide_dt<0>(const lb_handle *, const void *, void *, const float *, float *);
+extern template cudaError_t launch_stream_collide_dt<1>(const lb_handle *, const void *, void *, const float *, float *);
+extern template cudaError_t launch_stream_collide_dt<2>(const lb_handle *, const void *, void *, const float *, float *);
 
 namespace {
 
@@ -69,122 +69,145 @@ __device__ __forceinline__ void pull_source(int i, int x, int y, int z, int xm, 
     }
 }
 
-template <int DT, bool WALLS>
-__global__ void __launch_bounds__(kAdjBX)
-    k_adjoint_step(const typename lbd::Store<DT>::T *__restrict__ state, const float *__restrict__ lam_in,
-                   float *__restrict__ lam_out, const float *__restrict__ ffield, const float *__restrict__ impulse,
-                   float *grad_f, const StepArgs a)
+// Store of the pushed pair dn to the entries the pair pulls from: nodes x0,
+// x0 + 1 of one row (even nx), the mirror of load_pair.
+template <bool WALLS>
+__device__ __forceinline__ void push_pair(float *lam_out, const StepArgs &a, const PairAt &at, const lbp::F2 dn[19])
 {
-    using S = lbd::Store<DT>;
-    const int x = blockIdx.x * kAdjBX + threadIdx.x;
-    if (x >= a.nx) return;
-    const int y = blockIdx.y;
-    const int z = blockIdx.z + a.z0;
-    int xm, xp, ym, yp, zm, zp;
-    neighbours<WALLS>(x, y, z, a, xm, xp, ym, yp, zm, zp);
+    const int xm = at.x == 0 ? a.nx - 1 : at.x - 1, xp = at.x + 2 == a.nx ? 0 : at.x + 2;
+    const PullAt p = pull_at<WALLS>(a, at.x, at.y, at.z);
     const size_t P = a.pitch;
-    const uint32_t self = (uint32_t)((z * a.ny + y) * a.nx + x);
-
-    // forward quantities at this node
-    float n[19];
-    int plane[19];
-    uint32_t src[19];
 #pragma unroll
     for (int i = 0; i < 19; ++i) {
-        pull_source<WALLS>(i, x, y, z, xm, xp, ym, yp, zm, zp, a, plane[i], src[i]);
-        n[i] = S::load(state + (size_t)plane[i] * P + src[i], a.inv_scale);
-    }
-    float m[19];
-    lbd::forward(n, m);
-    float f[3] = {a.fx, a.fy, a.fz};
-    if (ffield) {
-        f[0] += ffield[self];
-        f[1] += ffield[a.nn + self];
-        f[2] += ffield[2 * a.nn + self];
-    }
-    if (impulse) {  // particle impulses of the step ([3][pitch])
-        f[0] += impulse[self];
-        f[1] += impulse[P + self];
-        f[2] += impulse[2 * P + self];
-    }
-    const float rho = a.rho0 + m[0];
-    const float ir = 1.0f / rho;
-    const float u[3] = {(m[1] + 0.5f * f[0]) * ir, (m[2] + 0.5f * f[1]) * ir, (m[3] + 0.5f * f[2]) * ir};
-
-    // adjoint of the back transform
-    float al[19];
-#pragma unroll
-    for (int i = 0; i < 19; ++i) al[i] = lbd::weight(i) * __ldg(lam_in + (size_t)i * P + self);
-    float mus[19];
-    lbd::forward(al, mus);
-#pragma unroll
-    for (int k = 0; k < 19; ++k) mus[k] *= lbd::inv_w(k);
-
-    // adjoint of the relaxation, the equilibrium and the force moments
-    const float gs = a.g_shear, gv = a.g_bulk;
-    const float cs = 1.0f + gs, cv = 1.0f + gv;
-    const float ux = u[0], uy = u[1], uz = u[2];
-    const float u2 = ux * ux + uy * uy + uz * uz;
-    const float Pk[6] = {u2, 3.0f * ux * ux - u2, uy * uy - uz * uz, ux * uy, uy * uz, uz * ux};
-    const float gk[6] = {gv, gs, gs, gs, gs, gs};
-    // dP_k/du rows
-    const float dP[6][3] = {{2.0f * ux, 2.0f * uy, 2.0f * uz},
-                            {4.0f * ux, -2.0f * uy, -2.0f * uz},
-                            {0.0f, 2.0f * uy, -2.0f * uz},
-                            {uy, ux, 0.0f},
-                            {0.0f, uz, uy},
-                            {uz, 0.0f, ux}};
-    // dF_k/du rows (F4 = cv u.f, F5 = cs (3 ux fx - u.f), F6 = cs (uy fy - uz fz),
-    // F7 = cs/2 (ux fy + uy fx), F8 = cs/2 (uy fz + uz fy), F9 = cs/2 (uz fx + ux fz))
-    const float dFu[6][3] = {{cv * f[0], cv * f[1], cv * f[2]},
-                             {2.0f * cs * f[0], -cs * f[1], -cs * f[2]},
-                             {0.0f, cs * f[1], -cs * f[2]},
-                             {0.5f * cs * f[1], 0.5f * cs * f[0], 0.0f},
-                             {0.0f, 0.5f * cs * f[2], 0.5f * cs * f[1]},
-                             {0.5f * cs * f[2], 0.0f, 0.5f * cs * f[0]}};
-    // dF_k/df rows: the same expressions with u and f exchanged
-    const float dFf[6][3] = {{cv * ux, cv * uy, cv * uz},
-                             {2.0f * cs * ux, -cs * uy, -cs * uz},
-                             {0.0f, cs * uy, -cs * uz},
-                             {0.5f * cs * uy, 0.5f * cs * ux, 0.0f},
-                             {0.0f, 0.5f * cs * uz, 0.5f * cs * uy},
-                             {0.5f * cs * uz, 0.0f, 0.5f * cs * ux}};
-    float rbar = 0.0f, ubar[3] = {0.f, 0.f, 0.f}, fbar[3] = {mus[1], mus[2], mus[3]};
-#pragma unroll
-    for (int q = 0; q < 6; ++q) {
-        const float mk = mus[4 + q];
-        const float one_g = 1.0f - gk[q];
-        rbar += mk * one_g * Pk[q];
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            ubar[d] += mk * (one_g * rho * dP[q][d] + dFu[q][d]);
-            fbar[d] += mk * dFf[q][d];
+        float v0, v1;
+        lbp::split(dn[i], v0, v1);
+        const bool bounce = WALLS && ((lbd::cz(i) == 1 && p.lo) || (lbd::cz(i) == -1 && p.hi));
+        if (bounce || lbd::cx(i) == 0) {
+            const size_t k = bounce ? (size_t)lbd::opposite(i) * P + at.s
+                                    : (size_t)i * P + p.z[1 - lbd::cz(i)] + p.y[1 - lbd::cy(i)] + (uint32_t)at.x;
+            if (in_bounds(k + 1, 19 * P, a.err)) Pair<0>::store(lam_out + k, v0, v1, 1.0f);
+            continue;
         }
+        float *row = lam_out + ((size_t)i * P + p.z[1 - lbd::cz(i)] + p.y[1 - lbd::cy(i)]);
+        row[lbd::cx(i) == 1 ? xm : at.x + 1] = v0;
+        row[lbd::cx(i) == 1 ? at.x : xp] = v1;
     }
-    float mu[19];
-    mu[0] = mus[0] + rbar - (ubar[0] * ux + ubar[1] * uy + ubar[2] * uz) * ir;
+}
+
+// The reverse of one step for two consecutive nodes per thread, in packed
+// FP32 over the linear node index (the mapping and the addresses of
+// k_stream_collide_linear).  Of the state only rho and u enter, so only the
+// conserved moments of the pulled populations are formed.  With the quadratic
+// forms P_k = u^T Q_k u (Q_4 = 1, Q_5 = diag(2, -1, -1), Q_6 = diag(0, 1, -1),
+// Q_7..9 = 1/2 off the diagonal) and F_k = (1 + g_k) u^T Q_k f, the adjoint of
+// the equilibrium and the forcing is that of T = sum_5..9 mu*_k Q_k and mu*_4:
+// two matrix-vector products T u, T f instead of the rows of six Jacobians.
+// Bound by memory (264 bytes a node); at 64^3, where part of it stays in the
+// L2, about 12 us a step against 19 us with one node a thread in scalar arithmetic
+// (802 instructions a node, half the threads of a 64-node row's block idle).
+template <int DT, bool WALLS, bool ODD>
+__global__ void __launch_bounds__(kLinBX)
+    k_adjoint_step(const typename lbd::Store<DT>::T *state, const float *lam_in, float *lam_out, const float *ffield,
+                   const float *impulse, float *grad_f, const StepArgs a)
+{
+    using lbp::F2;
+    using lbp::f2s;
+    using lbp::fma2;
+    PairAt at;
+    const bool mine = locate_pair<WALLS>(a, at);
+    wait_for_previous();
+    if (!mine) return;
+    const size_t P = a.pitch;
+
+    // rho and u of the forward step; al_i = a_i lambda_i
+    F2 n[19], m[4], al[19];
+    float f0[3], f1[3];
+    load_linear<DT, true, WALLS, ODD>(state, ffield, impulse, a, at, n, f0, f1);
+#pragma unroll
+    for (int i = 0; i < 19; ++i) {  // s is even, and s + 1 lies in the plane's padding at most
+        const float *p = lam_in + (size_t)i * P + at.s;
+        const float2 v = ODD ? make_float2(ld_f32(p), ld_f32(p + 1)) : ld_f32x2(p);
+        al[i] = lbp::f2(v.x, v.y) * lbd::weight(i);
+    }
+    lbp::forward2_conserved(n, m);
+    const F2 rho = f2s(a.rho0) + m[0];
+    float rl, rh;
+    lbp::split(rho, rl, rh);
+    const F2 ir = lbp::f2(__frcp_rn(rl), __frcp_rn(rh));
+    F2 f[3], u[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-        mu[1 + d] = mus[1 + d] + ubar[d] * ir;
-        fbar[d] += 0.5f * ubar[d] * ir;
+        f[d] = lbp::f2(f0[d], f1[d]);
+        u[d] = fma2(f2s(0.5f), f[d], m[1 + d]) * ir;
     }
-    mu[4] = gv * mus[4];
-#pragma unroll
-    for (int k = 5; k < 10; ++k) mu[k] = gs * mus[k];
-#pragma unroll
-    for (int k = 10; k < 16; ++k) mu[k] = a.g_odd * mus[k];
-#pragma unroll
-    for (int k = 16; k < 19; ++k) mu[k] = a.g_even * mus[k];
 
-    // dL/dn_i = sum_k e_ki mu_k = backward(mu)_i / a_i, pushed to the pull sources
-    float dn[19];
-    lbd::backward(mu, dn);
+    // adjoint of the back transform
+    F2 mu[19];
+    lbp::forward2(al, mu);
 #pragma unroll
-    for (int i = 0; i < 19; ++i) lam_out[(size_t)plane[i] * P + src[i]] = dn[i] * (1.0f / lbd::weight(i));
+    for (int k = 1; k < 19; ++k) mu[k] = mu[k] * lbd::inv_w(k);
+
+    // adjoint of the relaxation, the equilibrium and the force moments
+    const F2 txx = mu[5] + mu[5], tyy = mu[6] - mu[5], tzz = f2s(0.0f) - mu[5] - mu[6];
+    const F2 txy = mu[7] * 0.5f, tyz = mu[8] * 0.5f, tzx = mu[9] * 0.5f;
+    const F2 Tu[3] = {fma2(txx, u[0], fma2(txy, u[1], tzx * u[2])), fma2(txy, u[0], fma2(tyy, u[1], tyz * u[2])),
+                      fma2(tzx, u[0], fma2(tyz, u[1], tzz * u[2]))};
+    const F2 Tf[3] = {fma2(txx, f[0], fma2(txy, f[1], tzx * f[2])), fma2(txy, f[0], fma2(tyy, f[1], tyz * f[2])),
+                      fma2(tzx, f[0], fma2(tyz, f[1], tzz * f[2]))};
+    const F2 a4 = mu[4] * (1.0f - a.g_bulk), b4 = mu[4] * (1.0f + a.g_bulk);
+    F2 rbar = f2s(0.0f), udot = f2s(0.0f), ubar[3], fbar[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        const F2 Au = fma2(a4, u[d], Tu[d] * (1.0f - a.g_shear));
+        const F2 Bu = fma2(b4, u[d], Tu[d] * (1.0f + a.g_shear));
+        const F2 Bf = fma2(b4, f[d], Tf[d] * (1.0f + a.g_shear));
+        rbar = fma2(u[d], Au, rbar);
+        ubar[d] = fma2(rho, Au + Au, Bf);
+        udot = fma2(ubar[d], u[d], udot);
+        fbar[d] = mu[1 + d] + Bu;
+    }
+    mu[0] = mu[0] + rbar - udot * ir;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        const F2 w = ubar[d] * ir;
+        mu[1 + d] = mu[1 + d] + w;
+        fbar[d] = fma2(w, 0.5f, fbar[d]);
+    }
+    mu[4] = mu[4] * a.g_bulk;
+#pragma unroll
+    for (int k = 5; k < 10; ++k) mu[k] = mu[k] * a.g_shear;
+#pragma unroll
+    for (int k = 10; k < 16; ++k) mu[k] = mu[k] * a.g_odd;
+#pragma unroll
+    for (int k = 16; k < 19; ++k) mu[k] = mu[k] * a.g_even;
+
+    // dL/dn_i = sum_k e_ki mu_k, pushed to the pull sources
+    F2 dn[19];
+    lbp::backward2<false>(mu, dn);
+    if (ODD) {
+        int xb, yb, zb;
+        second_node(a, at, xb, yb, zb);
+        const PullAt pa = pull_at<WALLS>(a, at.x, at.y, at.z), pb = pull_at<WALLS>(a, xb, yb, zb);
+#pragma unroll
+        for (int i = 0; i < 19; ++i) {
+            float v0, v1;
+            lbp::split(dn[i], v0, v1);
+            const size_t ka = pull_index<WALLS>(a, pa, i), kb = pull_index<WALLS>(a, pb, i);
+            if (at.va && in_bounds(ka, 19 * P, a.err)) lam_out[ka] = v0;
+            if (at.vb && in_bounds(kb, 19 * P, a.err)) lam_out[kb] = v1;
+        }
+    } else {
+        push_pair<WALLS>(lam_out, a, at, dn);
+    }
     if (grad_f) {
-        grad_f[self] += fbar[0];
-        grad_f[a.nn + self] += fbar[1];
-        grad_f[2 * a.nn + self] += fbar[2];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {  // component stride N: no 8-byte alignment in general
+            float v0, v1;
+            lbp::split(fbar[d], v0, v1);
+            float *g = grad_f + d * a.nn + at.s;
+            if (at.va) g[0] += v0;
+            if (at.vb) g[1] += v1;
+        }
     }
 }
 
@@ -255,13 +278,12 @@ cudaError_t launch_adjoint_dt(const lb_handle *h, const void *state, const float
 {
     using T = typename lbd::Store<DT>::T;
     const StepArgs a = make_args(h);
-    dim3 grid((a.nx + kAdjBX - 1) / kAdjBX, a.ny, a.z1 - a.z0);
     const T *s = static_cast<const T *>(state);
-    if (h->p.walls)
-        k_adjoint_step<DT, true><<<grid, kAdjBX, 0, h->stream>>>(s, lam_in, lam_out, h->force, impulse, grad_f, a);
-    else
-        k_adjoint_step<DT, false><<<grid, kAdjBX, 0, h->stream>>>(s, lam_in, lam_out, h->force, impulse, grad_f, a);
-    return cudaGetLastError();
+    const bool odd = !sc_paired(h) || !pair_aligned(state, 2 * sizeof(T)) || !pair_aligned(lam_in, 8) ||
+                     !pair_aligned(lam_out, 8) || !pair_aligned(impulse, 8);
+    return launch_chained(h->p.walls ? (odd ? k_adjoint_step<DT, true, true> : k_adjoint_step<DT, true, false>)
+                                     : (odd ? k_adjoint_step<DT, false, true> : k_adjoint_step<DT, false, false>),
+                          linear_grid(a), kLinBX, h->stream, s, lam_in, lam_out, h->force, impulse, grad_f, a);
 }
 
 // dL/du at the nodes (lam_u, [3][pitch], set by the coupling reverse pass)

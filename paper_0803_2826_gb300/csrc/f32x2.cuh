@@ -125,13 +125,31 @@ __device__ __forceinline__ void forward2(const F2 n[19], F2 m[19])
     m[15] = Qz - Pz;
 }
 
+// The conserved moments m_0 .. m_3 alone (mass and momentum).
+__device__ __forceinline__ void forward2_conserved(const F2 n[19], F2 m[4])
+{
+    const F2 sa = n[7] + n[10], sb = n[8] + n[9], sc = n[11] + n[14], sd = n[12] + n[13];
+    const F2 se = n[15] + n[18], sg = n[16] + n[17];
+    const F2 pa = n[7] - n[10], pb = n[8] - n[9], pc = n[11] - n[14], pd = n[12] - n[13];
+    const F2 pe = n[15] - n[18], pg = n[16] - n[17];
+    const F2 A = (n[1] + n[2]) + (n[3] + n[4]) + (n[5] + n[6]);
+    m[0] = n[0] + A + ((sa + sb) + (sc + sd) + (se + sg));
+    m[1] = (n[1] - n[2]) + ((pa + pb) + (pe + pg));
+    m[2] = (n[3] - n[4]) + ((pa - pb) + (pc + pd));
+    m[3] = (n[5] - n[6]) + ((pc - pd) + (pe - pg));
+}
+
 // Back transform n_i = a_i sum_k e_ki M_k (M_k = m_k / w_k) of both nodes:
-// lbd::backward in packed form.
+// lbd::backward in packed form.  WEIGHTED false leaves the a_i out, which is
+// the transpose of forward2 (the reverse mode's dL/dn_i = sum_k e_ki mu_k).
+template <bool WEIGHTED>
+__device__ __forceinline__ F2 weigh(float a, F2 v) { return WEIGHTED ? f2s(a) * v : v; }
+
+template <bool WEIGHTED = true>
 __device__ __forceinline__ void backward2(const F2 M[19], F2 n[19])
 {
-    const F2 A0 = f2s(lbd::kA0), A1 = f2s(lbd::kA1), A2 = f2s(lbd::kA2);
     const F2 M5x2 = M[5] + M[5], M16x2 = M[16] + M[16], M17x2 = M[17] + M[17];
-    n[0] = A0 * (M[0] - M[4] + M[16]);
+    n[0] = weigh<WEIGHTED>(lbd::kA0, M[0] - M[4] + M[16]);
     {
         const F2 base = M[0] - M16x2;
         const F2 Ex = base + M5x2 - M17x2;
@@ -141,12 +159,12 @@ __device__ __forceinline__ void backward2(const F2 M[19], F2 n[19])
         const F2 Ez = Eyz - M[6] + M[18];
         const F2 Oy = M[2] - (M[11] + M[11]);
         const F2 Oz = M[3] - (M[12] + M[12]);
-        n[1] = A1 * (Ex + Ox);
-        n[2] = A1 * (Ex - Ox);
-        n[3] = A1 * (Ey + Oy);
-        n[4] = A1 * (Ey - Oy);
-        n[5] = A1 * (Ez + Oz);
-        n[6] = A1 * (Ez - Oz);
+        n[1] = weigh<WEIGHTED>(lbd::kA1, Ex + Ox);
+        n[2] = weigh<WEIGHTED>(lbd::kA1, Ex - Ox);
+        n[3] = weigh<WEIGHTED>(lbd::kA1, Ey + Oy);
+        n[4] = weigh<WEIGHTED>(lbd::kA1, Ey - Oy);
+        n[5] = weigh<WEIGHTED>(lbd::kA1, Ez + Oz);
+        n[6] = weigh<WEIGHTED>(lbd::kA1, Ez - Oz);
     }
     {
         const F2 base = M[0] + M[4] + M[16];
@@ -155,28 +173,28 @@ __device__ __forceinline__ void backward2(const F2 M[19], F2 n[19])
         const F2 oxy1 = M[1] + M[10] + M[13];
         const F2 oxy2 = M[2] + M[11] - M[14];
         const F2 O7 = oxy1 + oxy2, O8 = oxy1 - oxy2;
-        n[7] = A2 * (E7 + O7);
-        n[10] = A2 * (E7 - O7);
-        n[8] = A2 * (E8 + O8);
-        n[9] = A2 * (E8 - O8);
+        n[7] = weigh<WEIGHTED>(lbd::kA2, E7 + O7);
+        n[10] = weigh<WEIGHTED>(lbd::kA2, E7 - O7);
+        n[8] = weigh<WEIGHTED>(lbd::kA2, E8 + O8);
+        n[9] = weigh<WEIGHTED>(lbd::kA2, E8 - O8);
         const F2 Eyz = base - M5x2 - M17x2;
         const F2 E11 = Eyz + M[8], E12 = Eyz - M[8];
         const F2 oyz2 = M[2] + M[11] + M[14];
         const F2 oyz3 = M[3] + M[12] - M[15];
         const F2 O11 = oyz2 + oyz3, O12 = oyz2 - oyz3;
-        n[11] = A2 * (E11 + O11);
-        n[14] = A2 * (E11 - O11);
-        n[12] = A2 * (E12 + O12);
-        n[13] = A2 * (E12 - O12);
+        n[11] = weigh<WEIGHTED>(lbd::kA2, E11 + O11);
+        n[14] = weigh<WEIGHTED>(lbd::kA2, E11 - O11);
+        n[12] = weigh<WEIGHTED>(lbd::kA2, E12 + O12);
+        n[13] = weigh<WEIGHTED>(lbd::kA2, E12 - O12);
         const F2 Exz = base + M[5] - M[6] + M[17] - M[18];
         const F2 E15 = Exz + M[9], E16 = Exz - M[9];
         const F2 oxz1 = M[1] + M[10] - M[13];
         const F2 oxz3 = M[3] + M[12] + M[15];
         const F2 O15 = oxz1 + oxz3, O16 = oxz1 - oxz3;
-        n[15] = A2 * (E15 + O15);
-        n[18] = A2 * (E15 - O15);
-        n[16] = A2 * (E16 + O16);
-        n[17] = A2 * (E16 - O16);
+        n[15] = weigh<WEIGHTED>(lbd::kA2, E15 + O15);
+        n[18] = weigh<WEIGHTED>(lbd::kA2, E15 - O15);
+        n[16] = weigh<WEIGHTED>(lbd::kA2, E16 + O16);
+        n[17] = weigh<WEIGHTED>(lbd::kA2, E16 - O16);
     }
 }
 

@@ -616,6 +616,14 @@ struct PairAt {
     bool va, vb;
 };
 
+// Blocks of kLinBX threads that cover the fluid nodes (locate_pair).
+inline dim3 linear_grid(const StepArgs &a)
+{
+    const size_t first = a.z0 > 0 ? (size_t)a.nx * a.ny : 0;
+    const size_t pairs = (a.nn - first - (first & ~(size_t)1) + 1) / 2;
+    return dim3((unsigned)((pairs + kLinBX - 1) / kLinBX));
+}
+
 template <bool WALLS>
 __device__ __forceinline__ bool locate_pair(const StepArgs &a, PairAt &p)
 {
@@ -669,15 +677,36 @@ __device__ __forceinline__ PullAt pull_at(const StepArgs &a, int x, int y, int z
     return p;
 }
 
+// Index of the stored entry that population i of the node is pulled from.
+template <bool WALLS>
+__device__ __forceinline__ size_t pull_index(const StepArgs &a, const PullAt &p, int i)
+{
+    const uint32_t off = p.z[1 - lbd::cz(i)] + p.y[1 - lbd::cy(i)] + (uint32_t)p.x[1 - lbd::cx(i)];
+    const bool bounce = WALLS && ((lbd::cz(i) == 1 && p.lo) || (lbd::cz(i) == -1 && p.hi));
+    return WALLS && bounce ? (size_t)lbd::opposite(i) * a.pitch + p.self : (size_t)i * a.pitch + off;
+}
+
 // Population i as pulled by the node (stored value, FP16 / BF16 still scaled).
 template <int DT, bool WALLS>
 __device__ __forceinline__ float pull_one(const typename lbd::Store<DT>::T *__restrict__ src, const StepArgs &a,
                                           const PullAt &p, int i)
 {
-    const uint32_t off = p.z[1 - lbd::cz(i)] + p.y[1 - lbd::cy(i)] + (uint32_t)p.x[1 - lbd::cx(i)];
-    const bool bounce = WALLS && ((lbd::cz(i) == 1 && p.lo) || (lbd::cz(i) == -1 && p.hi));
-    const size_t k = WALLS && bounce ? (size_t)lbd::opposite(i) * a.pitch + p.self : (size_t)i * a.pitch + off;
+    const size_t k = pull_index<WALLS>(a, p, i);
     return in_bounds(k, 19 * a.pitch, a.err) ? lbd::Store<DT>::load(src + k, 1.0f) : 0.0f;
+}
+
+// Node s + 1 of a located pair; the located node itself where there is only one.
+__device__ __forceinline__ void second_node(const StepArgs &a, const PairAt &at, int &xb, int &yb, int &zb)
+{
+    xb = at.x;
+    yb = at.y;
+    zb = at.z;
+    if (!(at.va && at.vb)) return;
+    if (++xb < a.nx) return;
+    xb = 0;
+    if (++yb < a.ny) return;
+    yb = 0;
+    zb += 1;
 }
 
 template <int DT, bool FIELD, bool WALLS>
@@ -686,18 +715,8 @@ __device__ __forceinline__ void load_pair_any(const typename lbd::Store<DT>::T *
                                               const StepArgs &a, const PairAt &at, lbp::F2 n[19], float f0[3],
                                               float f1[3])
 {
-    int xb = at.x, yb = at.y, zb = at.z;  // node s + 1; the located node where there is only one
-    if (at.va && at.vb) {
-        xb += 1;
-        if (xb == a.nx) {
-            xb = 0;
-            yb += 1;
-            if (yb == a.ny) {
-                yb = 0;
-                zb += 1;
-            }
-        }
-    }
+    int xb, yb, zb;
+    second_node(a, at, xb, yb, zb);
     const PullAt pa = pull_at<WALLS>(a, at.x, at.y, at.z), pb = pull_at<WALLS>(a, xb, yb, zb);
 #pragma unroll
     for (int i = 0; i < 19; ++i) {
@@ -735,16 +754,18 @@ __device__ __forceinline__ void store_one(typename lbd::Store<DT>::T *__restrict
     }
 }
 
-// The pair's store; a lone node (va or vb false) is stored by itself.
+// The pair's store, node by node where only one is fluid (va or vb false) or
+// the buffer does not start on a pair.
 template <int DT>
 __device__ __forceinline__ void store_pair_any(typename lbd::Store<DT>::T *__restrict__ dst, const StepArgs &a,
                                                const PairAt &at, const lbp::F2 out[19])
 {
-    if (at.va && at.vb) {
+    if (at.va && at.vb && ((uintptr_t)dst & (2 * sizeof(*dst) - 1)) == 0) {
         store_pair<DT>(dst, a, at.s, out);
         return;
     }
-    store_one<DT>(dst, a, at.va ? at.s : at.s + 1u, out, !at.va);
+    if (at.va) store_one<DT>(dst, a, at.s, out, false);
+    if (at.vb) store_one<DT>(dst, a, at.s + 1u, out, true);
 }
 
 template <int DT, bool FIELD, bool WALLS, bool ODD>
@@ -831,6 +852,10 @@ inline bool sc_paired(const lb_handle *h)
     return (h->p.nx % 2 == 0) && (19.0 * (double)h->pitch < 4294967296.0);
 }
 
+// A caller's buffer may start at any element; pairs that move as one access
+// need an address that is a multiple of the pair.
+inline bool pair_aligned(const void *p, size_t bytes) { return ((uintptr_t)p & (bytes - 1)) == 0; }
+
 inline dim3 sc_grid(const lb_handle *h)
 {
     const int nzf = h->p.walls ? h->p.nz - 2 : h->p.nz;
@@ -850,13 +875,13 @@ cudaError_t launch_stream_collide_dt(const lb_handle *h, const void *src, void *
     const bool noise = a.kT > 0.0f;
     const bool field = (h->force != nullptr) || (facc != nullptr);
     const bool walls = h->p.walls != 0;
-    const bool paired = sc_paired(h);
+    const bool aligned = pair_aligned(src, 2 * sizeof(T)) && pair_aligned(dst, 2 * sizeof(T)) && pair_aligned(facc, 8);
+    const bool paired = sc_paired(h) && aligned;
     const T *s = static_cast<const T *>(src);
     T *d = static_cast<T *>(dst);
     const bool rows = !partials && paired && (h->p.nx / 2) % kBX == 0;
     const bool odd = !paired;
-    const uint32_t first = walls ? (uint32_t)(a.nx * a.ny) : 0u;
-    const dim3 linear((unsigned)(((a.nn - first - (first & ~1u) + 1) / 2 + kLinBX - 1) / kLinBX));
+    const dim3 linear = linear_grid(a);
 #define LBI_SC(NZ, FL, WL)                                                                                        \
     (partials ? (paired ? launch_chained(k_stream_collide2<DT, NZ, FL, WL, true>, grid, block, h->stream, s, d,     \
                                          h->force, facc, a, partials)                                             \
