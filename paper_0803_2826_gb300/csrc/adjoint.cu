@@ -585,17 +585,34 @@ lb_status lb_adjoint_forward(lb_handle *h, int nsteps, int checkpoint_every, con
         return LB_ENOMEM;
     }
     h->adj_ready = 0;
-    const size_t pop_bytes = 19 * h->pitch * h->elem;
     const uint32_t step0 = h->step;
+    // Each step writes its result where it is needed: a checkpoint at the end
+    // of a segment, the segment states themselves in the last segment (the
+    // reverse pass then has nothing to recompute there), the handle's buffers
+    // otherwise and at the end.
+    const int last0 = (nsteps - 1) / K * K;  // first step of the last segment
+    void *src = h->pops[h->cur];
+    e = cudaMemcpyAsync(b.ckpt[0], src, 19 * h->pitch * h->elem, cudaMemcpyDeviceToDevice, h->stream);
     for (int t = 0; t < nsteps && e == cudaSuccess; ++t) {
-        if (t % K == 0) e = cudaMemcpyAsync(b.ckpt[t / K], h->pops[h->cur], pop_bytes, cudaMemcpyDeviceToDevice, h->stream);
-        if (e == cudaSuccess && lb_step(h, 1) != LB_OK) e = cudaErrorLaunchFailure;
+        const int other = src == h->pops[0] ? 1 : 0;
+        void *dst = h->pops[other];
+        if (t + 1 < nsteps && (t + 1) % K == 0) dst = b.ckpt[(t + 1) / K];
+        else if (t + 1 < nsteps && t >= last0) dst = b.seg[t + 1 - last0];
+        timer_mark(h, 0, 0, h->stream);
+        e = step_from(h, src, dst, step0 + (uint32_t)t);
+        timer_mark(h, 0, 1, h->stream);
+        h->launches += 1;
+        src = dst;
     }
+    if (e != cudaSuccess) return cuda_fail("lb_adjoint_forward", e);
+    h->cur = src == h->pops[0] ? 0 : 1;
+    h->step = step0 + (uint32_t)nsteps;
     // the loss and its seed lambda_T = dL/dstate at the final state (first
-    // adjoint buffer) with its own dL/df (gseed), for lb_adjoint_backward
-    if (e == cudaSuccess) e = cudaMemsetAsync(loss, 0, sizeof(double), h->stream);
+    // adjoint buffer) with its own dL/df (gseed), for lb_adjoint_backward.
+    // The adjoint buffers are not cleared: every fluid entry is written before
+    // it is read, and the others only reach results that are not stored.
+    e = cudaMemsetAsync(loss, 0, sizeof(double), h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(b.gseed, 0, 3 * h->n_nodes * sizeof(float), h->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(b.lam[0], 0, 19 * h->pitch * sizeof(float), h->stream);
     if (e == cudaSuccess)
         e = launch_seed(h, h->pops[h->cur], b.lam[0], b.gseed, loss, make_int3(lo[0], lo[1], lo[2]),
                         make_int3(hi[0], hi[1], hi[2]));
@@ -626,8 +643,6 @@ lb_status lb_adjoint_backward(lb_handle *h, float *grad_force)
     KineticBuffers b;
     cudaError_t e = kinetic_buffers(h, nsteps, K, b);  // the forward's layout: no allocation
     if (e != cudaSuccess) return cuda_fail("lb_adjoint_backward", e);
-    const size_t lam_bytes = 19 * h->pitch * sizeof(float);
-    e = cudaMemsetAsync(b.lam[1], 0, lam_bytes, h->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(grad_force, b.gseed, 3 * h->n_nodes * sizeof(float), cudaMemcpyDeviceToDevice,
                             h->stream);
@@ -635,7 +650,7 @@ lb_status lb_adjoint_backward(lb_handle *h, float *grad_force)
     for (int s = nseg - 1; s >= 0 && e == cudaSuccess; --s) {
         const int t0 = s * K, t1 = std::min(nsteps, t0 + K);
         b.seg[0] = b.ckpt[s];
-        for (int t = t0; t < t1 - 1 && e == cudaSuccess; ++t) {
+        for (int t = t0; s < nseg - 1 && t < t1 - 1 && e == cudaSuccess; ++t) {
             e = step_from(h, b.seg[t - t0], b.seg[t - t0 + 1], h->adj_step0 + (uint32_t)t);
             h->launches += 1;
         }
