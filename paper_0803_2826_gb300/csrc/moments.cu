@@ -10,8 +10,7 @@
 //               block adds the partials in block order)
 #include <cstdio>
 
-#include "d3q19.cuh"
-#include "lbf_internal.h"
+#include "stream_collide.cuh"
 
 namespace lbi {
 
@@ -151,15 +150,12 @@ __global__ void __launch_bounds__(kRedThreads)
             pi_out[4 * N + s] = m[8];
             pi_out[5 * N + s] = m[9];
         }
-        if (partials) {
 #pragma unroll
-            for (int k = 0; k < 19; ++k) {
-                acc[k] += m[k];
-                acc[19 + k] = fmaf(m[k], m[k], acc[19 + k]);
-            }
+        for (int k = 0; k < 19; ++k) {
+            acc[k] += m[k];
+            acc[19 + k] = fmaf(m[k], m[k], acc[19 + k]);
         }
     }
-    if (!partials) return;
 
     // block reduction in a fixed order: warp shuffles, then warps in order
     __shared__ double red[kRedThreads / 32][38];
@@ -176,6 +172,92 @@ __global__ void __launch_bounds__(kRedThreads)
         double v = 0.0;
         for (int w = 0; w < kRedThreads / 32; ++w) v += red[w][threadIdx.x];
         partials[(size_t)blockIdx.x * 38 + threadIdx.x] = v;
+    }
+}
+
+// Component stores of a pair: one access where pair says the address allows.
+__device__ __forceinline__ void put_pair(float *out, size_t k, lbp::F2 v, bool pair, bool second)
+{
+    float v0, v1;
+    lbp::split(v, v0, v1);
+    if (pair) {
+        *reinterpret_cast<float2 *>(out + k) = make_float2(v0, v1);
+        return;
+    }
+    out[k] = v0;
+    if (second) out[k + 1] = v1;
+}
+
+// The fields alone (no sums): two consecutive nodes per thread over the
+// linear index of all nodes, the loads of k_stream_collide_linear, solid
+// nodes rho0 and zeros.  wide: component stride and outputs allow 8-byte
+// stores.  Bound by memory (76 bytes a node read, 40 written).  256^3:
+// 272 us, against 428 us with the 38 unused sums of k_moments in registers
+// (96 of them, a quarter of the warps) and one node a thread.
+template <int DT, bool WALLS, bool ODD>
+__global__ void __launch_bounds__(kLinBX)
+    k_fields(const typename lbd::Store<DT>::T *src, const float *ffield, float *rho_out, float *j_out, float *pi_out,
+             const StepArgs a, bool wide)
+{
+    using lbp::F2;
+    using lbp::f2s;
+    const uint32_t N = (uint32_t)a.nn;
+    PairAt at;
+    at.s = 2u * (blockIdx.x * (uint32_t)kLinBX + threadIdx.x);
+    wait_for_previous();
+    if (at.s >= N) return;
+    const bool second = at.s + 1u < N;
+    const uint32_t row = divide(at.s, a.dnx), z = divide(row, a.dny);
+    at.x = (int)(at.s - row * (uint32_t)a.nx);
+    at.y = (int)(row - z * (uint32_t)a.ny);
+    at.z = (int)z;
+    at.va = true;
+    at.vb = second;
+    bool solid0 = false, solid1 = false;
+    if (WALLS) {
+        int xb, yb, zb;
+        second_node(a, at, xb, yb, zb);
+        solid0 = at.z < a.z0 || at.z >= a.z1;
+        solid1 = zb < a.z0 || zb >= a.z1;
+        at.va = !solid0;
+        at.vb = second && !solid1;
+        if (solid0) {  // the pulls are those of the fluid node of the pair
+            at.x = xb;
+            at.y = yb;
+            at.z = zb;
+        }
+    }
+    F2 n[19], m[19];
+    float f0[3], f1[3];
+    if (!WALLS || at.va || at.vb) {
+        load_linear<DT, true, WALLS, ODD>(src, ffield, nullptr, a, at, n, f0, f1);
+    } else {
+#pragma unroll
+        for (int i = 0; i < 19; ++i) n[i] = f2s(0.0f);
+        f0[0] = f0[1] = f0[2] = f1[0] = f1[1] = f1[2] = 0.0f;
+    }
+    lbp::forward2(n, m);
+    const bool pair = wide && second;
+    // solid nodes: rho0, and zeros
+    const auto fluid = [&](F2 v) {
+        return WALLS ? lbp::f2(solid0 ? 0.0f : lbp::lo(v), solid1 ? 0.0f : lbp::hi(v)) : v;
+    };
+    const F2 rho = f2s(a.rho0) + fluid(m[0]);
+    if (rho_out) put_pair(rho_out, at.s, rho, pair, second);
+    if (j_out) {
+#pragma unroll
+        for (int d = 0; d < 3; ++d)
+            put_pair(j_out, d * a.nn + at.s, fluid(lbp::fma2(f2s(0.5f), lbp::f2(f0[d], f1[d]), m[1 + d])), pair, second);
+    }
+    if (pi_out) {
+        const F2 third = f2s(1.0f / 3.0f), sixth = f2s(1.0f / 6.0f);
+        const F2 b = (rho + rho) + (m[4] + m[4]) - m[5];
+        const F2 t6 = m[6] * 3.0f;
+        put_pair(pi_out, at.s, fluid((rho + m[4] + m[5]) * third), pair, second);
+        put_pair(pi_out, a.nn + at.s, fluid((b + t6) * sixth), pair, second);
+        put_pair(pi_out, 2 * a.nn + at.s, fluid((b - t6) * sixth), pair, second);
+#pragma unroll
+        for (int c = 3; c < 6; ++c) put_pair(pi_out, c * a.nn + at.s, fluid(m[4 + c]), pair, second);
     }
 }
 
@@ -237,13 +319,23 @@ cudaError_t launch_get_populations(const lb_handle *h, const void *src, double *
 cudaError_t launch_moments(const lb_handle *h, const void *src, float *rho, float *j, float *pi, double *sums)
 {
     const StepArgs a = make_args(h);
+    if (!sums) {
+        const bool wide = a.nn % 2 == 0 && pair_aligned(rho, 8) && pair_aligned(j, 8) && pair_aligned(pi, 8);
+        const dim3 grid((unsigned)(((a.nn + 1) / 2 + kLinBX - 1) / kLinBX));
+        const bool odd = !sc_paired(h), walls = h->p.walls != 0;
+        LBI_DT_SWITCH(h->p.dtype, return launch_chained(walls ? (odd ? k_fields<DT, true, true> : k_fields<DT, true, false>)
+                                                              : (odd ? k_fields<DT, false, true> : k_fields<DT, false, false>),
+                                                        grid, kLinBX, h->stream,
+                                                        static_cast<const typename lbd::Store<DT>::T *>(src), h->force,
+                                                        rho, j, pi, a, wide));
+    }
     const int g = grid_for(a.nn, h->red_blocks);
-    double *partials = sums ? h->d_partials : nullptr;
+    double *partials = h->d_partials;
     LBI_DT_SWITCH(h->p.dtype, (k_moments<DT><<<g, kRedThreads, 0, h->stream>>>(
                                   static_cast<const typename lbd::Store<DT>::T *>(src), h->force, rho, j,
                                   pi, partials, a)));
     cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess || !sums) return e;
+    if (e != cudaSuccess) return e;
     k_sum_partials<<<1, 64, 0, h->stream>>>(h->d_partials, g, sums, h->d_err);
     return cudaGetLastError();
 }
