@@ -866,16 +866,14 @@ __global__ void k_clear_records(float *facc, const int *records, size_t n, StepA
     }
 }
 
-// The same for live records laid out [nsub][n]: eight lanes per particle
-// walk its cells, skip a cell equal to the one before (a particle keeps its
-// cell for many sub-steps) and zero nodes q, q + 8, ... of the block.
-template <int SPAN>
-__global__ void k_clear_records_by_particle(float *facc, const int *records, int n, int nsub, StepArgs g)
+// Particle p's share of the same for live records laid out [nsub][n]: lane q
+// of LANES walks the particle's cells, skips a cell equal to the one before
+// (a particle keeps its cell for many sub-steps) and zeroes nodes q, q +
+// LANES, ... of the block.
+template <int SPAN, int LANES>
+__device__ __forceinline__ void clear_particle_records(float *facc, const int *records, int n, int nsub, int p, int q,
+                                                       const StepArgs &g)
 {
-    const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    wait_for_previous();
-    if (t >= (size_t)n * 8) return;
-    const int p = (int)(t >> 3), q = (int)(t & 7);
     constexpr int lo = SPAN == 4 ? -1 : 0, nk = SPAN * SPAN * SPAN;
     int prev = -1;
     for (int s = 0; s < nsub; ++s) {
@@ -884,7 +882,7 @@ __global__ void k_clear_records_by_particle(float *facc, const int *records, int
         prev = base;
         const int x0 = base % g.nx, y0 = (base / g.nx) % g.ny, z0 = base / (g.nx * g.ny);
 #pragma unroll
-        for (int k = q; k < nk; k += 8) {
+        for (int k = q; k < nk; k += LANES) {
             const int x = wrap_node(x0 + lo + k % SPAN, g.nx), y = wrap_node(y0 + lo + (k / SPAN) % SPAN, g.ny);
             int z = z0 + lo + k / (SPAN * SPAN);
             if (g.z0 > 0) z = z < 0 ? 0 : (z >= g.nz ? g.nz - 1 : z);
@@ -895,6 +893,15 @@ __global__ void k_clear_records_by_particle(float *facc, const int *records, int
             facc[2 * g.pitch + i] = 0.0f;
         }
     }
+}
+
+template <int SPAN>
+__global__ void k_clear_records_by_particle(float *facc, const int *records, int n, int nsub, StepArgs g)
+{
+    const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    wait_for_previous();
+    if (t >= (size_t)n * 8) return;
+    clear_particle_records<SPAN, 8>(facc, records, n, nsub, (int)(t >> 3), (int)(t & 7), g);
 }
 
 // Interpolated velocity at caller positions with phi_KW; eight lanes per
@@ -1872,6 +1879,278 @@ __global__ void __launch_bounds__(kPThreads) k_couple_persistent_wide(PersistArg
 }
 
 // ---------------------------------------------------------------------------
+// Persistent coupling of the wide stencils with LANES threads a particle, for
+// counts that can be resident that way.  The same sub-step loop,
+// list rebuilds and barriers, every lane of a group following the particle
+// (the same forces and interpolation in the same order, so a particle moves
+// as in the one-thread form, bit for bit); what is split is the work that
+// made that form long: lane q gathers the velocities of the stencil nodes q,
+// q + LANES, ... into the group's row of shared memory, and keeps and hands
+// in the impulse sums of those nodes.  A sub-step is a serial chain
+// (neighbour positions from L2, forces, update, barrier), so what counts is
+// its length: with one thread a particle it had 27 / 64 read-modify-writes in
+// shared memory and 64 x 19 loads after each move in it, on one block of 128
+// particles per SM.  The impulses of the previous call are cleared in the
+// first phase.  768 monomers in 72 x 64 x 60, phi_4, ten sub-steps and the
+// step: 96 us against 275 us.
+// ---------------------------------------------------------------------------
+template <int DT, int KW, int LANES>
+__global__ void __launch_bounds__(kPThreads) k_couple_lanes(PersistArgs a)
+{
+    using T = typename lbd::Store<DT>::T;
+    constexpr int kNodes = KW * KW * KW, kPer = (kNodes + LANES - 1) / LANES;
+    __shared__ unsigned int ticket;  // arrival word of the split barrier
+    // node velocities of the block's particles (a padded row each, so the
+    // groups of a warp read different banks)
+    __shared__ float4 su[kPThreads / LANES][kNodes + 1];
+    float4 *mine = su[threadIdx.x / LANES];
+    const CoupleArgs &c = a.c;
+    const StepArgs &g = c.g;
+    const int tid = blockIdx.x * blockDim.x + threadIdx.x;
+    const int p = tid / LANES, q = tid % LANES;
+    const bool active = p < c.n;  // whole groups
+    const bool lead = active && q == 0;
+    const T *src = static_cast<const T *>(a.src);
+    if (c.use_wca && tid == 0) a.flags[0] = 0u;  // the pre-launch build has run
+
+    // phase 0: clear the previous call's impulses, first half drift, neighbours
+    CPos me{}, refp{};
+    float pm[3] = {0.f, 0.f, 0.f};
+    float m = 1.f, G = 1.f, C1 = c.C1, C2 = c.C2, C3 = c.C3;
+    const int self = active ? p : 0;
+    int nnb = 0;
+    int nb[kNbReg];
+#pragma unroll
+    for (int k = 0; k < kNbReg; ++k) nb[k] = self;
+    bool bond_lo = false, bond_hi = false;
+    if (active) {
+        if (c.use_wca && lead) unbin_particle(p, a.head, a.bucket_of);
+        clear_particle_records<record_span<KW>(), LANES>(a.facc, a.stale, c.n, a.nstale_sub, p, q, g);
+        m = a.mass ? a.mass[p] : c.mass0;
+        G = a.gamma ? a.gamma[p] : c.gamma0;
+        if (!c.uniform_coef) {
+            const float x1 = G * c.dt / m;
+            C1 = expf(-x1);
+            C2 = (m / G) * (-expm1f(-x1));
+            C3 = sqrtf(m * g.kT * (-expm1f(-2.0f * x1)));
+        }
+        double r[3] = {a.pos[3 * p], a.pos[3 * p + 1], a.pos[3 * p + 2]};
+        pm[0] = a.mom[3 * p];
+        pm[1] = a.mom[3 * p + 1];
+        pm[2] = a.mom[3 * p + 2];
+        const double hd = 0.5 * (double)c.dt / (double)m;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) r[k] += hd * (double)pm[k];
+        confine_d(r, pm, g, KW);
+        if (!split(r, g, me) && lead) atomicOr(a.err, LB_DERR_PARTICLE_RANGE);
+        if (lead) a.sh[0][p] = pack(me);
+        if (c.use_wca) {
+            nnb = a.ncount[p];
+            const int *lst = a.nlist + (size_t)p * kMaxNb;
+#pragma unroll
+            for (int k = 0; k < kNbReg; ++k)
+                if (k < nnb) nb[k] = lst[k];
+            refp = unpack(a.ref[p]);
+        }
+        if (c.chain_len > 1) {
+            const int k = p % c.chain_len;
+            bond_lo = k > 0;
+            bond_hi = k < c.chain_len - 1 && p + 1 < c.n;
+        }
+    }
+    const int jlo = bond_lo ? p - 1 : self, jhi = bond_hi ? p + 1 : self;
+    int kmax = __reduce_max_sync(kFullMask, min(nnb, kNbReg));  // register slots any lane of the warp uses
+    int org[3];
+    {
+        Stencil<KW> st;
+        make_stencil<KW>(me, st);
+        org[0] = st.o[0];
+        org[1] = st.o[1];
+        org[2] = st.o[2];
+    }
+    float acc[kPer][3];
+    const auto gather = [&]() {
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+            const int qq = q + LANES * i;
+            if (kNodes % LANES == 0 || qq < kNodes) {
+                int x, y, z;
+                stencil_coords<KW>(org, qq, g, x, y, z);
+                float u[3];
+                node_velocity<DT>(src, a.ffield, x, y, z, g, u);
+                mine[qq] = make_float4(u[0], u[1], u[2], 0.0f);
+            }
+        }
+    };
+    const auto flush = [&]() {
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+            const int qq = q + LANES * i;
+            if (kNodes % LANES == 0 || qq < kNodes) {
+                int x, y, z;
+                stencil_coords<KW>(org, qq, g, x, y, z);
+                const size_t node = ((size_t)z * g.ny + y) * g.nx + x;
+                if (in_bounds(node, g.nn, g.err)) {
+                    atomicAdd(a.facc + node, acc[i][0]);
+                    atomicAdd(a.facc + g.pitch + node, acc[i][1]);
+                    atomicAdd(a.facc + 2 * g.pitch + node, acc[i][2]);
+                }
+                acc[i][0] = acc[i][1] = acc[i][2] = 0.0f;
+            }
+        }
+    };
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) acc[i][0] = acc[i][1] = acc[i][2] = 0.0f;
+    if (active) gather();
+    if (!grid_barrier(a.bar, a.err, a.spin_limit)) return;
+
+    bool binned = false;
+    const float h = 0.5f * c.dt / m;
+    for (int s = 0; s < a.nsub; ++s) {
+        const float4 *shin = a.sh[s & 1];
+        float4 *shout = a.sh[(s + 1) & 1];
+        // neighbour positions and the rebuild flag (written before the last
+        // barrier; L1 is bypassed), then the work of this particle alone
+        float4 v[kNbReg];
+#pragma unroll
+        for (int k = 0; k < kNbReg; ++k)
+            if (k < kmax) v[k] = __ldcg(shin + nb[k]);
+        const float4 vlo = __ldcg(shin + jlo), vhi = __ldcg(shin + jhi);
+        const unsigned int req = c.use_wca ? __ldcg(a.flags + 1 + (s & 1)) : 0u;
+        float th[3] = {0.f, 0.f, 0.f};
+        if (g.kT > 0.0f) particle_theta((uint32_t)p, c.md_step + (uint32_t)s, c, th);
+        Stencil<KW> st;
+        make_stencil<KW>(me, st);
+        float w[kPer];  // of the nodes this lane spreads to
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+            const int qq = q + LANES * i;
+            w[i] = 0.0f;
+            if (kNodes % LANES == 0 || qq < kNodes) {
+                int x, y, z;
+                w[i] = stencil_node_k<KW>(st, qq, g, x, y, z);
+            }
+        }
+
+        if (c.use_wca && req == a.epoch0 + (uint32_t)s) {
+            // a particle moved more than half the skin: re-bin all, rebuild every list
+            if (binned) {
+                if (lead) unbin_particle(p, a.head, a.bucket_of);
+                if (!grid_barrier(a.bar, a.err, a.spin_limit)) return;
+            }
+            if (lead) bin_particle(p, me, c, a.head, a.next, a.bucket_of);
+            if (!grid_barrier(a.bar, a.err, a.spin_limit)) return;
+            binned = true;
+            if (active) refp = me;
+            if (lead) {
+                nnb = build_own_list(p, me, shin, a.head, a.next, c, a.nlist + (size_t)p * kMaxNb, a.err);
+                a.ncount[p] = nnb;
+                a.ref[p] = pack(me);
+            }
+            __threadfence_block();  // the list the lead wrote, read by its group
+            __syncwarp();
+            nnb = __shfl_sync(kFullMask, nnb, 0, LANES);
+#pragma unroll
+            for (int k = 0; k < kNbReg; ++k) nb[k] = k < nnb ? __ldcg(a.nlist + (size_t)p * kMaxNb + k) : self;
+            kmax = __reduce_max_sync(kFullMask, min(nnb, kNbReg));
+#pragma unroll
+            for (int k = 0; k < kNbReg; ++k)
+                if (k < kmax) v[k] = __ldcg(shin + nb[k]);
+        }
+
+        // conservative forces at the half-step positions, from the external force
+        float F[3] = {c.fext[0], c.fext[1], c.fext[2]};
+        if (c.use_wca) {
+#pragma unroll
+            for (int k = 0; k < kNbReg; ++k)
+                if (k < kmax) wca_add(me, unpack(v[k]), c, F, k < nnb);
+            for (int k = kNbReg; k < nnb; ++k)
+                wca_add(me, unpack(__ldcg(shin + __ldcg(a.nlist + (size_t)p * kMaxNb + k))), c, F);
+        }
+        if (c.chain_len > 1) {
+            if (bond_lo && !fene_add(me, unpack(vlo), c, F)) atomicOr(a.err, LB_DERR_FENE_BROKEN);
+            if (bond_hi && !fene_add(me, unpack(vhi), c, F)) atomicOr(a.err, LB_DERR_FENE_BROKEN);
+        }
+        // (the row holds the velocities of this stencil: gathered before the
+        // first sub-step or, after a move, inside the previous barrier)
+        float up[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+        for (int n = 0; n < kNodes; ++n) {
+            const float wn = st.w[0][n % KW] * st.w[1][(n / KW) % KW] * st.w[2][n / (KW * KW)];
+            const float4 u = mine[n];
+            up[0] = fmaf(wn, u.x, up[0]);
+            up[1] = fmaf(wn, u.y, up[1]);
+            up[2] = fmaf(wn, u.z, up[2]);
+        }
+        if (active) {
+            float pn[3], J[3];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                pn[k] = C1 * pm[k] + C2 * (F[k] + G * up[k]) + C3 * th[k];
+                J[k] = pn[k] - pm[k] - c.dt * F[k];
+            }
+#pragma unroll
+            for (int i = 0; i < kPer; ++i)
+#pragma unroll
+                for (int k = 0; k < 3; ++k) acc[i][k] = fmaf(-J[k], w[i], acc[i][k]);
+            if (lead) a.records[(size_t)s * c.n + p] = stencil_record<KW>(me, g);
+
+            // second half drift of this sub-step, then the first of the next one
+            const bool last = (s == a.nsub - 1);
+            bool ok = drift(me, pn, h, g, KW);
+            if (last) {
+                if (lead) {
+                    a.pos[3 * p] = join1(me.c[0], me.f[0]);
+                    a.pos[3 * p + 1] = join1(me.c[1], me.f[1]);
+                    a.pos[3 * p + 2] = join1(me.c[2], me.f[2]);
+                    a.mom[3 * p] = pn[0];
+                    a.mom[3 * p + 1] = pn[1];
+                    a.mom[3 * p + 2] = pn[2];
+                }
+            } else {
+                ok = drift(me, pn, h, g, KW) && ok;
+            }
+            if (!ok && lead) atomicOr(a.err, LB_DERR_PARTICLE_RANGE);
+            pm[0] = pn[0];
+            pm[1] = pn[1];
+            pm[2] = pn[2];
+            if (lead) shout[p] = pack(me);
+            if (c.use_wca && lead) {
+                float d[3];
+                separation(me, refp, g, d);
+                const float d2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
+                if (!last && d2 > c.half_skin2) atomicMax(&a.flags[1 + ((s + 1) & 1)], a.epoch0 + (uint32_t)s + 1u);
+                if (last && d2 > 0.25f * c.half_skin2) a.flags[0] = 1u;  // build before the next call
+            }
+        }
+        if (s + 1 == a.nsub) break;  // nothing of another block is read after the last sub-step
+        // the barrier in two halves: between them, groups whose stencil origin
+        // moves for the next sub-step hand in their impulse sums and gather the
+        // new stencil (this reads only the frozen fluid and writes only
+        // registers and the accumulator, which no block reads during the call)
+        grid_arrive(a.bar, &ticket);
+        __syncwarp();  // the group has read its row
+        if (active) {
+            Stencil<KW> sn;
+            make_stencil<KW>(me, sn);
+            if (sn.o[0] != org[0] || sn.o[1] != org[1] || sn.o[2] != org[2]) {
+                flush();
+                org[0] = sn.o[0];
+                org[1] = sn.o[1];
+                org[2] = sn.o[2];
+                gather();
+            }
+        }
+        if (!grid_wait(a.bar, a.err, a.spin_limit, &ticket)) return;
+    }
+    if (active) flush();
+    if (binned) {  // (the same in every block) the others may still read the buckets
+        if (!grid_barrier(a.bar, a.err, a.spin_limit)) return;
+        if (lead) unbin_particle(p, a.head, a.bucket_of);
+    }
+}
+
+// ---------------------------------------------------------------------------
 // Free particles (no pair or bond forces): with the fluid frozen during a
 // call, a particle's sub-steps depend on no other particle, so one launch
 // runs all sub-steps of every particle with no grid barrier and no limit on
@@ -2115,6 +2394,114 @@ cudaError_t build_list_before(lb_handle *h, const lb_particles *pp, const Couple
     return e;
 }
 
+// One cooperative launch for the whole call: kernel `kfn` on `blocks` blocks of
+// kPThreads threads.  folds: the kernel clears the previous call's impulses
+// in its first phase when their records are those of one call with these
+// particles and this stencil; otherwise they are cleared before it.
+cudaError_t launch_persistent(lb_handle *h, const lb_particles *pp, const lb_couple_params *cp, const CoupleArgs &c,
+                              const void *kfn, int blocks, size_t smem, bool folds)
+{
+    Particles *P = h->parts;
+    const int n = pp->n;
+    const int span = c.kw == 3 ? 3 : (c.kw == 4 ? 4 : 2);
+    cudaError_t e = cudaSuccess;
+    if (c.use_wca && P->nlist_n != n) {
+        const unsigned int init[kFlagWords] = {0u, 0u, 1u, 0u, 0u};  // [2]: build before the launch
+        e = cudaMemcpyAsync(P->flags, init, sizeof(init), cudaMemcpyHostToDevice, h->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+        if (e != cudaSuccess) return e;
+        P->nlist_n = n;
+    }
+    const size_t need = (size_t)n * (size_t)cp->n_substeps, half = P->rec_cap / 2;
+    const bool fold_clear = folds && h->facc_stale && P->rec_span == span &&
+                            P->n_records == (size_t)n * (size_t)P->last_nsub && P->n_records <= half && need <= half;
+    if (h->facc_stale && !fold_clear) {
+        e = clear_particle_forces(h);
+        if (e != cudaSuccess) return e;
+        h->facc_stale = 0;
+    }
+    if (c.use_wca) {
+        e = build_list_before(h, pp, c);
+        if (e != cudaSuccess) return e;
+    }
+    PersistArgs a;
+    a.c = c;
+    a.nsub = cp->n_substeps;
+    a.src = h->pops[h->cur];
+    a.ffield = h->force;
+    a.pos = pp->pos;
+    a.mom = pp->mom;
+    a.mass = pp->mass;
+    a.gamma = pp->gamma;
+    a.sh[0] = P->shadow[0];
+    a.sh[1] = P->shadow[1];
+    a.nlist = P->nlist;
+    a.ncount = P->ncount;
+    a.ref = P->ref;
+    a.head = P->head;
+    a.next = P->next;
+    a.bucket_of = P->bucket_of;
+    a.facc = h->facc;
+    // the record buffer has two halves: the stale records (cleared in the
+    // kernel's first phase) stay in one, this call's go to the other
+    const size_t new_off = fold_clear ? (P->rec_off == 0 ? half : 0) : P->rec_off + P->n_records;
+    a.stale = fold_clear ? P->records + P->rec_off : nullptr;
+    a.nstale_sub = fold_clear ? P->last_nsub : 0;
+    a.records = P->records + new_off;
+    a.flags = P->flags + 2;
+    a.epoch0 = P->sub_counter + 1u;
+    a.bar = P->bar;
+    a.err = h->d_err;
+    a.spin_limit = 1u << 22;
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3(blocks);
+    lc.blockDim = dim3(kPThreads);
+    lc.dynamicSmemBytes = smem;
+    lc.stream = h->stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    lc.attrs = attr;
+    lc.numAttrs = 1;
+    void *args[] = {&a};
+    e = cudaLaunchKernelExC(&lc, kfn, args);
+    if (e != cudaSuccess) return e;
+    h->launches += 1;
+    if (fold_clear) {
+        P->rec_off = new_off;
+        P->n_records = 0;
+        h->facc_stale = 0;
+    }
+    note_records(P, n, need);
+    P->rec_span = std::max(P->rec_span, span);
+    P->sub_counter += (uint32_t)cp->n_substeps;
+    P->last_nsub = cp->n_substeps;
+    return cudaGetLastError();
+}
+
+// Blocks of kernel kfn that can be resident at once (0 where it cannot run).
+int resident_blocks(const void *kfn, size_t smem)
+{
+    int per_sm = 0;
+    cudaError_t e = cudaSuccess;
+    if (smem) e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kfn, kPThreads, smem);
+    if (e != cudaSuccess) {
+        (void)cudaGetLastError();
+        return 0;
+    }
+    return per_sm * device_sm_count();
+}
+
+// The lanes form: a warp a particle where that is at most two blocks per SM,
+// eight lanes otherwise.
+template <int DT>
+const void *lanes_kernel(int kw, bool warp)
+{
+    if (kw == 3) return warp ? (const void *)k_couple_lanes<DT, 3, 32> : (const void *)k_couple_lanes<DT, 3, 8>;
+    return warp ? (const void *)k_couple_lanes<DT, 4, 32> : (const void *)k_couple_lanes<DT, 4, 8>;
+}
+
 template <int DT>
 cudaError_t run_substeps(lb_handle *h, const lb_particles *pp, const lb_couple_params *cp)
 {
@@ -2171,159 +2558,27 @@ cudaError_t run_substeps(lb_handle *h, const lb_particles *pp, const lb_couple_p
     }
 
     // persistent path when every particle group can be resident at once
-    const int pblocks = (n + kPThreads - 1) / kPThreads;                                   // one thread a particle
-    int per_sm = 0;
-    if (!(cp->flags & LB_COUPLE_PER_SUBSTEP) && c.kw > 2) {
-        // phi_3 / phi_4: the persistent kernel with the stencil caches in shared memory
-        const size_t smem = c.kw == 3 ? wide_smem_bytes<3>() : wide_smem_bytes<4>();
-        const void *kfn = c.kw == 3 ? (const void *)k_couple_persistent_wide<DT, 3>
-                                    : (const void *)k_couple_persistent_wide<DT, 4>;
-        cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kfn, kPThreads, smem);
-        if (e != cudaSuccess) {
-            (void)cudaGetLastError();  // no wide persistent kernel here: the per-sub-step path below
-            per_sm = 0;
+    if (!(cp->flags & LB_COUPLE_PER_SUBSTEP)) {
+        const int sms = device_sm_count();
+        const int pblocks = (n + kPThreads - 1) / kPThreads;  // one thread a particle
+        const int wblocks = (int)(((size_t)n * 32 + kPThreads - 1) / kPThreads);
+        const int eblocks = (int)(((size_t)n * 8 + kPThreads - 1) / kPThreads);
+        if (c.kw > 2) {
+            // several lanes a particle while they can all be resident (up to
+            // ~9700 particles), the stencil caches in shared memory beyond
+            const bool warp = wblocks <= 2 * sms;
+            const int lblocks = warp ? wblocks : eblocks;
+            const void *lfn = lanes_kernel<DT>(c.kw, warp);
+            if (lblocks <= resident_blocks(lfn, 0)) return launch_persistent(h, pp, cp, c, lfn, lblocks, 0, true);
+            const size_t smem = c.kw == 3 ? wide_smem_bytes<3>() : wide_smem_bytes<4>();
+            const void *kfn = c.kw == 3 ? (const void *)k_couple_persistent_wide<DT, 3>
+                                        : (const void *)k_couple_persistent_wide<DT, 4>;
+            if (pblocks <= resident_blocks(kfn, smem)) return launch_persistent(h, pp, cp, c, kfn, pblocks, smem, false);
+        } else {
+            const void *kfn = h->n_nodes >= kLeanCouplingNodes ? (const void *)k_couple_persistent_lean<DT>
+                                                               : (const void *)k_couple_persistent<DT>;
+            if (pblocks <= resident_blocks(kfn, 0)) return launch_persistent(h, pp, cp, c, kfn, pblocks, 0, true);
         }
-        if (per_sm > 0 && pblocks <= per_sm * device_sm_count()) {
-            if (need_nlist && P->nlist_n != n) {
-                const unsigned int init[kFlagWords] = {0u, 0u, 1u, 0u, 0u};  // [2]: build before the launch
-                e = cudaMemcpyAsync(P->flags, init, sizeof(init), cudaMemcpyHostToDevice, h->stream);
-                if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-                if (e != cudaSuccess) return e;
-                P->nlist_n = n;
-            }
-            if (h->facc_stale) {
-                e = clear_particle_forces(h);
-                if (e != cudaSuccess) return e;
-                h->facc_stale = 0;
-            }
-            if (need_nlist) {
-                e = build_list_before(h, pp, c);
-                if (e != cudaSuccess) return e;
-            }
-            PersistArgs a;
-            a.c = c;
-            a.nsub = cp->n_substeps;
-            a.src = src;
-            a.ffield = h->force;
-            a.pos = pp->pos;
-            a.mom = pp->mom;
-            a.mass = pp->mass;
-            a.gamma = pp->gamma;
-            a.sh[0] = P->shadow[0];
-            a.sh[1] = P->shadow[1];
-            a.nlist = P->nlist;
-            a.ncount = P->ncount;
-            a.ref = P->ref;
-            a.head = P->head;
-            a.next = P->next;
-            a.bucket_of = P->bucket_of;
-            a.facc = h->facc;
-            a.records = P->records + P->rec_off + P->n_records;
-            a.stale = nullptr;
-            a.nstale_sub = 0;
-            a.flags = P->flags + 2;
-            a.epoch0 = P->sub_counter + 1u;
-            a.bar = P->bar;
-            a.err = h->d_err;
-            a.spin_limit = 1u << 22;
-            cudaLaunchConfig_t lc = {};
-            lc.gridDim = dim3(pblocks);
-            lc.blockDim = dim3(kPThreads);
-            lc.dynamicSmemBytes = smem;
-            lc.stream = h->stream;
-            cudaLaunchAttribute attr[1];
-            attr[0].id = cudaLaunchAttributeCooperative;
-            attr[0].val.cooperative = 1;
-            lc.attrs = attr;
-            lc.numAttrs = 1;
-            void *args[] = {&a};
-            e = cudaLaunchKernelExC(&lc, kfn, args);
-            if (e != cudaSuccess) return e;
-            h->launches += 1;
-            note_records(P, n, (size_t)n * (size_t)cp->n_substeps);
-            P->rec_span = std::max(P->rec_span, c.kw == 3 ? 3 : 4);
-            P->sub_counter += (uint32_t)cp->n_substeps;
-            P->last_nsub = cp->n_substeps;
-            return cudaGetLastError();
-        }
-    }
-    if (!(cp->flags & LB_COUPLE_PER_SUBSTEP) && c.kw == 2 &&
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)(h->n_nodes >= kLeanCouplingNodes ? k_couple_persistent_lean<DT> : k_couple_persistent<DT>), kPThreads, 0) == cudaSuccess &&
-        pblocks <= per_sm * device_sm_count()) {
-        cudaError_t e = cudaSuccess;
-        if (need_nlist && P->nlist_n != n) {
-            const unsigned int init[kFlagWords] = {0u, 0u, 1u, 0u, 0u};  // [2]: build before the launch
-            e = cudaMemcpyAsync(P->flags, init, sizeof(init), cudaMemcpyHostToDevice, h->stream);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-            if (e != cudaSuccess) return e;
-            P->nlist_n = n;
-        }
-        const bool fold_clear = h->facc_stale && P->rec_span == 2 && P->n_records == (size_t)n * (size_t)P->last_nsub &&
-                                P->n_records <= P->rec_cap / 2 && (size_t)n * cp->n_substeps <= P->rec_cap / 2;
-        if (h->facc_stale && !fold_clear) {
-            e = clear_particle_forces(h);
-            if (e != cudaSuccess) return e;
-            h->facc_stale = 0;
-        }
-        if (need_nlist) {
-            e = build_list_before(h, pp, c);
-            if (e != cudaSuccess) return e;
-        }
-        PersistArgs a;
-        a.c = c;
-        a.nsub = cp->n_substeps;
-        a.src = src;
-        a.ffield = h->force;
-        a.pos = pp->pos;
-        a.mom = pp->mom;
-        a.mass = pp->mass;
-        a.gamma = pp->gamma;
-        a.sh[0] = P->shadow[0];
-        a.sh[1] = P->shadow[1];
-        a.nlist = P->nlist;
-        a.ncount = P->ncount;
-        a.ref = P->ref;
-        a.head = P->head;
-        a.next = P->next;
-        a.bucket_of = P->bucket_of;
-        a.facc = h->facc;
-        // the record buffer has two halves: the stale records (cleared in the
-        // kernel's first phase) stay in one, this call's go to the other
-        const size_t half = P->rec_cap / 2;
-        const size_t new_off = fold_clear ? (P->rec_off == 0 ? half : 0) : P->rec_off + P->n_records;
-        a.stale = fold_clear ? P->records + P->rec_off : nullptr;
-        a.nstale_sub = fold_clear ? P->last_nsub : 0;
-        a.records = P->records + new_off;
-        a.flags = P->flags + 2;
-        a.epoch0 = P->sub_counter + 1u;
-        a.bar = P->bar;
-        a.err = h->d_err;
-        a.spin_limit = 1u << 22;
-        cudaLaunchConfig_t lc = {};
-        lc.gridDim = dim3(pblocks);
-        lc.blockDim = dim3(kPThreads);
-        lc.stream = h->stream;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeCooperative;
-        attr[0].val.cooperative = 1;
-        lc.attrs = attr;
-        lc.numAttrs = 1;
-        void *args[] = {&a};
-        const void *kfn = h->n_nodes >= kLeanCouplingNodes ? (const void *)k_couple_persistent_lean<DT>
-                                                           : (const void *)k_couple_persistent<DT>;
-        e = cudaLaunchKernelExC(&lc, kfn, args);
-        if (e != cudaSuccess) return e;
-        h->launches += 1;
-        if (fold_clear) {
-            P->rec_off = new_off;
-            P->n_records = 0;
-            h->facc_stale = 0;
-        }
-        note_records(P, n, (size_t)n * (size_t)cp->n_substeps);
-        P->sub_counter += (uint32_t)cp->n_substeps;
-        P->last_nsub = cp->n_substeps;
-        return cudaGetLastError();
     }
 
     if (h->facc_stale) {
