@@ -83,6 +83,15 @@ StepArgs make_args(const lb_handle *h)
                                     : std::sqrt(1.0 - p.gamma_even * p.gamma_even);
         a.amp[k - 4] = (float)(phi * (double)lbd::sqrt_inv_w(k));
     }
+    const double gm[4] = {p.gamma_bulk, p.gamma_shear, p.gamma_odd, p.gamma_even};
+    for (int k = 4; k < 19; ++k)
+        a.rel[k - 4] = (float)(gm[k == 4 ? 0 : k < 10 ? 1 : k < 16 ? 2 : 3] * (double)lbd::inv_w(k));
+    for (int q = 0; q < 4; ++q) {
+        const double g = q == 0 ? p.gamma_bulk : p.gamma_shear, iw = (double)lbd::inv_w(4 + q);
+        a.eq[q] = (float)((1.0 - g) * iw);
+        a.frc[q] = (float)((1.0 + g) * iw * (q == 3 ? 0.5 : 1.0));
+    }
+    a.forced = h->force || p.body_force[0] != 0.0 || p.body_force[1] != 0.0 || p.body_force[2] != 0.0;
     a.fx = (float)p.body_force[0];
     a.fy = (float)p.body_force[1];
     a.fz = (float)p.body_force[2];

@@ -44,8 +44,7 @@ struct BatchDesc {
     uint32_t replica;  // Philox counter word 3
     uint32_t phase;    // offset of this replica's phase table (mode records)
     Div dx, dxy;
-    lbd::RoundKeys rk;
-    uint32_t key0, key1;  // the seed's two key words (the paired kernels form the round keys from them)
+    uint32_t key0, key1;  // the seed's two key words (the kernels form the round keys from them)
 };
 
 struct BatchTile {
@@ -66,7 +65,6 @@ struct BatchArgs {
     int ntiles;
     void *pops[2];
     int nsteps;
-    int nodes_per_thread;
     BatchState *state;
     unsigned int *bar;  // [0] arrivals, [1] generation, [2] abort
     unsigned int *err;
@@ -95,60 +93,14 @@ __device__ __forceinline__ bool batch_barrier(const BatchArgs &a)
     return lbi::grid_barrier(a.bar, a.err, a.spin_limit);
 }
 
-template <int DT, bool NOISE, bool OBS>
-__device__ __forceinline__ void batch_node(const BatchDesc &d, uint32_t s, const typename lbd::Store<DT>::T *src,
-                                           typename lbd::Store<DT>::T *dst, const StepArgs &ph, uint32_t step,
-                                           const float2 *phase, float acc[kModeVals])
+template <bool NOISE>
+__device__ __forceinline__ void collide_tile_pair(const lbp::F2 m[19], const StepArgs &ph, const BatchDesc &d, uint32_t s,
+                                                  uint32_t step, lbp::F2 out[19])
 {
-    using S = lbd::Store<DT>;
-    const uint32_t row = divide(s, d.dx);
-    const int x = (int)(s - row * (uint32_t)d.nx);
-    const uint32_t zz = divide(s, d.dxy);
-    const int y = (int)(row - zz * (uint32_t)d.ny);
-    const int z = (int)zz;
-    const int xm = (x == 0) ? d.nx - 1 : x - 1, xp = (x == d.nx - 1) ? 0 : x + 1;
-    const int ym = (y == 0) ? d.ny - 1 : y - 1, yp = (y == d.ny - 1) ? 0 : y + 1;
-    const int zm = (z == 0) ? d.nz - 1 : z - 1, zp = (z == d.nz - 1) ? 0 : z + 1;
-    const size_t P = d.pitch;
-    const typename S::T *base = src + d.off;
-    float n[19];
-#pragma unroll
-    for (int i = 0; i < 19; ++i) {
-        const int sx = lbd::cx(i) == 1 ? xm : (lbd::cx(i) == -1 ? xp : x);
-        const int sy = lbd::cy(i) == 1 ? ym : (lbd::cy(i) == -1 ? yp : y);
-        const int sz = lbd::cz(i) == 1 ? zm : (lbd::cz(i) == -1 ? zp : z);
-        const uint32_t off = (uint32_t)((sz * d.ny + sy) * d.nx + sx);
-        n[i] = in_bounds((size_t)i * P + off, 19 * P, ph.err) ? S::cvt(__ldcg(base + (size_t)i * P + off), ph.inv_scale)
-                                                             : 0.0f;
-    }
-    StepArgs a = ph;
-    a.step = step;
-    float m[19], out[19];
-    lbd::forward(n, m);
-    if (OBS) {  // u = (sum n c + f/2) / rho of the streamed state (Sec. 3.7)
-        const float ir = 1.0f / (ph.rho0 + m[0]);
-        const float ux = (m[1] + 0.5f * ph.fx) * ir, uy = (m[2] + 0.5f * ph.fy) * ir, uz = (m[3] + 0.5f * ph.fz) * ir;
-        const float2 ex = __ldg(phase + d.phase + x);
-        const float2 ey = __ldg(phase + d.phase + d.nx + y);
-        const float2 ez = __ldg(phase + d.phase + d.nx + d.ny + z);
-        acc[0] = fmaf(ux, ez.x, acc[0]);
-        acc[1] = fmaf(ux, ez.y, acc[1]);
-        acc[2] = fmaf(uy, ez.x, acc[2]);
-        acc[3] = fmaf(uy, ez.y, acc[3]);
-        acc[4] = fmaf(uy, ex.x, acc[4]);
-        acc[5] = fmaf(uy, ex.y, acc[5]);
-        acc[6] = fmaf(uz, ex.x, acc[6]);
-        acc[7] = fmaf(uz, ex.y, acc[7]);
-        acc[8] = fmaf(uz, ey.x, acc[8]);
-        acc[9] = fmaf(uz, ey.y, acc[9]);
-        acc[10] = fmaf(ux, ey.x, acc[10]);
-        acc[11] = fmaf(ux, ey.y, acc[11]);
-    }
-    collide_moments<NOISE>(m, ph.fx, ph.fy, ph.fz, a, d.rk, s, d.replica, out);
-    typename S::T *o = dst + d.off;
-#pragma unroll
-    for (int i = 0; i < 19; ++i)
-        if (in_bounds((size_t)i * P + s, 19 * P, ph.err)) o[(size_t)i * P + s] = S::pack(out[i], ph.scale);
+    lbp::F2 M[19], rho;
+    lbp::relax2(m, lbp::f2s(ph.fx), lbp::f2s(ph.fy), lbp::f2s(ph.fz), ph, M, rho);
+    if (NOISE) lbp::add_noise2(M, rho, ph, lbp::RunningKeys{d.key0, d.key1}, s, step, d.replica);
+    lbp::backward2(M, out);
 }
 
 // Nodes s and s + 1 (s even, nx even: the same row) of replica d: the pair
@@ -219,8 +171,6 @@ __device__ __forceinline__ void batch_pair(const BatchDesc &d, uint32_t s, const
         }
         n[i] = DT == 0 ? lbp::f2(v0, v1) : lbp::f2(v0, v1) * lbp::f2s(ph.inv_scale);
     }
-    StepArgs a = ph;
-    a.step = step;
     lbp::F2 m[19], out[19];
     lbp::forward2(n, m);
     const lbp::F2 fx = lbp::f2s(ph.fx), fy = lbp::f2s(ph.fy), fz = lbp::f2s(ph.fz);
@@ -256,13 +206,87 @@ __device__ __forceinline__ void batch_pair(const BatchDesc &d, uint32_t s, const
         acc[10] = fmaf(sx, ey.x, acc[10]);
         acc[11] = fmaf(sx, ey.y, acc[11]);
     }
-    lbp::collide_moments2k<NOISE>(m, fx, fy, fz, a, lbp::RunningKeys{d.key0, d.key1}, s, d.replica, out);
+    collide_tile_pair<NOISE>(m, ph, d, s, step, out);
     typename S::T *o = dst + d.off;
 #pragma unroll
     for (int i = 0; i < 19; ++i) {
         float o0, o1;
         lbp::split(DT == 0 ? out[i] : out[i] * lbp::f2s(ph.scale), o0, o1);
         if (in_bounds((uint32_t)i * P + s + 1, 19 * (size_t)P, ph.err)) Pair<DT>::store(o + (uint32_t)i * P + s, o0, o1, 1.0f);
+    }
+}
+
+// Box of a replica as the pull functions take it (periodic).
+struct TileGeo {
+    int nx, ny, nz, z0, z1;
+    size_t pitch;
+};
+
+// The same for a replica with rows of odd length: the pair (s even) may
+// straddle two rows or planes, and its second node may not exist (the last of
+// an odd number of nodes), so each node takes its own addresses.
+template <int DT, bool NOISE, bool OBS>
+__device__ __forceinline__ void batch_pair_any(const BatchDesc &d, uint32_t s, const typename lbd::Store<DT>::T *src,
+                                               typename lbd::Store<DT>::T *dst, const StepArgs &ph, uint32_t step,
+                                               const float2 *phase, float acc[kModeVals])
+{
+    using S = lbd::Store<DT>;
+    const TileGeo g{d.nx, d.ny, d.nz, 0, d.nz, d.pitch};
+    PairAt at;
+    const uint32_t row = divide(s, d.dx), zz = divide(s, d.dxy);
+    at.s = s;
+    at.x = (int)(s - row * (uint32_t)d.nx);
+    at.y = (int)(row - zz * (uint32_t)d.ny);
+    at.z = (int)zz;
+    at.va = true;
+    at.vb = s + 1u < d.nodes;
+    int xb, yb, zb;
+    second_node(g, at, xb, yb, zb);
+    const PullAt pa = pull_at<false>(g, at.x, at.y, at.z), pb = pull_at<false>(g, xb, yb, zb);
+    const size_t P = d.pitch;
+    const typename S::T *base = src + d.off;
+    lbp::F2 n[19], m[19], out[19];
+#pragma unroll
+    for (int i = 0; i < 19; ++i) {
+        const size_t ka = pull_index<false>(g, pa, i), kb = pull_index<false>(g, pb, i);
+        const lbp::F2 v = lbp::f2(in_bounds(ka, 19 * P, ph.err) ? S::cvt(__ldcg(base + ka), 1.0f) : 0.0f,
+                                  in_bounds(kb, 19 * P, ph.err) ? S::cvt(__ldcg(base + kb), 1.0f) : 0.0f);
+        n[i] = DT == 0 ? v : v * lbp::f2s(ph.inv_scale);
+    }
+    lbp::forward2(n, m);
+    if (OBS) {
+        const lbp::F2 rho = lbp::f2s(ph.rho0) + m[0];
+        float rl, rh;
+        lbp::split(rho, rl, rh);
+        const float2 *px = phase + d.phase, *py = px + d.nx, *pz = py + d.ny;
+        const auto add = [&](float ir, float mx, float my, float mz, int x, int y, int z) {
+            const float ux = (mx + 0.5f * ph.fx) * ir, uy = (my + 0.5f * ph.fy) * ir, uz = (mz + 0.5f * ph.fz) * ir;
+            const float2 ex = __ldg(px + x), ey = __ldg(py + y), ez = __ldg(pz + z);
+            acc[0] = fmaf(ux, ez.x, acc[0]);
+            acc[1] = fmaf(ux, ez.y, acc[1]);
+            acc[2] = fmaf(uy, ez.x, acc[2]);
+            acc[3] = fmaf(uy, ez.y, acc[3]);
+            acc[4] = fmaf(uy, ex.x, acc[4]);
+            acc[5] = fmaf(uy, ex.y, acc[5]);
+            acc[6] = fmaf(uz, ex.x, acc[6]);
+            acc[7] = fmaf(uz, ex.y, acc[7]);
+            acc[8] = fmaf(uz, ey.x, acc[8]);
+            acc[9] = fmaf(uz, ey.y, acc[9]);
+            acc[10] = fmaf(ux, ey.x, acc[10]);
+            acc[11] = fmaf(ux, ey.y, acc[11]);
+        };
+        add(1.0f / rl, lbp::lo(m[1]), lbp::lo(m[2]), lbp::lo(m[3]), at.x, at.y, at.z);
+        if (at.vb) add(1.0f / rh, lbp::hi(m[1]), lbp::hi(m[2]), lbp::hi(m[3]), xb, yb, zb);
+    }
+    collide_tile_pair<NOISE>(m, ph, d, s, step, out);
+    typename S::T *o = dst + d.off + s;
+#pragma unroll
+    for (int i = 0; i < 19; ++i) {
+        float o0, o1;
+        lbp::split(DT == 0 ? out[i] : out[i] * lbp::f2s(ph.scale), o0, o1);
+        if (!in_bounds((size_t)i * P + s + (at.vb ? 1 : 0), 19 * P, ph.err)) continue;
+        if (at.vb) Pair<DT>::store(o + (size_t)i * P, o0, o1, 1.0f);
+        else o[(size_t)i * P] = S::pack(o0, 1.0f);
     }
 }
 
@@ -290,7 +314,8 @@ __device__ __forceinline__ void record_warp(const float acc[kModeVals], double *
     if (rec && !(lane & 1) && pos < 3) atomicAdd(rec + k, (double)v);
 }
 
-template <int DT, bool NOISE, bool OBS, bool PAIR>
+// ODD: some replica has rows of odd length (pairs node by node).
+template <int DT, bool NOISE, bool OBS, bool ODD>
 __device__ __forceinline__ void batch_run(const BatchArgs &a)
 {
     using T = typename lbd::Store<DT>::T;
@@ -305,16 +330,11 @@ __device__ __forceinline__ void batch_run(const BatchArgs &a)
             const BatchTile tl = a.tiles[tile];
             const BatchDesc &d = a.desc[tl.rep];
             float acc[kModeVals];
-            if (PAIR) {  // every replica has even nx: tiles hold whole pairs
 #pragma unroll
-                for (int q = 0; q < kModeVals; ++q) acc[q] = 0.0f;
-                for (uint32_t k = 2 * threadIdx.x; k < tl.count; k += 2 * blockDim.x)
-                    batch_pair<DT, NOISE, OBS>(d, tl.begin + k, src, dst, a.phys, step, a.phase, acc);
-            } else {
-#pragma unroll
-                for (int q = 0; q < kModeVals; ++q) acc[q] = 0.0f;
-                for (uint32_t k = threadIdx.x; k < tl.count; k += blockDim.x)
-                    batch_node<DT, NOISE, OBS>(d, tl.begin + k, src, dst, a.phys, step, a.phase, acc);
+            for (int q = 0; q < kModeVals; ++q) acc[q] = 0.0f;
+            for (uint32_t k = 2 * threadIdx.x; k < tl.count; k += 2 * blockDim.x) {
+                if (ODD) batch_pair_any<DT, NOISE, OBS>(d, tl.begin + k, src, dst, a.phys, step, a.phase, acc);
+                else batch_pair<DT, NOISE, OBS>(d, tl.begin + k, src, dst, a.phys, step, a.phase, acc);
             }
             if (OBS) {
                 double *rec = trec < a.rec_cap ? a.modes + ((size_t)tl.rep * a.rec_cap + trec) * kModeVals : nullptr;
@@ -331,22 +351,16 @@ __device__ __forceinline__ void batch_run(const BatchArgs &a)
     }
 }
 
-template <int DT, bool NOISE, bool OBS>
-__global__ void k_batch(BatchArgs a)
-{
-    batch_run<DT, NOISE, OBS, false>(a);
-}
-
-template <int DT, bool NOISE>
+template <int DT, bool NOISE, bool ODD>
 __global__ void __maxnreg__(kBatchPairMaxRegs) k_batch_pair(BatchArgs a)
 {
-    batch_run<DT, NOISE, false, true>(a);
+    batch_run<DT, NOISE, false, ODD>(a);
 }
 
-template <int DT, bool NOISE>
+template <int DT, bool NOISE, bool ODD>
 __global__ void __maxnreg__(kBatchPairObsMaxRegs) k_batch_pair_obs(BatchArgs a)
 {
-    batch_run<DT, NOISE, true, true>(a);
+    batch_run<DT, NOISE, true, ODD>(a);
 }
 
 __global__ void k_set_rec_step0(BatchState *st, uint32_t v)
@@ -415,7 +429,7 @@ struct lb_batch {
     int rec_cap = 0;
     uint32_t rec_step0 = 0;
     float2 *phase = nullptr;        // library: per-replica (cos, -sin) tables
-    bool pairs = false;             // every replica has even nx: two nodes per thread
+    bool pairs = false;             // every replica has even nx: pairs lie in one row
 };
 
 using namespace lbi;
@@ -437,8 +451,8 @@ lb_status build_tiles(lb_batch *b, int tile_nodes)
     std::vector<BatchTile> tl;
     for (int r = 0; r < b->n; ++r) {
         const uint32_t nodes = b->desc_h[r].nodes;
-        for (uint32_t s = 0; s < nodes; s += (uint32_t)tile_nodes)
-            tl.push_back(BatchTile{r, s, std::min<uint32_t>((uint32_t)tile_nodes, nodes - s)});
+        const uint32_t run = ((uint32_t)tile_nodes + 1u) & ~1u;  // pairs start at even nodes
+        for (uint32_t s = 0; s < nodes; s += run) tl.push_back(BatchTile{r, s, std::min<uint32_t>(run, nodes - s)});
     }
     // largest replicas' tiles first gives the strided schedule a balanced tail
     std::stable_sort(tl.begin(), tl.end(), [&](const BatchTile &x, const BatchTile &y) {
@@ -467,10 +481,10 @@ StepArgs batch_phys(const lb_batch *b)
 }
 
 template <int DT, bool NOISE, bool OBS>
-void *kernel_ptr(bool pair)
+void *kernel_ptr(bool even)
 {
-    if (!pair) return (void *)k_batch<DT, NOISE, OBS>;
-    return OBS ? (void *)k_batch_pair_obs<DT, NOISE> : (void *)k_batch_pair<DT, NOISE>;
+    if (OBS) return even ? (void *)k_batch_pair_obs<DT, NOISE, false> : (void *)k_batch_pair_obs<DT, NOISE, true>;
+    return even ? (void *)k_batch_pair<DT, NOISE, false> : (void *)k_batch_pair<DT, NOISE, true>;
 }
 
 template <bool OBS>
@@ -510,7 +524,6 @@ cudaError_t launch_batch(lb_batch *b, int nsteps)
     a.pops[0] = b->pops[0];
     a.pops[1] = b->pops[1];
     a.nsteps = nsteps;
-    a.nodes_per_thread = 1;
     a.state = b->state;
     a.bar = b->bar;
     a.err = b->err;
@@ -654,7 +667,6 @@ lb_status lb_batch_create(const lb_params *per_replica, int n, void *pops_a, voi
         d.phase = 0;  // set by lb_batch_record_modes
         d.dx = make_div((uint32_t)p.nx);
         d.dxy = make_div((uint32_t)(p.nx * p.ny));
-        d.rk = lbd::make_round_keys(p.seed);
         d.key0 = (uint32_t)(p.seed & 0xffffffffu);
         d.key1 = (uint32_t)(p.seed >> 32);
         b->desc_h.push_back(d);

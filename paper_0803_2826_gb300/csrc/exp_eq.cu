@@ -221,22 +221,7 @@ __device__ __forceinline__ void collide_exp2(const F2 m[19], F2 fx, F2 fy, F2 fz
     for (int k = 10; k < 16; ++k) M[k] = lbp::fma2(lbp::f2s(a.g_odd), m[k] - meq[k], meq[k]) * lbd::inv_w(k);
 #pragma unroll
     for (int k = 16; k < 19; ++k) M[k] = lbp::fma2(lbp::f2s(a.g_even), m[k] - meq[k], meq[k]) * lbd::inv_w(k);
-    if (NOISE) {
-        const F2 sd = lbp::noise_sd(a, rho);
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            const lbd::U4 r0 = lbd::philox10(lbd::U4{node0, a.step, (uint32_t)b, a.replica}, a.rk);
-            const lbd::U4 r1 = lbd::philox10(lbd::U4{node0 + 1u, a.step, (uint32_t)b, a.replica}, a.rk);
-            F2 g[4];
-            lbp::box_muller2(r0.x, r0.y, r1.x, r1.y, g[0], g[1], sd);
-            lbp::box_muller2(r0.z, r0.w, r1.z, r1.w, g[2], g[3], sd);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int k = 4 + 4 * b + j;
-                if (k < 19) M[k] = lbp::fma2(g[j], a.amp[k - 4], M[k]);
-            }
-        }
-    }
+    if (NOISE) lbp::add_noise2(M, rho, a, lbp::ParamKeys{a.rk}, node0, a.step, a.replica);
     lbp::backward2(M, out);
 }
 

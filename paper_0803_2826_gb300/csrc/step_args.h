@@ -48,7 +48,11 @@ struct StepArgs {
     float g_shear, g_bulk, g_odd, g_even;
     float phi_shear, phi_bulk, phi_odd, phi_even;  // sqrt(1 - gamma^2)
     float amp[15];         // noise of mode k = 4..18 per unit sqrt(mu rho): phi_k / sqrt(w_k)
+    float rel[15];         // gamma_k / w_k of mode k = 4..18
+    float eq[4];           // (1 - gamma_k) / w_k of modes 4, 5, 6 and 7..9
+    float frc[4];          // (1 + gamma_k) / w_k of modes 4, 5, 6, half of it of modes 7..9
     float fx, fy, fz;      // uniform body force
+    int forced;            // a body force, a force field or particle impulses act
     float scale, inv_scale;  // storage scale of FP16/BF16 deviations
     int noise_rho0;
     uint32_t key0, key1;   // Philox key (seed)

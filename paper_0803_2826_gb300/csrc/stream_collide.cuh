@@ -6,7 +6,7 @@
 // the nodes in one of two ways.  Rows whose pairs fill whole blocks (nx a
 // multiple of 256) keep one row per block: no division, y and z from the
 // block index (k_stream_collide2; 256^3 FP32 with noise 383 us a step against
-// 389 us in the linear mapping).  All other boxes run over the linear node
+// 389 us in the linear mapping when the two were compared).  All other boxes run over the linear node
 // index (k_stream_collide_linear), so no lane is idle however short or odd the
 // rows are: 64^3 10.3 us against 12.3 us with a block per row, 200^3 189 us
 // against 248 us, and rows of odd length, which went one node a thread in
@@ -643,7 +643,8 @@ __device__ __forceinline__ bool locate_pair(const StepArgs &a, PairAt &p)
     return true;
 }
 
-// Pull addresses of one node: row offsets of its neighbours and their x.
+// Pull addresses of one node: row offsets of its neighbours and their x.  The
+// box (nx, ny, nz, z0, z1, pitch) comes from any struct that has them.
 struct PullAt {
     int x[3];          // x - 1, x, x + 1 (wrapped)
     uint32_t y[3], z[3];  // row offsets y nx and plane offsets z nx ny, the same way
@@ -651,8 +652,8 @@ struct PullAt {
     bool lo, hi;       // next to the lower / upper wall: c_z = +1 / -1 bounce back
 };
 
-template <bool WALLS>
-__device__ __forceinline__ PullAt pull_at(const StepArgs &a, int x, int y, int z)
+template <bool WALLS, class Geo>
+__device__ __forceinline__ PullAt pull_at(const Geo &a, int x, int y, int z)
 {
     PullAt p;
     p.x[0] = x == 0 ? a.nx - 1 : x - 1;
@@ -678,8 +679,8 @@ __device__ __forceinline__ PullAt pull_at(const StepArgs &a, int x, int y, int z
 }
 
 // Index of the stored entry that population i of the node is pulled from.
-template <bool WALLS>
-__device__ __forceinline__ size_t pull_index(const StepArgs &a, const PullAt &p, int i)
+template <bool WALLS, class Geo>
+__device__ __forceinline__ size_t pull_index(const Geo &a, const PullAt &p, int i)
 {
     const uint32_t off = p.z[1 - lbd::cz(i)] + p.y[1 - lbd::cy(i)] + (uint32_t)p.x[1 - lbd::cx(i)];
     const bool bounce = WALLS && ((lbd::cz(i) == 1 && p.lo) || (lbd::cz(i) == -1 && p.hi));
@@ -696,7 +697,8 @@ __device__ __forceinline__ float pull_one(const typename lbd::Store<DT>::T *__re
 }
 
 // Node s + 1 of a located pair; the located node itself where there is only one.
-__device__ __forceinline__ void second_node(const StepArgs &a, const PairAt &at, int &xb, int &yb, int &zb)
+template <class Geo>
+__device__ __forceinline__ void second_node(const Geo &a, const PairAt &at, int &xb, int &yb, int &zb)
 {
     xb = at.x;
     yb = at.y;
@@ -869,7 +871,8 @@ cudaError_t launch_stream_collide_dt(const lb_handle *h, const void *src, void *
                                      float *partials)
 {
     using T = typename lbd::Store<DT>::T;
-    const StepArgs a = make_args(h);
+    StepArgs a = make_args(h);
+    a.forced |= facc != nullptr;
     const dim3 grid = sc_grid(h);
     const dim3 block(kBX);
     const bool noise = a.kT > 0.0f;
