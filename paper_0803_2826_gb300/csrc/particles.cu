@@ -1452,27 +1452,18 @@ __device__ __forceinline__ void couple_persistent_run(const PersistArgs &a)
     }
 }
 
-// The phi_2 persistent coupling, and the same code capped at 112 registers
-// for large boxes: its blocks then leave room for five instead of four
-// stream-collide blocks on the SMs they share while the two run side by side.
-// The cap spills (the coupling takes ~0.37 instead of ~0.23 ms at 256^3,
-// still shorter than the stream-collide launch beside it, 0.44 ms) and took
-// the 256^3 step from 0.470 to 0.464 ms; in small boxes, where the coupling
-// is the longer of the two, the uncapped kernel is faster.
+// The phi_2 persistent coupling.  168 registers, no spills: beside the
+// stream-collide launch of a 256^3 box (80 registers) it leaves four of that
+// kernel's six blocks on the SMs it shares, and ends in 0.22 ms; capped at
+// 112 registers it left five but spilled and took 0.40 ms, for the same
+// stream-collide time (0.41 ms) and a longer step (0.4289 against 0.4257 ms).
+// Blocks of 256 or 512 particles on fewer SMs slowed the launch beside them
+// more (0.418 ms).
 template <int DT>
 __global__ void __launch_bounds__(kPThreads) k_couple_persistent(PersistArgs a)
 {
     couple_persistent_run<DT>(a);
 }
-
-template <int DT>
-__global__ void __maxnreg__(112) k_couple_persistent_lean(PersistArgs a)
-{
-    couple_persistent_run<DT>(a);
-}
-
-// Boxes from this many nodes take k_couple_persistent_lean.
-constexpr size_t kLeanCouplingNodes = (size_t)1 << 24;
 
 // ---------------------------------------------------------------------------
 // Persistent variant for the wide stencils (phi_3, phi_4: 27 / 64 nodes) of
@@ -2575,8 +2566,7 @@ cudaError_t run_substeps(lb_handle *h, const lb_particles *pp, const lb_couple_p
                                         : (const void *)k_couple_persistent_wide<DT, 4>;
             if (pblocks <= resident_blocks(kfn, smem)) return launch_persistent(h, pp, cp, c, kfn, pblocks, smem, false);
         } else {
-            const void *kfn = h->n_nodes >= kLeanCouplingNodes ? (const void *)k_couple_persistent_lean<DT>
-                                                               : (const void *)k_couple_persistent<DT>;
+            const void *kfn = (const void *)k_couple_persistent<DT>;
             if (pblocks <= resident_blocks(kfn, 0)) return launch_persistent(h, pp, cp, c, kfn, pblocks, 0, true);
         }
     }

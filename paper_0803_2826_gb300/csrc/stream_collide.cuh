@@ -290,12 +290,16 @@ __global__ void __launch_bounds__(kBX) k_patch_impulse_nodes(const typename lbd:
     if (t >= n * 8) return;
     const int p = t >> 3, q = t & 7;
     const int nk = span * span * span;
-    int prev = -1;
+    const unsigned group = 0xFFu << (threadIdx.x & 24);
+    int prev = -1, mine = 0;
     for (int s = 0; s < nsub; ++s) {
-        const int base = records[(size_t)s * n + p];
+        // eight sub-steps' records at a time, one in a lane: one load's latency for all
+        if ((s & 7) == 0) mine = s + q < nsub ? records[(size_t)(s + q) * n + p] : -1;
+        const int base = __shfl_sync(group, mine, s & 7, 8);
         if (base == prev) continue;  // same cell as the sub-step before
         prev = base;
-        const int bx = base % a.nx, by = (base / a.nx) % a.ny, bz = base / (a.nx * a.ny);
+        const uint32_t row = divide((uint32_t)base, a.dnx), plane = divide(row, a.dny);
+        const int bx = base - (int)(row * (uint32_t)a.nx), by = (int)(row - plane * (uint32_t)a.ny), bz = (int)plane;
         for (int e = q; e < nk; e += 8) {
             int x, y, z;
             if (!patch_node<WALLS>(bx, by, bz, e, span, a, x, y, z)) continue;  // solid node
@@ -332,12 +336,16 @@ __global__ void __launch_bounds__(kBX, 8) k_patch_impulse_nodes_f32(float *dst, 
     const int p = t >> 3, q = t & 7;
     const size_t P = a.pitch;
     const int nk = span * span * span;
-    int prev = -1;
+    const unsigned group = 0xFFu << (threadIdx.x & 24);
+    int prev = -1, mine = 0;
     for (int s = 0; s < nsub; ++s) {
-        const int base = records[(size_t)s * n + p];
+        // eight sub-steps' records at a time, one in a lane: one load's latency for all
+        if ((s & 7) == 0) mine = s + q < nsub ? records[(size_t)(s + q) * n + p] : -1;
+        const int base = __shfl_sync(group, mine, s & 7, 8);
         if (base == prev) continue;  // same cell as the sub-step before
         prev = base;
-        const int bx = base % a.nx, by = (base / a.nx) % a.ny, bz = base / (a.nx * a.ny);
+        const uint32_t row = divide((uint32_t)base, a.dnx), plane = divide(row, a.dny);
+        const int bx = base - (int)(row * (uint32_t)a.nx), by = (int)(row - plane * (uint32_t)a.ny), bz = (int)plane;
         for (int e = q; e < nk; e += 8) {
             int x, y, z;
             if (!patch_node<WALLS>(bx, by, bz, e, span, a, x, y, z)) continue;  // solid node
