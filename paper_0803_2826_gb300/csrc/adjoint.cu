@@ -25,9 +25,9 @@
 
 namespace lbi {
 
-extern template cudaError_t launch_stream_collide_dt<0>(const lb_handle *, const void *, void *, const float *, float *);
-extern template cudaError_t launch_stream_collide_dt<1>(const lb_handle *, const void *, void *, const float *, float *);
-extern template cudaError_t launch_stream_collide_dt<2>(const lb_handle *, const void *, void *, const float *, float *);
+extern template cudaError_t launch_stream_collide_dt<0>(const lb_handle *, const void *, void *, float *, float *);
+extern template cudaError_t launch_stream_collide_dt<1>(const lb_handle *, const void *, void *, float *, float *);
+extern template cudaError_t launch_stream_collide_dt<2>(const lb_handle *, const void *, void *, float *, float *);
 
 namespace {
 
@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(kLinBX)
     // rho and u of the forward step; al_i = a_i lambda_i
     F2 n[19], m[4], al[19];
     float f0[3], f1[3];
-    load_linear<DT, true, WALLS, ODD>(state, ffield, impulse, a, at, n, f0, f1);
+    load_linear<DT, true, WALLS, ODD>(state, ffield, const_cast<float *>(impulse), a, at, n, f0, f1);  // (only read)
 #pragma unroll
     for (int i = 0; i < 19; ++i) {  // s is even, and s + 1 lies in the plane's padding at most
         const float *p = lam_in + (size_t)i * P + at.s;
@@ -408,7 +408,7 @@ cudaError_t launch_seed(const lb_handle *h, const void *state, float *lam_out, f
     }
 }
 
-cudaError_t step_from(lb_handle *h, const void *src, void *dst, uint32_t step, const float *impulse = nullptr)
+cudaError_t step_from(lb_handle *h, const void *src, void *dst, uint32_t step, float *impulse = nullptr)
 {
     const uint32_t saved = h->step;
     h->step = step;
@@ -790,10 +790,6 @@ lb_status lb_adjoint_kinetic_coupled(lb_handle *h, const lb_particles *parts, co
             return st;
         }
     }
-    // the last step applied its impulses: clear them now, so the recompute
-    // below can reuse the stencil records
-    if (e == cudaSuccess) e = clear_particle_forces(h);
-    h->facc_stale = 0;
     int cur = 0;
     if (e == cudaSuccess) e = cudaMemsetAsync(lam[0], 0, lam_bytes, h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(lam[1], 0, lam_bytes, h->stream);

@@ -12,10 +12,10 @@
 namespace lbi {
 
 template <int DT>
-cudaError_t launch_stream_collide_dt(const lb_handle *h, const void *src, void *dst, const float *facc, float *partials);
-extern template cudaError_t launch_stream_collide_dt<0>(const lb_handle *, const void *, void *, const float *, float *);
-extern template cudaError_t launch_stream_collide_dt<1>(const lb_handle *, const void *, void *, const float *, float *);
-extern template cudaError_t launch_stream_collide_dt<2>(const lb_handle *, const void *, void *, const float *, float *);
+cudaError_t launch_stream_collide_dt(const lb_handle *h, const void *src, void *dst, float *facc, float *partials);
+extern template cudaError_t launch_stream_collide_dt<0>(const lb_handle *, const void *, void *, float *, float *);
+extern template cudaError_t launch_stream_collide_dt<1>(const lb_handle *, const void *, void *, float *, float *);
+extern template cudaError_t launch_stream_collide_dt<2>(const lb_handle *, const void *, void *, float *, float *);
 template <int DT>
 cudaError_t launch_patch_dt(const lb_handle *h, const void *src, void *dst, float *facc, const int *records,
                             int n, int nsub, int span, unsigned int *claim, unsigned int tag);
@@ -92,6 +92,7 @@ StepArgs make_args(const lb_handle *h)
         a.frc[q] = (float)((1.0 + g) * iw * (q == 3 ? 0.5 : 1.0));
     }
     a.forced = h->force || p.body_force[0] != 0.0 || p.body_force[1] != 0.0 || p.body_force[2] != 0.0;
+    a.consume = 0;
     a.fx = (float)p.body_force[0];
     a.fy = (float)p.body_force[1];
     a.fz = (float)p.body_force[2];
@@ -247,13 +248,12 @@ lb_status step_once(lb_handle *h, float *partials)
         if (e != cudaSuccess) return cuda_fail("lb_step", e);
         h->launches += 2;
         h->facc_dirty = 0;
-        h->facc_stale = 0;  // the patch cleared every impulse node it applied
         drop_particle_records(h);
         h->cur = 1 - h->cur;
         h->step += 1;
         return LB_OK;
     }
-    const float *facc = h->facc_dirty ? h->facc : nullptr;
+    float *facc = h->facc_dirty ? h->facc : nullptr;
     timer_mark(h, 0, 0, h->stream);
     if (h->p.equilibrium) {
         e = launch_stream_collide_exp(h, src, dst, facc);
@@ -267,9 +267,9 @@ lb_status step_once(lb_handle *h, float *partials)
     timer_mark(h, 0, 1, h->stream);
     if (e != cudaSuccess) return cuda_fail("lb_step", e);
     h->launches += 1;
-    if (facc) {  // applied once; cleared by the next lb_couple_particles
+    if (facc) {  // applied once; the launch cleared what it read
         h->facc_dirty = 0;
-        h->facc_stale = 1;
+        drop_particle_records(h);
     }
     h->cur = 1 - h->cur;
     h->step += 1;

@@ -232,7 +232,7 @@ __device__ __forceinline__ void collide_exp2(const F2 m[19], F2 fx, F2 fy, F2 fz
 template <int DT, bool NOISE, bool WALLS, bool ODD>
 __global__ void __launch_bounds__(kLinBX) k_stream_collide_exp2(const typename lbd::Store<DT>::T *src,
                                                                 typename lbd::Store<DT>::T *dst, const float *ffield,
-                                                                const float *facc, const StepArgs a)
+                                                                float *facc, const StepArgs a)
 {
     PairAt at;
     const bool mine = locate_pair<WALLS>(a, at);
@@ -250,10 +250,11 @@ __global__ void __launch_bounds__(kLinBX) k_stream_collide_exp2(const typename l
 }
 
 template <int DT>
-cudaError_t launch_exp_dt(const lb_handle *h, const void *src, void *dst, const float *facc)
+cudaError_t launch_exp_dt(const lb_handle *h, const void *src, void *dst, float *facc)
 {
     using T = typename lbd::Store<DT>::T;
-    const StepArgs a = make_args(h);
+    StepArgs a = make_args(h);
+    a.consume = facc && facc == h->facc;
     const T *s = static_cast<const T *>(src);
     T *d = static_cast<T *>(dst);
     const bool noise = a.kT > 0.0f, walls = h->p.walls != 0;
@@ -270,7 +271,7 @@ cudaError_t launch_exp_dt(const lb_handle *h, const void *src, void *dst, const 
 
 // One stream-collide launch of a handle whose lb_params.equilibrium selects
 // the exponential form.
-cudaError_t launch_stream_collide_exp(const lb_handle *h, const void *src, void *dst, const float *facc)
+cudaError_t launch_stream_collide_exp(const lb_handle *h, const void *src, void *dst, float *facc)
 {
     switch (h->p.dtype) {
     case LB_F32: return launch_exp_dt<0>(h, src, dst, facc);

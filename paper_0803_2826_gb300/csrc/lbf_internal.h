@@ -43,9 +43,8 @@ struct lb_handle {
     unsigned int *d_err;  // device error word
     double *d_partials;   // reduction scratch [nblocks][LB_NSUMS]
     int red_blocks;
-    float *facc;          // particle impulse accumulator [3][pitch]
+    float *facc;          // particle impulse accumulator [3][pitch], zero outside pending impulses
     int facc_dirty;       // facc holds impulses the next lb_step applies
-    int facc_stale;       // facc holds applied impulses not yet cleared
     uint64_t launches;    // kernels launched through this handle
     lbi::Particles *parts;
     // an overlapped coupling (LB_COUPLE_OVERLAP) runs on `aux` while the next
@@ -97,10 +96,8 @@ lb_status cuda_fail(const char *what, cudaError_t e);
 StepArgs make_args(const lb_handle *h);
 int device_sm_count();
 
-// stream_collide.cu
-cudaError_t launch_stream_collide(const lb_handle *h, const void *src, void *dst, const float *facc);
 // exp_eq.cu: the update with the exponential equilibrium (lb_params.equilibrium = 1)
-cudaError_t launch_stream_collide_exp(const lb_handle *h, const void *src, void *dst, const float *facc);
+cudaError_t launch_stream_collide_exp(const lb_handle *h, const void *src, void *dst, float *facc);
 // moments.cu
 cudaError_t launch_init_equilibrium(const lb_handle *h, void *dst, const double *rho, const double *u);
 cudaError_t launch_set_populations(const lb_handle *h, void *dst, const double *n);
@@ -111,7 +108,6 @@ cudaError_t launch_moments(const lb_handle *h, const void *src, float *rho, floa
 lb_status couple_particles(lb_handle *h, const lb_particles *parts, const lb_couple_params *cp,
                           void *ready = nullptr, void *done = nullptr);
 lb_status interpolate(lb_handle *h, int kernel, int n, const double *pos, float *u_out);
-cudaError_t clear_particle_forces(lb_handle *h);
 void join_overlap(const lb_handle *h);  // order h->stream after a pending overlapped coupling
 // step_sums.cu
 size_t sc_block_count(const lb_handle *h);
@@ -120,7 +116,7 @@ cudaError_t reduce_step_sums(const lb_handle *h, const float *partials, size_t n
                              double *sums);
 void timer_mark(lb_handle *h, int which, int end, cudaStream_t s);  // record a timer event
 cudaError_t reset_particle_barrier(lb_handle *h);
-// Forget the stencil records of applied impulses that are already cleared.
+// Forget the stencil records of applied impulses (the launch that applied them cleared them).
 void drop_particle_records(lb_handle *h);
 bool adjoint_couple_ok(const lb_handle *h, const lb_particles *pp, const lb_couple_params *cp, const char *who);
 lb_status couple_adjoint(lb_handle *h, const void *state, const lb_particles *pp, const lb_couple_params *cp,

@@ -53,8 +53,6 @@ struct Particles {
     unsigned int *flags = nullptr;  // rebuild requests (kFlagWords words)
     uint32_t sub_counter = 0;
     int nlist_n = -1;            // particle count the list was built for
-    size_t rec_off = 0;          // offset of the live records in `records`
-    int last_nsub = 0;           // sub-steps of the previous call
     unsigned int *bar = nullptr; // grid barrier words of the persistent kernel
     // cell list of the Verlet-list build: particles binned into cells of edge
     // >= r_list, cells hashed into `nbuckets` linked-list buckets
@@ -62,8 +60,6 @@ struct Particles {
     int *next = nullptr;         // [cap] next particle in the same bucket
     int *bucket_of = nullptr;    // [cap] bucket of each particle (to empty it again)
     int nb_log2 = 0;             // log2 nbuckets
-    int rec_span = 2;            // nodes per axis the live records' stencils touch (2, or 4 for phi_3 / phi_4)
-    int rec_n = 0;               // particles per sub-step of the live records (-1: calls with different counts)
     // fluid velocities at the stencil nodes of each particle, kept over the
     // sub-steps of a call (the fluid is frozen during a call): [cap][64]
     // float4, valid while the particle's stencil origin and the call epoch
@@ -841,69 +837,6 @@ __global__ void __launch_bounds__(kPartThreads)
     }
 }
 
-// Zero the accumulator nodes around each recorded cell: [b, b + 1] per axis
-// for span 2 (phi_2), [b - 1, b + 2] for span 4 (covers phi_3 and phi_4).
-template <int SPAN>
-__global__ void k_clear_records(float *facc, const int *records, size_t n, StepArgs g)
-{
-    constexpr int lo = SPAN == 4 ? -1 : 0;
-    for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < n; q += (size_t)gridDim.x * blockDim.x) {
-        const int base = records[q];
-        const int x0 = base % g.nx;
-        const int y0 = (base / g.nx) % g.ny;
-        const int z0 = base / (g.nx * g.ny);
-#pragma unroll
-        for (int k = 0; k < SPAN * SPAN * SPAN; ++k) {
-            const int x = wrap_node(x0 + lo + k % SPAN, g.nx), y = wrap_node(y0 + lo + (k / SPAN) % SPAN, g.ny);
-            int z = z0 + lo + k / (SPAN * SPAN);
-            if (g.z0 > 0) z = z < 0 ? 0 : (z >= g.nz ? g.nz - 1 : z);
-            else z = wrap_node(z, g.nz);
-            const size_t s = ((size_t)z * g.ny + y) * g.nx + x;
-            facc[s] = 0.0f;
-            facc[g.pitch + s] = 0.0f;
-            facc[2 * g.pitch + s] = 0.0f;
-        }
-    }
-}
-
-// Particle p's share of the same for live records laid out [nsub][n]: lane q
-// of LANES walks the particle's cells, skips a cell equal to the one before
-// (a particle keeps its cell for many sub-steps) and zeroes nodes q, q +
-// LANES, ... of the block.
-template <int SPAN, int LANES>
-__device__ __forceinline__ void clear_particle_records(float *facc, const int *records, int n, int nsub, int p, int q,
-                                                       const StepArgs &g)
-{
-    constexpr int lo = SPAN == 4 ? -1 : 0, nk = SPAN * SPAN * SPAN;
-    int prev = -1;
-    for (int s = 0; s < nsub; ++s) {
-        const int base = records[(size_t)s * n + p];
-        if (base == prev) continue;
-        prev = base;
-        const int x0 = base % g.nx, y0 = (base / g.nx) % g.ny, z0 = base / (g.nx * g.ny);
-#pragma unroll
-        for (int k = q; k < nk; k += LANES) {
-            const int x = wrap_node(x0 + lo + k % SPAN, g.nx), y = wrap_node(y0 + lo + (k / SPAN) % SPAN, g.ny);
-            int z = z0 + lo + k / (SPAN * SPAN);
-            if (g.z0 > 0) z = z < 0 ? 0 : (z >= g.nz ? g.nz - 1 : z);
-            else z = wrap_node(z, g.nz);
-            const size_t i = ((size_t)z * g.ny + y) * g.nx + x;
-            facc[i] = 0.0f;
-            facc[g.pitch + i] = 0.0f;
-            facc[2 * g.pitch + i] = 0.0f;
-        }
-    }
-}
-
-template <int SPAN>
-__global__ void k_clear_records_by_particle(float *facc, const int *records, int n, int nsub, StepArgs g)
-{
-    const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    wait_for_previous();
-    if (t >= (size_t)n * 8) return;
-    clear_particle_records<SPAN, 8>(facc, records, n, nsub, (int)(t >> 3), (int)(t & 7), g);
-}
-
 // Interpolated velocity at caller positions with phi_KW; eight lanes per
 // position, lane q takes stencil nodes q, q + 8, ...
 template <int DT, int KW>
@@ -1037,17 +970,17 @@ lb_status ensure_buffers(lb_handle *h, int n, int nsub)
         }
     }
     const size_t need = (size_t)n * (size_t)nsub;
-    if (P->rec_cap < P->rec_off + P->n_records + need || P->rec_cap < 2 * need) {
-        // grow, keeping the records not yet cleared (moved to offset 0)
+    if (P->rec_cap < P->n_records + need) {
+        // grow, keeping the records of impulses no step has applied yet
         int *nr = nullptr;
-        const size_t cap = std::max((P->n_records + need) * 2, 2 * need);
+        const size_t cap = (P->n_records + need) * 2;
         cudaError_t e = cudaMalloc((void **)&nr, cap * sizeof(int));
         if (e != cudaSuccess) {
             set_error("lb_couple_particles: record allocation failed");
             return LB_ENOMEM;
         }
         if (P->n_records) {
-            e = cudaMemcpyAsync(nr, P->records + P->rec_off, P->n_records * sizeof(int), cudaMemcpyDeviceToDevice,
+            e = cudaMemcpyAsync(nr, P->records, P->n_records * sizeof(int), cudaMemcpyDeviceToDevice,
                                 h->stream);
             if (e != cudaSuccess) return cuda_fail("lb_couple_particles", e);
             e = cudaStreamSynchronize(h->stream);
@@ -1056,8 +989,7 @@ lb_status ensure_buffers(lb_handle *h, int n, int nsub)
         cudaFree(P->records);
         P->records = nr;
         P->rec_cap = cap;
-        P->rec_off = 0;
-    }
+        }
     return LB_OK;
 }
 
@@ -1093,9 +1025,7 @@ struct PersistArgs {
     float4 *ref;
     int *head, *next, *bucket_of;  // cell list; every bucket is empty again when the kernel ends
     float *facc;
-    int *records;            // this call: [nsub][n]
-    const int *stale;        // previous call's records to clear: [nstale_sub][n], or NULL
-    int nstale_sub;
+    int *records;            // this call: [nsub][n]; NULL in the serial order
     unsigned int *flags;     // [0] build before the next call, [1 + (s & 1)] rebuild epoch of sub-step s
     uint32_t epoch0;         // epoch of this call's first sub-step
     unsigned int *bar;
@@ -1241,7 +1171,7 @@ __device__ __forceinline__ void couple_persistent_run(const PersistArgs &a)
     const T *src = static_cast<const T *>(a.src);
     if (c.use_wca && blockIdx.x == 0 && threadIdx.x == 0) a.flags[0] = 0u;  // the pre-launch build has run
 
-    // phase 0: clear the previous call's impulses, first half drift
+    // phase 0: first half drift
     CPos me{}, refp{};
     float pm[3] = {0.f, 0.f, 0.f};
     float m = 1.f, G = 1.f, C1 = c.C1, C2 = c.C2, C3 = c.C3;
@@ -1256,25 +1186,6 @@ __device__ __forceinline__ void couple_persistent_run(const PersistArgs &a)
     bool bond_lo = false, bond_hi = false;
     if (active) {
         if (c.use_wca) unbin_particle(p, a.head, a.bucket_of);
-        int prev = -1;
-        for (int s = 0; s < a.nstale_sub; ++s) {
-            const int base = a.stale[(size_t)s * c.n + p];
-            if (base == prev) continue;  // same cell as the sub-step before
-            prev = base;
-            CPos bq{};
-            bq.c[0] = base % g.nx;
-            bq.c[1] = (base / g.nx) % g.ny;
-            bq.c[2] = base / (g.nx * g.ny);
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                int x, y, z;
-                (void)stencil_node(bq, q, g, x, y, z);
-                const size_t node = ((size_t)z * g.ny + y) * g.nx + x;
-                a.facc[node] = 0.0f;
-                a.facc[g.pitch + node] = 0.0f;
-                a.facc[2 * g.pitch + node] = 0.0f;
-            }
-        }
         m = a.mass ? a.mass[p] : c.mass0;
         G = a.gamma ? a.gamma[p] : c.gamma0;
         if (!c.uniform_coef) {
@@ -1399,7 +1310,7 @@ __device__ __forceinline__ void couple_persistent_run(const PersistArgs &a)
                 acc[q][1] = fmaf(-J[1], w[q], acc[q][1]);
                 acc[q][2] = fmaf(-J[2], w[q], acc[q][2]);
             }
-            a.records[(size_t)s * c.n + p] = (me.c[2] * g.ny + me.c[1]) * g.nx + me.c[0];
+            if (a.records) a.records[(size_t)s * c.n + p] = (me.c[2] * g.ny + me.c[1]) * g.nx + me.c[0];
 
             // second half drift of this sub-step, then the first of the next one
             const bool last = (s == a.nsub - 1);
@@ -1674,8 +1585,7 @@ __global__ void __launch_bounds__(kPThreads) k_couple_persistent_wide(PersistArg
     const T *src = static_cast<const T *>(a.src);
     if (c.use_wca && blockIdx.x == 0 && threadIdx.x == 0) a.flags[0] = 0u;  // the pre-launch build has run
 
-    // phase 0: first half drift, neighbours (the previous call's impulses were
-    // cleared before the launch)
+    // phase 0: first half drift, neighbours
     CPos me{}, refp{};
     float pm[3] = {0.f, 0.f, 0.f};
     float m = 1.f, G = 1.f, C1 = c.C1, C2 = c.C2, C3 = c.C3;
@@ -1814,7 +1724,7 @@ __global__ void __launch_bounds__(kPThreads) k_couple_persistent_wide(PersistArg
                 jy = fmaf(-J[1], w, jy);
                 jz = fmaf(-J[2], w, jz);
             }
-            a.records[(size_t)s * c.n + p] = stencil_record<KW>(me, g);
+            if (a.records) a.records[(size_t)s * c.n + p] = stencil_record<KW>(me, g);
 
             const bool last = (s == a.nsub - 1);
             bool ok = drift(me, pn, h, g, KW);
@@ -1881,9 +1791,8 @@ __global__ void __launch_bounds__(kPThreads) k_couple_persistent_wide(PersistArg
 // (neighbour positions from L2, forces, update, barrier), so what counts is
 // its length: with one thread a particle it had 27 / 64 read-modify-writes in
 // shared memory and 64 x 19 loads after each move in it, on one block of 128
-// particles per SM.  The impulses of the previous call are cleared in the
-// first phase.  768 monomers in 72 x 64 x 60, phi_4, ten sub-steps and the
-// step: 96 us against 275 us.
+// particles per SM.  768 monomers in 72 x 64 x 60, phi_4, ten sub-steps and
+// the step: 96 us against 275 us.
 // ---------------------------------------------------------------------------
 template <int DT, int KW, int LANES>
 __global__ void __launch_bounds__(kPThreads) k_couple_lanes(PersistArgs a)
@@ -1904,7 +1813,7 @@ __global__ void __launch_bounds__(kPThreads) k_couple_lanes(PersistArgs a)
     const T *src = static_cast<const T *>(a.src);
     if (c.use_wca && tid == 0) a.flags[0] = 0u;  // the pre-launch build has run
 
-    // phase 0: clear the previous call's impulses, first half drift, neighbours
+    // phase 0: first half drift, neighbours
     CPos me{}, refp{};
     float pm[3] = {0.f, 0.f, 0.f};
     float m = 1.f, G = 1.f, C1 = c.C1, C2 = c.C2, C3 = c.C3;
@@ -1916,7 +1825,6 @@ __global__ void __launch_bounds__(kPThreads) k_couple_lanes(PersistArgs a)
     bool bond_lo = false, bond_hi = false;
     if (active) {
         if (c.use_wca && lead) unbin_particle(p, a.head, a.bucket_of);
-        clear_particle_records<record_span<KW>(), LANES>(a.facc, a.stale, c.n, a.nstale_sub, p, q, g);
         m = a.mass ? a.mass[p] : c.mass0;
         G = a.gamma ? a.gamma[p] : c.gamma0;
         if (!c.uniform_coef) {
@@ -2084,7 +1992,7 @@ __global__ void __launch_bounds__(kPThreads) k_couple_lanes(PersistArgs a)
             for (int i = 0; i < kPer; ++i)
 #pragma unroll
                 for (int k = 0; k < 3; ++k) acc[i][k] = fmaf(-J[k], w[i], acc[i][k]);
-            if (lead) a.records[(size_t)s * c.n + p] = stencil_record<KW>(me, g);
+            if (lead && a.records) a.records[(size_t)s * c.n + p] = stencil_record<KW>(me, g);
 
             // second half drift of this sub-step, then the first of the next one
             const bool last = (s == a.nsub - 1);
@@ -2181,12 +2089,16 @@ __global__ void __launch_bounds__(kPartThreads) k_couple_free(FreeArgs a)
     const int tid = blockIdx.x * blockDim.x + threadIdx.x;
     const int p = tid / LANES, q = tid % LANES;
     wait_for_previous();
-    if (p >= c.n) return;  // whole groups leave together (LANES divides the block)
+    // whole groups leave together; with one lane a particle all stay, for the
+    // gathers of the warp
+    const bool active = p < c.n;
+    if (LANES > 1 && !active) return;
     const unsigned gmask = LANES == 1 ? 0xFFFFFFFFu : (0xFFu << (threadIdx.x & 24));
     const T *src = static_cast<const T *>(a.src);
 
-    const float m = a.mass ? a.mass[p] : c.mass0;
-    const float G = a.gamma ? a.gamma[p] : c.gamma0;
+    const int pi = active ? p : 0;  // (an idle lane follows particle 0 and stores nothing)
+    const float m = a.mass ? a.mass[pi] : c.mass0;
+    const float G = a.gamma ? a.gamma[pi] : c.gamma0;
     float C1 = c.C1, C2 = c.C2, C3 = c.C3;
     if (!c.uniform_coef) {
         const float x1 = G * c.dt / m;
@@ -2195,15 +2107,15 @@ __global__ void __launch_bounds__(kPartThreads) k_couple_free(FreeArgs a)
         C3 = sqrtf(m * g.kT * (-expm1f(-2.0f * x1)));
     }
     // first half drift in FP64 from the caller's position, then cell + offset
-    float pm[3] = {a.mom[3 * p], a.mom[3 * p + 1], a.mom[3 * p + 2]};
+    float pm[3] = {a.mom[3 * pi], a.mom[3 * pi + 1], a.mom[3 * pi + 2]};
     CPos me;
     {
-        double r[3] = {a.pos[3 * p], a.pos[3 * p + 1], a.pos[3 * p + 2]};
+        double r[3] = {a.pos[3 * pi], a.pos[3 * pi + 1], a.pos[3 * pi + 2]};
         const double hd = 0.5 * (double)c.dt / (double)m;
 #pragma unroll
         for (int k = 0; k < 3; ++k) r[k] += hd * (double)pm[k];
         confine_d(r, pm, g, KW);
-        if (!split(r, g, me) && q == 0) atomicOr(a.err, LB_DERR_PARTICLE_RANGE);
+        if (!split(r, g, me) && q == 0 && active) atomicOr(a.err, LB_DERR_PARTICLE_RANGE);
     }
 
     float uc[kPer][3], acc[kPer][3];
@@ -2215,7 +2127,8 @@ __global__ void __launch_bounds__(kPartThreads) k_couple_free(FreeArgs a)
     for (int s = 0; s < a.nsub; ++s) {
         Stencil<KW> st;
         make_stencil<KW>(me, st);
-        if (st.o[0] != org[0] || st.o[1] != org[1] || st.o[2] != org[2]) {
+        const bool moved = active && (st.o[0] != org[0] || st.o[1] != org[1] || st.o[2] != org[2]);
+        if (moved) {
             if (org[0] != INT_MIN) {  // hand in the impulses summed at the old origin
 #pragma unroll
                 for (int i = 0; i < kPer; ++i) {
@@ -2236,15 +2149,23 @@ __global__ void __launch_bounds__(kPartThreads) k_couple_free(FreeArgs a)
             org[0] = st.o[0];
             org[1] = st.o[1];
             org[2] = st.o[2];
+            if (LANES > 1) {
 #pragma unroll
-            for (int i = 0; i < kPer; ++i) {
-                const int qq = q + LANES * i;
-                if (kNodes % LANES == 0 || qq < kNodes) {
-                    int x, y, z;
-                    stencil_coords<KW>(org, qq, g, x, y, z);
-                    node_velocity<DT>(src, a.ffield, x, y, z, g, uc[i]);
+                for (int i = 0; i < kPer; ++i) {
+                    const int qq = q + LANES * i;
+                    if (kNodes % LANES == 0 || qq < kNodes) {
+                        int x, y, z;
+                        stencil_coords<KW>(org, qq, g, x, y, z);
+                        node_velocity<DT>(src, a.ffield, x, y, z, g, uc[i]);
+                    }
                 }
             }
+        }
+        if constexpr (KW == 2) {
+            // the warp gathers together, one node per lane: neighbouring nodes
+            // share sectors and many loads are in flight
+            if (s == 0) warp_gather_all<DT>(active, org, src, a.ffield, g, uc);
+            else if (__any_sync(kFullMask, moved)) warp_gather<DT>(moved, org, src, a.ffield, g, uc);
         }
         float w[kPer];
         float up[3] = {0.f, 0.f, 0.f};
@@ -2280,7 +2201,7 @@ __global__ void __launch_bounds__(kPartThreads) k_couple_free(FreeArgs a)
             acc[i][1] = fmaf(-J[1], w[i], acc[i][1]);
             acc[i][2] = fmaf(-J[2], w[i], acc[i][2]);
         }
-        if (q == 0 && a.records) a.records[(size_t)s * c.n + p] = stencil_record<KW>(me, g);
+        if (q == 0 && active && a.records) a.records[(size_t)s * c.n + p] = stencil_record<KW>(me, g);
         // second half drift of this sub-step, then the first of the next one
         ok = drift(me, pn, h, g, KW) && ok;
         if (s + 1 < a.nsub) ok = drift(me, pn, h, g, KW) && ok;
@@ -2288,7 +2209,7 @@ __global__ void __launch_bounds__(kPartThreads) k_couple_free(FreeArgs a)
         pm[1] = pn[1];
         pm[2] = pn[2];
     }
-    if (org[0] != INT_MIN) {
+    if (active && org[0] != INT_MIN) {
 #pragma unroll
         for (int i = 0; i < kPer; ++i) {
             const int qq = q + LANES * i;
@@ -2304,7 +2225,7 @@ __global__ void __launch_bounds__(kPartThreads) k_couple_free(FreeArgs a)
             }
         }
     }
-    if (q != 0) return;
+    if (q != 0 || !active) return;
     if (!ok) atomicOr(a.err, LB_DERR_PARTICLE_RANGE);
     a.pos[3 * p] = join1(me.c[0], me.f[0]);
     a.pos[3 * p + 1] = join1(me.c[1], me.f[1]);
@@ -2362,11 +2283,14 @@ CoupleArgs make_couple_args(const lb_handle *h, const lb_particles *pp, const lb
     return c;
 }
 
-void note_records(Particles *P, int n, size_t count)
+// Room for `count` stencil records of an overlapped call (the step's
+// re-update of impulse nodes walks them); none in the serial order.
+int *take_records(lb_handle *h, size_t count)
 {
-    if (P->n_records == 0) P->rec_n = n;
-    else if (P->rec_n != n) P->rec_n = -1;
-    P->n_records += count;
+    if (!h->aux || h->stream != h->aux) return nullptr;
+    int *r = h->parts->records + h->parts->n_records;
+    h->parts->n_records += count;
+    return r;
 }
 
 // The list build a persistent launch may need before it (both kernels return
@@ -2386,15 +2310,12 @@ cudaError_t build_list_before(lb_handle *h, const lb_particles *pp, const Couple
 }
 
 // One cooperative launch for the whole call: kernel `kfn` on `blocks` blocks of
-// kPThreads threads.  folds: the kernel clears the previous call's impulses
-// in its first phase when their records are those of one call with these
-// particles and this stencil; otherwise they are cleared before it.
+// kPThreads threads.
 cudaError_t launch_persistent(lb_handle *h, const lb_particles *pp, const lb_couple_params *cp, const CoupleArgs &c,
-                              const void *kfn, int blocks, size_t smem, bool folds)
+                              const void *kfn, int blocks, size_t smem)
 {
     Particles *P = h->parts;
     const int n = pp->n;
-    const int span = c.kw == 3 ? 3 : (c.kw == 4 ? 4 : 2);
     cudaError_t e = cudaSuccess;
     if (c.use_wca && P->nlist_n != n) {
         const unsigned int init[kFlagWords] = {0u, 0u, 1u, 0u, 0u};  // [2]: build before the launch
@@ -2402,14 +2323,6 @@ cudaError_t launch_persistent(lb_handle *h, const lb_particles *pp, const lb_cou
         if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
         if (e != cudaSuccess) return e;
         P->nlist_n = n;
-    }
-    const size_t need = (size_t)n * (size_t)cp->n_substeps, half = P->rec_cap / 2;
-    const bool fold_clear = folds && h->facc_stale && P->rec_span == span &&
-                            P->n_records == (size_t)n * (size_t)P->last_nsub && P->n_records <= half && need <= half;
-    if (h->facc_stale && !fold_clear) {
-        e = clear_particle_forces(h);
-        if (e != cudaSuccess) return e;
-        h->facc_stale = 0;
     }
     if (c.use_wca) {
         e = build_list_before(h, pp, c);
@@ -2433,12 +2346,7 @@ cudaError_t launch_persistent(lb_handle *h, const lb_particles *pp, const lb_cou
     a.next = P->next;
     a.bucket_of = P->bucket_of;
     a.facc = h->facc;
-    // the record buffer has two halves: the stale records (cleared in the
-    // kernel's first phase) stay in one, this call's go to the other
-    const size_t new_off = fold_clear ? (P->rec_off == 0 ? half : 0) : P->rec_off + P->n_records;
-    a.stale = fold_clear ? P->records + P->rec_off : nullptr;
-    a.nstale_sub = fold_clear ? P->last_nsub : 0;
-    a.records = P->records + new_off;
+    a.records = take_records(h, (size_t)n * (size_t)cp->n_substeps);
     a.flags = P->flags + 2;
     a.epoch0 = P->sub_counter + 1u;
     a.bar = P->bar;
@@ -2458,15 +2366,7 @@ cudaError_t launch_persistent(lb_handle *h, const lb_particles *pp, const lb_cou
     e = cudaLaunchKernelExC(&lc, kfn, args);
     if (e != cudaSuccess) return e;
     h->launches += 1;
-    if (fold_clear) {
-        P->rec_off = new_off;
-        P->n_records = 0;
-        h->facc_stale = 0;
-    }
-    note_records(P, n, need);
-    P->rec_span = std::max(P->rec_span, span);
     P->sub_counter += (uint32_t)cp->n_substeps;
-    P->last_nsub = cp->n_substeps;
     return cudaGetLastError();
 }
 
@@ -2516,11 +2416,6 @@ cudaError_t run_substeps(lb_handle *h, const lb_particles *pp, const lb_couple_p
 
     // free particles: one launch runs every sub-step, no grid barrier, any count
     if (!(cp->flags & LB_COUPLE_PER_SUBSTEP) && !need_nlist && c.chain_len <= 1) {
-        if (h->facc_stale) {
-            cudaError_t e = clear_particle_forces(h);
-            if (e != cudaSuccess) return e;
-            h->facc_stale = 0;
-        }
         FreeArgs fa;
         fa.c = c;
         fa.nsub = cp->n_substeps;
@@ -2531,7 +2426,7 @@ cudaError_t run_substeps(lb_handle *h, const lb_particles *pp, const lb_couple_p
         fa.mass = pp->mass;
         fa.gamma = pp->gamma;
         fa.facc = h->facc;
-        fa.records = P->records + P->rec_off + P->n_records;
+        fa.records = take_records(h, (size_t)n * (size_t)cp->n_substeps);
         fa.err = h->d_err;
         const int lanes = c.kw == 2 ? free_lanes<2>() : free_lanes<3>();
         const unsigned int fblocks = (unsigned int)(((size_t)n * lanes + kPartThreads - 1) / kPartThreads);
@@ -2541,11 +2436,8 @@ cudaError_t run_substeps(lb_handle *h, const lb_particles *pp, const lb_couple_p
                                               fblocks, kPartThreads, h->stream, fa);
         if (le != cudaSuccess) return le;
         h->launches += 1;
-        note_records(P, n, (size_t)n * (size_t)cp->n_substeps);
-        P->rec_span = std::max(P->rec_span, c.kw == 3 ? 3 : (c.kw == 4 ? 4 : 2));
         P->sub_counter += (uint32_t)cp->n_substeps;
-        P->last_nsub = cp->n_substeps;
-        return cudaGetLastError();
+            return cudaGetLastError();
     }
 
     // persistent path when every particle group can be resident at once
@@ -2560,22 +2452,17 @@ cudaError_t run_substeps(lb_handle *h, const lb_particles *pp, const lb_couple_p
             const bool warp = wblocks <= 2 * sms;
             const int lblocks = warp ? wblocks : eblocks;
             const void *lfn = lanes_kernel<DT>(c.kw, warp);
-            if (lblocks <= resident_blocks(lfn, 0)) return launch_persistent(h, pp, cp, c, lfn, lblocks, 0, true);
+            if (lblocks <= resident_blocks(lfn, 0)) return launch_persistent(h, pp, cp, c, lfn, lblocks, 0);
             const size_t smem = c.kw == 3 ? wide_smem_bytes<3>() : wide_smem_bytes<4>();
             const void *kfn = c.kw == 3 ? (const void *)k_couple_persistent_wide<DT, 3>
                                         : (const void *)k_couple_persistent_wide<DT, 4>;
-            if (pblocks <= resident_blocks(kfn, smem)) return launch_persistent(h, pp, cp, c, kfn, pblocks, smem, false);
+            if (pblocks <= resident_blocks(kfn, smem)) return launch_persistent(h, pp, cp, c, kfn, pblocks, smem);
         } else {
             const void *kfn = (const void *)k_couple_persistent<DT>;
-            if (pblocks <= resident_blocks(kfn, 0)) return launch_persistent(h, pp, cp, c, kfn, pblocks, 0, true);
+            if (pblocks <= resident_blocks(kfn, 0)) return launch_persistent(h, pp, cp, c, kfn, pblocks, 0);
         }
     }
 
-    if (h->facc_stale) {
-        cudaError_t e = clear_particle_forces(h);
-        if (e != cudaSuccess) return e;
-        h->facc_stale = 0;
-    }
     if (need_nlist && P->nlist_n != n) {
         cudaError_t e = cudaMemsetAsync(P->flags, 0xff, 2 * sizeof(unsigned int), h->stream);
         if (e != cudaSuccess) return e;
@@ -2614,7 +2501,7 @@ cudaError_t run_substeps(lb_handle *h, const lb_particles *pp, const lb_couple_p
         c.md_step = cp->md_step0 + (uint32_t)s;
         c.last = (s == cp->n_substeps - 1);
         c.slot = wr;
-        int *rec = P->records + P->rec_off + P->n_records;
+        int *rec = take_records(h, (size_t)n);
 #define LBI_SUBSTEP(KW)                                                                                          \
     k_substep<DT, KW><<<sblocks, kPartThreads, 0, h->stream>>>(                                                  \
         src, h->force, P->shadow[s & 1], P->shadow[(s + 1) & 1], pp->pos, pp->mom, pp->mass, pp->gamma, P->nlist, \
@@ -2624,8 +2511,6 @@ cudaError_t run_substeps(lb_handle *h, const lb_particles *pp, const lb_couple_p
         else if (c.kw == 4) LBI_SUBSTEP(4);
         else LBI_SUBSTEP(2);
 #undef LBI_SUBSTEP
-        note_records(P, n, (size_t)n);
-        P->rec_span = std::max(P->rec_span, c.kw == 3 ? 3 : (c.kw == 4 ? 4 : 2));
         P->sub_counter += 1;
         h->launches += 1;
     }
@@ -2867,8 +2752,6 @@ lb_status couple_particles(lb_handle *h, const lb_particles *pp, const lb_couple
     lb_status st = ensure_buffers(h, pp->n, cp->n_substeps);
     if (st != LB_OK) return st;
     cudaError_t e;
-    // impulses of the previous call that lb_step already applied are cleared
-    // inside run_substeps (by the persistent kernel, or by k_clear_records)
     timer_mark(h, 1, 0, h->stream);
     switch (h->p.dtype) {
     case LB_F32: e = run_substeps<0>(h, pp, cp); break;
@@ -2886,42 +2769,10 @@ lb_status couple_particles(lb_handle *h, const lb_particles *pp, const lb_couple
         h->overlap_pending = 1;
         h->patch_n = pp->n;
         h->patch_nsub = cp->n_substeps;
-        h->patch_rec = P->records + P->rec_off + P->n_records - (size_t)pp->n * (size_t)cp->n_substeps;
+        h->patch_rec = P->records + P->n_records - (size_t)pp->n * (size_t)cp->n_substeps;
         h->patch_span = stencil_width(cp->flags);  // the record span: 2, 3 (origin records) or 4
     }
     return LB_OK;
-}
-
-cudaError_t clear_particle_forces(lb_handle *h)
-{
-    Particles *P = h->parts;
-    if (!P || !h->facc) return cudaSuccess;
-    if (P->n_records) {
-        const StepArgs g = make_args(h);
-        const int *rec = P->records + P->rec_off;
-        if (P->rec_n > 0 && P->n_records % (size_t)P->rec_n == 0) {  // [nsub][n]: skip repeated cells
-            const int nsub = (int)(P->n_records / (size_t)P->rec_n);
-            const unsigned int blocks = (unsigned int)(((size_t)P->rec_n * 8 + 255) / 256);
-            const cudaError_t e = launch_chained(P->rec_span == 4   ? k_clear_records_by_particle<4>
-                                                 : P->rec_span == 3 ? k_clear_records_by_particle<3>
-                                                                    : k_clear_records_by_particle<2>,
-                                                 blocks, 256, h->stream, h->facc, rec, P->rec_n, nsub, g);
-            if (e != cudaSuccess) return e;
-        } else {
-            int blocks = (int)std::min<size_t>((P->n_records + 255) / 256, (size_t)8 * device_sm_count());
-            if (P->rec_span == 4)
-                k_clear_records<4><<<blocks, 256, 0, h->stream>>>(h->facc, rec, P->n_records, g);
-            else if (P->rec_span == 3)
-                k_clear_records<3><<<blocks, 256, 0, h->stream>>>(h->facc, rec, P->n_records, g);
-            else
-                k_clear_records<2><<<blocks, 256, 0, h->stream>>>(h->facc, rec, P->n_records, g);
-        }
-        h->launches += 1;
-        P->n_records = 0;
-        P->rec_off = 0;
-        P->rec_span = 2;
-    }
-    return cudaGetLastError();
 }
 
 template <int DT>
@@ -3013,30 +2864,22 @@ lb_status couple_adjoint(lb_handle *h, const void *state, const lb_particles *pp
 
 // A coupling call against the populations `state` whose impulses go to
 // facc_out ([3][pitch], zeroed here) instead of the handle's accumulator; the
-// particles are updated in place.  The handle's accumulator must hold no
-// uncleared impulses (its stencil records are reused here).
+// particles are updated in place.
 lb_status couple_on(lb_handle *h, const void *state, const lb_particles *pp, const lb_couple_params *cp,
                     float *facc_out)
 {
     void *saved_pop = h->pops[h->cur];
     float *saved_facc = h->facc;
-    const int saved_dirty = h->facc_dirty, saved_stale = h->facc_stale;
+    const int saved_dirty = h->facc_dirty;
     h->pops[h->cur] = const_cast<void *>(state);
     h->facc = facc_out;
-    h->facc_stale = 0;
     cudaError_t e = cudaMemsetAsync(facc_out, 0, 3 * h->pitch * sizeof(float), h->stream);
     lb_couple_params c2 = *cp;
     c2.flags &= ~LB_COUPLE_OVERLAP;
     lb_status st = e == cudaSuccess ? couple_particles(h, pp, &c2) : cuda_fail("lb_adjoint_kinetic_coupled", e);
-    if (h->parts) {  // these records index facc_out
-        h->parts->n_records = 0;
-        h->parts->rec_off = 0;
-        h->parts->rec_span = 2;
-    }
     h->pops[h->cur] = saved_pop;
     h->facc = saved_facc;
     h->facc_dirty = saved_dirty;
-    h->facc_stale = saved_stale;
     return st;
 }
 
@@ -3054,8 +2897,6 @@ void drop_particle_records(lb_handle *h)
     Particles *P = h->parts;
     if (!P) return;
     P->n_records = 0;
-    P->rec_off = 0;
-    P->rec_span = 2;
 }
 
 void destroy_particles(lb_handle *h)

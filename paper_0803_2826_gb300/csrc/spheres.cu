@@ -36,7 +36,7 @@
 
 namespace lbi {
 
-extern template cudaError_t launch_stream_collide_dt<0>(const lb_handle *, const void *, void *, const float *,
+extern template cudaError_t launch_stream_collide_dt<0>(const lb_handle *, const void *, void *, float *,
                                                         float *);
 
 namespace {

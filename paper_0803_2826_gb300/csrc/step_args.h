@@ -60,6 +60,9 @@ struct StepArgs {
     uint32_t step;
     lbd::RoundKeys rk;     // Philox round keys of (key0, key1)
     unsigned int *err;     // device error word (index checks of LB_DEBUG_BOUNDS builds)
+    // (last: one word before the noise constants shifts the pairs they are read
+    // in, and the 256^3 FP32 update goes from 72 registers and 365 us to 76 and 376)
+    int consume;           // the impulses read are applied for good: clear them
 };
 
 // Index checks of a library built with -DLB_DEBUG_BOUNDS: the element index i

@@ -460,12 +460,13 @@ struct Pair<2> {
 // Pull streaming of nodes x0, x0 + 1 of row (y, z) (link bounce-back at solid
 // z-planes) into packed pairs n (node x0 in the low halves, FP16 / BF16
 // unscaled), and their force densities f0, f1 (body force + caller's field +
-// library accumulator).
-template <int DT, bool FIELD, bool WALLS>
-__device__ __forceinline__ void load_pair(const typename lbd::Store<DT>::T *__restrict__ src,
-                                          const float *__restrict__ ffield, const float *__restrict__ facc,
-                                          const StepArgs &a, int x0, int y, int z, lbp::F2 n[19], float f0[3],
-                                          float f1[3])
+// library accumulator).  Impulses that are applied for good (a.consume) are
+// cleared here, by the thread that owns their nodes (take), so no other pass
+// has to find them again: few nodes carry any, and the test is three ORs and a
+// branch (512^3 FP16 with 1e5 particles: 50 us of clearing less a step).
+template <int DT, bool WALLS>
+__device__ __forceinline__ void pull_pair(const typename lbd::Store<DT>::T *__restrict__ src, const StepArgs &a, int x0,
+                                          int y, int z, uint32_t self, lbp::F2 n[19])
 {
     using S = lbd::Store<DT>;
     using PR = Pair<DT>;
@@ -483,7 +484,6 @@ __device__ __forceinline__ void load_pair(const typename lbd::Store<DT>::T *__re
         zp = (z == nz - 1) ? 0 : z + 1;
     }
     const uint32_t P = (uint32_t)a.pitch;
-    const uint32_t self = (uint32_t)((z * ny + y) * nx + x0);
     const size_t lim = 19 * (size_t)P;  // elements of a population buffer (index checks)
 #pragma unroll
     for (int i = 0; i < 19; ++i) {
@@ -515,7 +515,20 @@ __device__ __forceinline__ void load_pair(const typename lbd::Store<DT>::T *__re
         }
         n[i] = DT == 0 ? lbp::f2(v0, v1) : lbp::f2(v0, v1) * lbp::f2s(a.inv_scale);
     }
+}
 
+template <int DT, bool FIELD, bool WALLS>
+__device__ __forceinline__ void load_pair(const typename lbd::Store<DT>::T *__restrict__ src,
+                                          const float *__restrict__ ffield, float *facc,
+                                          const StepArgs &a, int x0, int y, int z, lbp::F2 n[19], float f0[3],
+                                          float f1[3], bool take = true)
+{
+    const uint32_t P = (uint32_t)a.pitch;
+    const uint32_t self = (uint32_t)((z * a.ny + y) * a.nx + x0);
+    // only the planes next to a wall look at their links (z is the same for
+    // a whole row, so a warp rarely takes both ways)
+    if (WALLS && (z == a.z0 || z == a.z1 - 1)) pull_pair<DT, true>(src, a, x0, y, z, self, n);
+    else pull_pair<DT, false>(src, a, x0, y, z, self, n);
     f0[0] = f1[0] = a.fx;
     f0[1] = f1[1] = a.fy;
     f0[2] = f1[2] = a.fz;
@@ -528,12 +541,18 @@ __device__ __forceinline__ void load_pair(const typename lbd::Store<DT>::T *__re
             }
         }
         if (facc) {  // library accumulator, component stride = plane pitch
+            unsigned int bits = 0u;
 #pragma unroll
             for (int d = 0; d < 3; ++d) {
                 float u, v;
                 Pair<0>::load(facc + d * (size_t)P + self, 1.0f, u, v);
                 f0[d] += u;
                 f1[d] += v;
+                bits |= __float_as_uint(u) | __float_as_uint(v);
+            }
+            if (bits && a.consume && take) {
+#pragma unroll
+                for (int d = 0; d < 3; ++d) Pair<0>::store(facc + d * (size_t)P + self, 0.0f, 0.0f, 1.0f);
             }
         }
     }
@@ -557,14 +576,14 @@ __device__ __forceinline__ void store_pair(typename lbd::Store<DT>::T *__restric
 template <int DT, bool NOISE, bool FIELD, bool WALLS, bool SUMS = false>
 __device__ __forceinline__ void update_pair(const typename lbd::Store<DT>::T *__restrict__ src,
                                             typename lbd::Store<DT>::T *__restrict__ dst,
-                                            const float *__restrict__ ffield, const float *__restrict__ facc,
+                                            const float *__restrict__ ffield, float *facc,
                                             const StepArgs &a, int x0, int y, int z, bool valid = true,
                                             float (*part)[38] = nullptr)
 {
     const uint32_t self = (uint32_t)((z * a.ny + y) * a.nx + x0);
     lbp::F2 n[19];
     float f0[3], f1[3];
-    load_pair<DT, FIELD, WALLS>(src, ffield, facc, a, x0, y, z, n, f0, f1);
+    load_pair<DT, FIELD, WALLS>(src, ffield, facc, a, x0, y, z, n, f0, f1, valid);
     // both nodes' moments, collision, noise and back transform in packed
     // FP32 (f32x2.cuh), node x0 in the low halves
     lbp::F2 m[19], out[19];
@@ -590,11 +609,10 @@ __device__ __forceinline__ size_t block_linear()
 }
 
 template <int DT, bool NOISE, bool FIELD, bool WALLS, bool SUMS>
-__global__ void __launch_bounds__(kBX) k_stream_collide2(const typename lbd::Store<DT>::T *__restrict__ src,
-                                                         typename lbd::Store<DT>::T *__restrict__ dst,
-                                                         const float *__restrict__ ffield,
-                                                         const float *__restrict__ facc, const StepArgs a,
-                                                         float *partials)
+__device__ __forceinline__ void rows_update(const typename lbd::Store<DT>::T *__restrict__ src,
+                                            typename lbd::Store<DT>::T *__restrict__ dst,
+                                            const float *__restrict__ ffield, float *facc, const StepArgs &a,
+                                            float *partials)
 {
     const int x0 = 2 * (blockIdx.x * kBX + threadIdx.x);
     wait_for_previous();
@@ -608,6 +626,34 @@ __global__ void __launch_bounds__(kBX) k_stream_collide2(const typename lbd::Sto
         if (x0 >= a.nx) return;
         update_pair<DT, NOISE, FIELD, WALLS>(src, dst, ffield, facc, a, x0, blockIdx.y, blockIdx.z + a.z0);
     }
+}
+
+template <int DT, bool NOISE, bool FIELD, bool WALLS, bool SUMS>
+__global__ void __launch_bounds__(kBX)
+    k_stream_collide2(const typename lbd::Store<DT>::T *__restrict__ src, typename lbd::Store<DT>::T *__restrict__ dst,
+                      const float *__restrict__ ffield, float *facc, const StepArgs a, float *partials)
+{
+    rows_update<DT, NOISE, FIELD, WALLS, SUMS>(src, dst, ffield, facc, a, partials);
+}
+
+// The same where a force field is read: room for seven blocks of 128 threads
+// per SM (FP32) or eight (FP16 / BF16).  The update wants warps more than
+// registers, and these kernels carry a few more registers than six blocks
+// leave room for (256^3 FP32 between walls with a field 412 us against 443 us a
+// step, 512 x 512 x 256 FP16 1576 us against 1612 us, for 24 to 88 bytes of
+// spills).  Without a field the compiler's own choice, 72 registers, is the
+// best (256^3 FP32 365 us; 371 us with room for six or seven blocks, 383 us for
+// eight).
+template <int DT>
+constexpr int field_blocks() { return DT == 0 ? 7 : 8; }
+
+template <int DT, bool NOISE, bool WALLS>
+__global__ void __launch_bounds__(kBX, field_blocks<DT>())
+    k_stream_collide2_field(const typename lbd::Store<DT>::T *__restrict__ src,
+                            typename lbd::Store<DT>::T *__restrict__ dst, const float *__restrict__ ffield, float *facc,
+                            const StepArgs a, float *partials)
+{
+    rows_update<DT, NOISE, true, WALLS, false>(src, dst, ffield, facc, a, partials);
 }
 
 // Two consecutive nodes s, s + 1 (s even) per thread over the fluid's linear
@@ -721,22 +767,31 @@ __device__ __forceinline__ void second_node(const Geo &a, const PairAt &at, int 
 
 template <int DT, bool FIELD, bool WALLS>
 __device__ __forceinline__ void load_pair_any(const typename lbd::Store<DT>::T *__restrict__ src,
-                                              const float *__restrict__ ffield, const float *__restrict__ facc,
+                                              const float *__restrict__ ffield, float *facc,
                                               const StepArgs &a, const PairAt &at, lbp::F2 n[19], float f0[3],
-                                              float f1[3])
+                                              float f1[3], bool take = true)
 {
     int xb, yb, zb;
     second_node(a, at, xb, yb, zb);
     const PullAt pa = pull_at<WALLS>(a, at.x, at.y, at.z), pb = pull_at<WALLS>(a, xb, yb, zb);
+    if (WALLS && (pa.lo || pa.hi || pb.lo || pb.hi)) {  // next to a wall (load_pair)
 #pragma unroll
-    for (int i = 0; i < 19; ++i) {
-        const lbp::F2 v = lbp::f2(pull_one<DT, WALLS>(src, a, pa, i), pull_one<DT, WALLS>(src, a, pb, i));
-        n[i] = DT == 0 ? v : v * lbp::f2s(a.inv_scale);
+        for (int i = 0; i < 19; ++i)
+            n[i] = lbp::f2(pull_one<DT, true>(src, a, pa, i), pull_one<DT, true>(src, a, pb, i));
+    } else {
+#pragma unroll
+        for (int i = 0; i < 19; ++i)
+            n[i] = lbp::f2(pull_one<DT, false>(src, a, pa, i), pull_one<DT, false>(src, a, pb, i));
+    }
+    if (DT != 0) {
+#pragma unroll
+        for (int i = 0; i < 19; ++i) n[i] = n[i] * lbp::f2s(a.inv_scale);
     }
     f0[0] = f1[0] = a.fx;
     f0[1] = f1[1] = a.fy;
     f0[2] = f1[2] = a.fz;
     if (FIELD) {
+        unsigned int bits = 0u;
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
             if (ffield) {  // caller's field, component stride N
@@ -744,9 +799,15 @@ __device__ __forceinline__ void load_pair_any(const typename lbd::Store<DT>::T *
                 f1[d] += ld_f32(ffield + d * a.nn + pb.self);
             }
             if (facc) {  // library accumulator, component stride = plane pitch
-                f0[d] += ld_f32(facc + d * a.pitch + pa.self);
-                f1[d] += ld_f32(facc + d * a.pitch + pb.self);
+                const float u = ld_f32(facc + d * a.pitch + pa.self), v = ld_f32(facc + d * a.pitch + pb.self);
+                f0[d] += u;
+                f1[d] += v;
+                bits |= __float_as_uint(u) | __float_as_uint(v);
             }
+        }
+        if (bits && a.consume && take) {
+#pragma unroll
+            for (int d = 0; d < 3; ++d) facc[d * a.pitch + pa.self] = facc[d * a.pitch + pb.self] = 0.0f;
         }
     }
 }
@@ -780,7 +841,7 @@ __device__ __forceinline__ void store_pair_any(typename lbd::Store<DT>::T *__res
 
 template <int DT, bool FIELD, bool WALLS, bool ODD>
 __device__ __forceinline__ void load_linear(const typename lbd::Store<DT>::T *__restrict__ src,
-                                            const float *__restrict__ ffield, const float *__restrict__ facc,
+                                            const float *__restrict__ ffield, float *facc,
                                             const StepArgs &a, const PairAt &at, lbp::F2 n[19], float f0[3],
                                             float f1[3])
 {
@@ -791,10 +852,9 @@ __device__ __forceinline__ void load_linear(const typename lbd::Store<DT>::T *__
 }
 
 template <int DT, bool NOISE, bool FIELD, bool WALLS, bool ODD>
-__global__ void __launch_bounds__(kLinBX) k_stream_collide_linear(const typename lbd::Store<DT>::T *__restrict__ src,
-                                                               typename lbd::Store<DT>::T *__restrict__ dst,
-                                                               const float *__restrict__ ffield,
-                                                               const float *__restrict__ facc, const StepArgs a)
+__device__ __forceinline__ void linear_update(const typename lbd::Store<DT>::T *__restrict__ src,
+                                              typename lbd::Store<DT>::T *__restrict__ dst,
+                                              const float *__restrict__ ffield, float *facc, const StepArgs &a)
 {
     PairAt at;
     const bool mine = locate_pair<WALLS>(a, at);
@@ -812,6 +872,41 @@ __global__ void __launch_bounds__(kLinBX) k_stream_collide_linear(const typename
         store_pair<DT>(dst, a, at.s, out);
 }
 
+template <int DT, bool NOISE, bool FIELD, bool WALLS, bool ODD>
+__global__ void __launch_bounds__(kLinBX)
+    k_stream_collide_linear(const typename lbd::Store<DT>::T *__restrict__ src,
+                            typename lbd::Store<DT>::T *__restrict__ dst, const float *__restrict__ ffield, float *facc,
+                            const StepArgs a)
+{
+    linear_update<DT, NOISE, FIELD, WALLS, ODD>(src, dst, ffield, facc, a);
+}
+
+// With a force field (k_stream_collide2_field); rows of odd length spill too
+// much for that and leave the count open (257 x 131 x 129 FP32 between walls
+// with a field 119 us a step, 133 us with room for seven blocks).
+template <int DT, bool NOISE, bool WALLS, bool ODD>
+__global__ void __launch_bounds__(kLinBX, ODD ? 0 : field_blocks<DT>() * kBX / kLinBX)
+    k_stream_collide_linear_field(const typename lbd::Store<DT>::T *__restrict__ src,
+                                  typename lbd::Store<DT>::T *__restrict__ dst, const float *__restrict__ ffield,
+                                  float *facc, const StepArgs a)
+{
+    linear_update<DT, NOISE, true, WALLS, ODD>(src, dst, ffield, facc, a);
+}
+
+// The step's kernel of either mapping.
+template <int DT, bool NOISE, bool FIELD, bool WALLS>
+auto rows_kernel()
+{
+    if constexpr (FIELD) return k_stream_collide2_field<DT, NOISE, WALLS>;
+    else return k_stream_collide2<DT, NOISE, false, WALLS, false>;
+}
+template <int DT, bool NOISE, bool FIELD, bool WALLS, bool ODD>
+auto linear_kernel()
+{
+    if constexpr (FIELD) return k_stream_collide_linear_field<DT, NOISE, WALLS, ODD>;
+    else return k_stream_collide_linear<DT, NOISE, false, WALLS, ODD>;
+}
+
 // The step with moment sums on boxes whose pairs cannot move as one access
 // (rows of odd length, or more elements than 32-bit indices reach): rows mapped to blocks
 // as in k_stream_collide2, the pair's addresses and stores one node at a time,
@@ -821,8 +916,7 @@ template <int DT, bool NOISE, bool FIELD, bool WALLS>
 __global__ void __launch_bounds__(kBX) k_stream_collide_sums_any(const typename lbd::Store<DT>::T *__restrict__ src,
                                                                  typename lbd::Store<DT>::T *__restrict__ dst,
                                                                  const float *__restrict__ ffield,
-                                                                 const float *__restrict__ facc, const StepArgs a,
-                                                                 float *partials)
+                                                                 float *facc, const StepArgs a, float *partials)
 {
     __shared__ float part[kBX / 32][38];
     const int x0 = 2 * (blockIdx.x * kBX + threadIdx.x);
@@ -837,7 +931,7 @@ __global__ void __launch_bounds__(kBX) k_stream_collide_sums_any(const typename 
     wait_for_previous();
     lbp::F2 n[19], m[19], out[19];
     float f0[3], f1[3];
-    load_pair_any<DT, FIELD, WALLS>(src, ffield, facc, a, at, n, f0, f1);
+    load_pair_any<DT, FIELD, WALLS>(src, ffield, facc, a, at, n, f0, f1, mine);
     lbp::forward2(n, m);
     float m0[19], m1[19];
 #pragma unroll
@@ -875,12 +969,13 @@ inline dim3 sc_grid(const lb_handle *h)
 // partials != NULL: the launch also writes per-block moment sums
 // (partials[block][38], block = blockIdx.x + gridDim.x (blockIdx.y + gridDim.y blockIdx.z)).
 template <int DT>
-cudaError_t launch_stream_collide_dt(const lb_handle *h, const void *src, void *dst, const float *facc,
+cudaError_t launch_stream_collide_dt(const lb_handle *h, const void *src, void *dst, float *facc,
                                      float *partials)
 {
     using T = typename lbd::Store<DT>::T;
     StepArgs a = make_args(h);
     a.forced |= facc != nullptr;
+    a.consume = facc && facc == h->facc;  // (the reverse pass keeps its impulse buffers)
     const dim3 grid = sc_grid(h);
     const dim3 block(kBX);
     const bool noise = a.kT > 0.0f;
@@ -898,11 +993,11 @@ cudaError_t launch_stream_collide_dt(const lb_handle *h, const void *src, void *
                                          h->force, facc, a, partials)                                             \
                         : launch_chained(k_stream_collide_sums_any<DT, NZ, FL, WL>, grid, block, h->stream, s, d,   \
                                          h->force, facc, a, partials))                                            \
-     : rows   ? launch_chained(k_stream_collide2<DT, NZ, FL, WL, false>, grid, block, h->stream, s, d, h->force,    \
+     : rows   ? launch_chained(rows_kernel<DT, NZ, FL, WL>(), grid, block, h->stream, s, d, h->force,    \
                                facc, a, nullptr)                                                                  \
-     : odd    ? launch_chained(k_stream_collide_linear<DT, NZ, FL, WL, true>, linear, dim3(kLinBX), h->stream, s, d, \
+     : odd    ? launch_chained(linear_kernel<DT, NZ, FL, WL, true>(), linear, dim3(kLinBX), h->stream, s, d, \
                                h->force, facc, a)                                                                 \
-              : launch_chained(k_stream_collide_linear<DT, NZ, FL, WL, false>, linear, dim3(kLinBX), h->stream, s,  \
+              : launch_chained(linear_kernel<DT, NZ, FL, WL, false>(), linear, dim3(kLinBX), h->stream, s,  \
                                d, h->force, facc, a))
     if (noise) {
         if (field) return walls ? LBI_SC(true, true, true) : LBI_SC(true, true, false);
