@@ -4,22 +4,21 @@
 // EOMUsol and the consistency equation for the velocity U~).
 //
 // One lb_step_spheres call, all on the handle's stream:
-//   k_sph_half     one thread per sphere: R(t+h/2) = R + U/2, accumulators zeroed
-//   k_sph_map      per sphere, the nodes of a box around it: the solid map
-//                  follows R(t+h/2); a covered fluid node gives its momentum
-//                  to the sphere, an uncovered node starts from n^eq(rho0, U)
-//                  and the sphere loses rho0 U
+//   k_sph_map      per sphere, the nodes of a box around it: R(t+h/2) = R + U/2
+//                  and the solid map follows it; a covered fluid node gives
+//                  its momentum to the sphere, an uncovered node starts from
+//                  n^eq(rho0, U) and the sphere loses rho0 U
 //   k_sph_links    per sphere, the fluid nodes of its box: F0 = sum 2 n*_b c_b
 //                  and zeta = 6 rho0 sum a_b c_b c_b^T over the boundary links
 //   k_sph_update   one thread per sphere: U(t+h) and U~ (zeta's eigenbasis
-//                  by FP32 Jacobi rotations; U kept in FP64)
+//                  by FP32 Jacobi rotations; U kept in FP64), and
+//                  R(t+h) = R(t+h/2) + U(t+h)/2
 //   the plain stream-collide launch over every node (exact for fluid nodes
 //                  without a solid neighbour), then
 //   k_sph_near_nodes  the near fluid nodes (listed by k_sph_links) again: pull
 //                  streaming in which a population whose source node is solid
 //                  returns as n*_-i(r) + 6 a_i rho0 U~.c_i, then the same
 //                  collision
-//   k_sph_finish   one thread per sphere: R(t+h) = R(t+h/2) + U(t+h)/2
 // The solid map holds the sphere index of a solid node, -2 for a fluid node
 // with a solid neighbour (the only nodes whose pull needs the map) and -1
 // for the other fluid nodes; k_sph_links sets the marks within a + 2.5 of
@@ -42,6 +41,7 @@ extern template cudaError_t launch_stream_collide_dt<0>(const lb_handle *, const
 namespace {
 
 constexpr int kSphThreads = 128;
+constexpr int kSphUpdThreads = 32;  // one sphere a thread in a long serial chain: spread over the SMs
 // per sphere: F0 (3), covering momentum (3), friction TT xx yy zz xy yz zx (6),
 // torque T0 (3), covering angular momentum (3), friction TR row-major (9),
 // friction RR xx yy zz xy yz zx (6)
@@ -133,23 +133,6 @@ __global__ void k_sph_place(int *owner, const double *pos, double a, int B, int 
     if (atomicCAS(owner + s, -1, p) != -1) atomicOr(err, LB_DERR_SPHERE);
 }
 
-__global__ void k_sph_half(const double *pos, const double *vel, const double *mass, double mass0, int n, double *rh,
-                           float *acc, unsigned int *count, StepArgs g, unsigned int *err)
-{
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    wait_for_previous();
-    if (p == 0) *count = 0u;  // the near-node list of this step
-    if (p >= n) return;
-    const double m = mass ? mass[p] : mass0;
-    const int L[3] = {g.nx, g.ny, g.nz};
-    for (int d = 0; d < 3; ++d) {
-        const double u = vel[3 * p + d];
-        if (!(fabs(u) <= 1.0)) atomicOr(err, LB_DERR_SPHERE);  // also catches NaN
-        rh[3 * p + d] = m > 0.0 ? wrap_pos(__dadd_rn(pos[3 * p + d], 0.5 * u), L[d]) : pos[3 * p + d];
-    }
-    for (int q = 0; q < kAcc; ++q) acc[kAcc * p + q] = 0.0f;
-}
-
 __device__ __forceinline__ void cross3f(const float a[3], const float b[3], float out[3])
 {
     out[0] = a[1] * b[2] - a[2] * b[1];
@@ -157,17 +140,34 @@ __device__ __forceinline__ void cross3f(const float a[3], const float b[3], floa
     out[2] = a[0] * b[1] - a[1] * b[0];
 }
 
-// The solid map follows the half-step centres (uncovered nodes get the
+// R(t+h/2) = R + U/2, and the solid map follows it (uncovered nodes get the
 // equilibrium of the surface velocity U + Omega x rho at time t, which this
-// kernel reads before any update).  om: angular velocities, or NULL.
-__global__ void k_sph_map(int *owner, float *pops, const double *rh, const double *vel, const double *om, double a,
-                          int B, int n, StepArgs g, float *acc, unsigned int *err)
+// kernel reads before any update).  om: angular velocities, or NULL.  Every
+// block of a sphere forms the centre itself; the first one stores it for the
+// kernels that follow.  The step's near-node list starts empty here (the
+// accumulators were emptied by the kernel that consumed them).
+__global__ void k_sph_map(int *owner, float *pops, const double *pos, const double *vel, const double *mass,
+                          double mass0, double *rh, const double *om, double a, int B, int n, StepArgs g, float *acc,
+                          unsigned int *count, unsigned int *err)
 {
     __shared__ Box b;
     const int p = blockIdx.y;
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     wait_for_previous();
-    const double c[3] = {rh[3 * p], rh[3 * p + 1], rh[3 * p + 2]};
+    if (p == 0 && k == 0) *count = 0u;
+    __shared__ double c[3];
+    if (threadIdx.x < 3) {  // one component a thread: FP64 is slow here
+        const int d = threadIdx.x;
+        const double m = mass ? mass[p] : mass0, u = vel[3 * p + d];
+        const int L = d == 0 ? g.nx : (d == 1 ? g.ny : g.nz);
+        const double v = m > 0.0 ? wrap_pos(__dadd_rn(pos[3 * p + d], 0.5 * u), L) : pos[3 * p + d];
+        c[d] = v;
+        if (blockIdx.x == 0) {
+            rh[3 * p + d] = v;
+            if (!(fabs(u) <= 1.0)) atomicOr(err, LB_DERR_SPHERE);  // also catches NaN
+        }
+    }
+    __syncthreads();
     box_setup(b, c, a);
     if (p >= n || k >= B * B * B) return;
     int x, y, z, o[3];
@@ -255,14 +255,25 @@ __global__ void __launch_bounds__(kSphThreads) k_sph_links(int *owner, const flo
             // only costs the exact recomputation of a far node)
         } else if (own < 0) {
             bool near = false;
+            // all the map entries, then all the populations: two memory round
+            // trips instead of one per link
+            int ow[19];
+            float pv[19];
 #pragma unroll
             for (int i = 1; i < 19; ++i) {
                 const int tx = wrap_i(x + lbd::cx(i), g.nx), ty = wrap_i(y + lbd::cy(i), g.ny),
                           tz = wrap_i(z + lbd::cz(i), g.nz);
-                const int ow = owner[((size_t)tz * g.ny + ty) * g.nx + tx];
-                near = near || ow >= 0;
-                if (ow != p) continue;
-                const float nb = 2.0f * pops[(size_t)i * g.pitch + s];
+                ow[i] = owner[((size_t)tz * g.ny + ty) * g.nx + tx];
+            }
+#pragma unroll
+            for (int i = 1; i < 19; ++i) {
+                near = near || ow[i] >= 0;
+                pv[i] = ow[i] == p ? pops[(size_t)i * g.pitch + s] : 0.0f;
+            }
+#pragma unroll
+            for (int i = 1; i < 19; ++i) {
+                if (ow[i] != p) continue;
+                const float nb = 2.0f * pv[i];
                 const float cb[3] = {(float)lbd::cx(i), (float)lbd::cy(i), (float)lbd::cz(i)};
                 const float za = 6.0f * g.rho0 * lbd::weight(i);
                 v[0] += nb * cb[0];
@@ -432,14 +443,21 @@ __device__ void velocity_update(const float Z[N][N], const float sq[N], double V
 
 // U(t+h), U~ (and with om Omega(t+h), Omega~) of each sphere; the moment of
 // inertia is 2/5 m a^2.
-__global__ void k_sph_update(double *vel, double *om, const double *mass, double mass0, double a, const double *force,
-                             int n, const float *acc, float4 *ut, float4 *uw)
+// Also R(t+h) = R(t+h/2) + U(t+h)/2, and the accumulators emptied for the next
+// step.
+__global__ void k_sph_update(double *pos, double *vel, double *om, const double *mass, double mass0, double a,
+                             const double *force, const double *rh, int n, float *acc, float4 *ut, float4 *uw, StepArgs g)
 {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     wait_for_previous();
     if (p >= n) return;
     const double m = mass ? mass[p] : mass0;
-    const float *ac = acc + kAcc * p;
+    float ac[kAcc];
+    for (int q = 0; q < kAcc; ++q) {
+        ac[q] = acc[kAcc * p + q];
+        acc[kAcc * p + q] = 0.0f;
+    }
+    const int L[3] = {g.nx, g.ny, g.nz};
     if (!(m > 0.0)) {  // held fixed: the surface moves with U (+ Omega x rho)
         ut[p] = make_float4((float)vel[3 * p], (float)vel[3 * p + 1], (float)vel[3 * p + 2], 0.0f);
         uw[p] = om ? make_float4((float)om[3 * p], (float)om[3 * p + 1], (float)om[3 * p + 2], 0.0f)
@@ -471,6 +489,7 @@ __global__ void k_sph_update(double *vel, double *om, const double *mass, double
         for (int d = 0; d < 3; ++d) {
             vel[3 * p + d] = V[d];
             om[3 * p + d] = V[3 + d];
+            pos[3 * p + d] = wrap_pos(__dadd_rn(rh[3 * p + d], 0.5 * V[d]), L[d]);
         }
         ut[p] = make_float4(Vt[0], Vt[1], Vt[2], 0.0f);
         uw[p] = make_float4(Vt[3], Vt[4], Vt[5], 0.0f);
@@ -485,21 +504,12 @@ __global__ void k_sph_update(double *vel, double *om, const double *mass, double
     }
     const float Z[3][3] = {{ac[6], ac[9], ac[11]}, {ac[9], ac[7], ac[10]}, {ac[11], ac[10], ac[8]}};
     velocity_update<3>(Z, sq, V, F, Vt);
-    for (int d = 0; d < 3; ++d) vel[3 * p + d] = V[d];
+    for (int d = 0; d < 3; ++d) {
+        vel[3 * p + d] = V[d];
+        pos[3 * p + d] = wrap_pos(__dadd_rn(rh[3 * p + d], 0.5 * V[d]), L[d]);
+    }
     ut[p] = make_float4(Vt[0], Vt[1], Vt[2], 0.0f);
     uw[p] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-}
-
-__global__ void k_sph_finish(double *pos, const double *vel, const double *mass, double mass0, const double *rh,
-                             int n, StepArgs g)
-{
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    wait_for_previous();
-    if (p >= n) return;
-    const double m = mass ? mass[p] : mass0;
-    if (!(m > 0.0)) return;
-    const int L[3] = {g.nx, g.ny, g.nz};
-    for (int d = 0; d < 3; ++d) pos[3 * p + d] = wrap_pos(__dadd_rn(rh[3 * p + d], 0.5 * vel[3 * p + d]), L[d]);
 }
 
 // Minimum image of d along an axis of length L (|d| < L).
@@ -509,60 +519,59 @@ __device__ __forceinline__ float image_f(float d, int L)
     return d > h ? d - (float)L : (d < -h ? d + (float)L : d);
 }
 
-// Stream and collide fluid node (x, y, z) whose map entry is own (< 0): a
+// Stream and collide fluid node (x, y, z) next to a sphere: a
 // population whose source node is solid (sphere o) returns from the node
 // itself with the moving-wall term, n_i(r) = n*_-i(r) + 2 a_i rho0
 // u_b.c_i / c_s^2 with u_b = U~_o + Omega~_o x (r_b - R_o), r_b = r - c_i / 2
-// (Eqs. MBB, NodeVel; c_b = -c_i); far fluid nodes pull without looking at
-// the map.  rot: the spheres rotate (uw, rh are read).
+// (Eqs. MBB, NodeVel; c_b = -c_i).  rot: the spheres rotate (uw, rh are read).
 template <bool NOISE>
 __device__ __forceinline__ void sphere_node(const float *src, float *dst,
                                             const float *ffield, const int *owner,
                                             const float4 *ut, const float4 *uw,
                                             const double *rh, bool rot, const StepArgs &a, int x, int y,
-                                            int z, int own)
+                                            int z)
 {
     const size_t self = ((size_t)z * a.ny + y) * a.nx + x;
     const int xm = (x == 0) ? a.nx - 1 : x - 1, xp = (x == a.nx - 1) ? 0 : x + 1;
     const int ym = (y == 0) ? a.ny - 1 : y - 1, yp = (y == a.ny - 1) ? 0 : y + 1;
     const int zm = (z == 0) ? a.nz - 1 : z - 1, zp = (z == a.nz - 1) ? 0 : z + 1;
     const size_t P = a.pitch;
+    // the map entries of all sources, then all populations (of the source, or
+    // of the node itself at a link), then the moving-wall terms: three memory
+    // round trips instead of two per link
+    int o[19];
+    size_t t[19];
     float n[19];
-    if (own == kFar) {
+    o[0] = kFar;
+    t[0] = self;
 #pragma unroll
-        for (int i = 0; i < 19; ++i) {
-            const int sx = lbd::cx(i) == 1 ? xm : (lbd::cx(i) == -1 ? xp : x);
-            const int sy = lbd::cy(i) == 1 ? ym : (lbd::cy(i) == -1 ? yp : y);
-            const int sz = lbd::cz(i) == 1 ? zm : (lbd::cz(i) == -1 ? zp : z);
-            n[i] = ld_f32(src + (size_t)i * P + ((size_t)sz * a.ny + sy) * a.nx + sx);
-        }
-    } else {
+    for (int i = 1; i < 19; ++i) {
+        const int sx = lbd::cx(i) == 1 ? xm : (lbd::cx(i) == -1 ? xp : x);
+        const int sy = lbd::cy(i) == 1 ? ym : (lbd::cy(i) == -1 ? yp : y);
+        const int sz = lbd::cz(i) == 1 ? zm : (lbd::cz(i) == -1 ? zp : z);
+        t[i] = ((size_t)sz * a.ny + sy) * a.nx + sx;
+        o[i] = owner[t[i]];
+    }
 #pragma unroll
-        for (int i = 0; i < 19; ++i) {
-            const int sx = lbd::cx(i) == 1 ? xm : (lbd::cx(i) == -1 ? xp : x);
-            const int sy = lbd::cy(i) == 1 ? ym : (lbd::cy(i) == -1 ? yp : y);
-            const int sz = lbd::cz(i) == 1 ? zm : (lbd::cz(i) == -1 ? zp : z);
-            const size_t t = ((size_t)sz * a.ny + sy) * a.nx + sx;
-            const int o = i == 0 ? kFar : owner[t];
-            if (o >= 0) {
-                const float4 v = ut[o];
-                float ub[3] = {v.x, v.y, v.z};
-                if (rot) {
-                    const float4 w = uw[o];
-                    const float rb[3] = {image_f((float)((double)x - 0.5 * lbd::cx(i) - rh[3 * o]), a.nx),
-                                         image_f((float)((double)y - 0.5 * lbd::cy(i) - rh[3 * o + 1]), a.ny),
-                                         image_f((float)((double)z - 0.5 * lbd::cz(i) - rh[3 * o + 2]), a.nz)};
-                    const float wv[3] = {w.x, w.y, w.z};
-                    float wr[3];
-                    cross3f(wv, rb, wr);
-                    for (int d = 0; d < 3; ++d) ub[d] += wr[d];
-                }
-                const float uc = lbd::cx(i) * ub[0] + lbd::cy(i) * ub[1] + lbd::cz(i) * ub[2];
-                n[i] = ld_f32(src + (size_t)lbd::opposite(i) * P + self) + 6.0f * lbd::weight(i) * a.rho0 * uc;
-            } else {
-                n[i] = ld_f32(src + (size_t)i * P + t);
-            }
+    for (int i = 0; i < 19; ++i)
+        n[i] = ld_f32(src + (o[i] >= 0 ? (size_t)lbd::opposite(i) * P + self : (size_t)i * P + t[i]));
+#pragma unroll
+    for (int i = 1; i < 19; ++i) {
+        if (o[i] < 0) continue;
+        const float4 v = ut[o[i]];
+        float ub[3] = {v.x, v.y, v.z};
+        if (rot) {
+            const float4 w = uw[o[i]];
+            const float rb[3] = {image_f((float)((double)x - 0.5 * lbd::cx(i) - rh[3 * o[i]]), a.nx),
+                                 image_f((float)((double)y - 0.5 * lbd::cy(i) - rh[3 * o[i] + 1]), a.ny),
+                                 image_f((float)((double)z - 0.5 * lbd::cz(i) - rh[3 * o[i] + 2]), a.nz)};
+            const float wv[3] = {w.x, w.y, w.z};
+            float wr[3];
+            cross3f(wv, rb, wr);
+            for (int d = 0; d < 3; ++d) ub[d] += wr[d];
         }
+        const float uc = lbd::cx(i) * ub[0] + lbd::cy(i) * ub[1] + lbd::cz(i) * ub[2];
+        n[i] += 6.0f * lbd::weight(i) * a.rho0 * uc;
     }
     float fx = a.fx, fy = a.fy, fz = a.fz;
     if (ffield) {
@@ -596,7 +605,7 @@ __global__ void __launch_bounds__(kSphThreads) k_sph_near_nodes(const float *src
     for (unsigned int q = blockIdx.x * blockDim.x + threadIdx.x; q < nl; q += gridDim.x * blockDim.x) {
         const int s = list[q];
         const int x = s % g.nx, y = (s / g.nx) % g.ny, z = s / (g.nx * g.ny);
-        sphere_node<NOISE>(src, dst, ffield, owner, ut, uw, rh, rot, g, x, y, z, kNear);
+        sphere_node<NOISE>(src, dst, ffield, owner, ut, uw, rh, rot, g, x, y, z);
     }
 }
 
@@ -728,6 +737,8 @@ lb_status lb_spheres_place(lb_handle *h, const lb_spheres *s)
                 h->sph_list, h->sph_count);
         h->launches += 2;
         if (e == cudaSuccess) e = cudaGetLastError();
+        // the steps find the accumulators empty
+        if (e == cudaSuccess) e = cudaMemsetAsync(h->sph_acc, 0, (size_t)s->n * kAcc * sizeof(float), h->stream);
     }
     if (e != cudaSuccess) return cuda_fail("lb_spheres_place", e);
     h->sph_n = s->n;
@@ -758,21 +769,18 @@ lb_status lb_step_spheres(lb_handle *h, const lb_spheres *s)
     cudaError_t e = cudaSuccess;
     if (n > 0) {
         const int B = box_edge(s->radius);
-        const unsigned pb = (unsigned)((n + kSphThreads - 1) / kSphThreads);
+        const unsigned pb = (unsigned)((n + kSphUpdThreads - 1) / kSphUpdThreads);
         const dim3 grid((unsigned)((B * B * B + kSphThreads - 1) / kSphThreads), (unsigned)n);
-        e = launch_chained(k_sph_half, pb, kSphThreads, h->stream, s->pos, s->vel, s->mass, s->mass0, n, h->sph_rh,
-                           h->sph_acc, h->sph_count, g, h->d_err);
-        if (e == cudaSuccess)
-            e = launch_chained(k_sph_map, grid, kSphThreads, h->stream, h->sph_owner, src, h->sph_rh, s->vel, s->omega,
-                               s->radius, B, n, g, h->sph_acc, h->d_err);
+        e = launch_chained(k_sph_map, grid, kSphThreads, h->stream, h->sph_owner, src, s->pos, s->vel, s->mass, s->mass0,
+                           h->sph_rh, s->omega, s->radius, B, n, g, h->sph_acc, h->sph_count, h->d_err);
         if (e == cudaSuccess)
             e = launch_chained(s->omega ? k_sph_links<true> : k_sph_links<false>, grid, kSphThreads, h->stream,
                                h->sph_owner, src, h->sph_rh, s->radius, B, n, g, h->sph_acc, h->sph_list,
                                h->sph_count);
         if (e == cudaSuccess)
-            e = launch_chained(k_sph_update, pb, kSphThreads, h->stream, s->vel, s->omega, s->mass, s->mass0, s->radius,
-                               s->force, n, h->sph_acc, h->sph_ut, h->sph_uw);
-        h->launches += 4;
+            e = launch_chained(k_sph_update, pb, kSphUpdThreads, h->stream, s->pos, s->vel, s->omega, s->mass, s->mass0,
+                               s->radius, s->force, h->sph_rh, n, h->sph_acc, h->sph_ut, h->sph_uw, g);
+        h->launches += 3;
     }
     if (e == cudaSuccess) {  // every node with the plain update (solid nodes get values nobody reads)
         e = launch_stream_collide_dt<0>(h, src, dst, nullptr, nullptr);
@@ -784,11 +792,6 @@ lb_status lb_step_spheres(lb_handle *h, const lb_spheres *s)
         e = launch_chained(g.kT > 0.0f ? k_sph_near_nodes<true> : k_sph_near_nodes<false>, grid, kSphThreads, h->stream,
                            src, dst, h->force, h->sph_owner, h->sph_ut, h->sph_uw, h->sph_rh, rot, h->sph_list,
                            h->sph_count, g);
-        h->launches += 1;
-    }
-    if (e == cudaSuccess && n > 0) {
-        e = launch_chained(k_sph_finish, (unsigned)((n + kSphThreads - 1) / kSphThreads), kSphThreads, h->stream, s->pos,
-                           s->vel, s->mass, s->mass0, h->sph_rh, n, g);
         h->launches += 1;
     }
     if (e != cudaSuccess) return cuda_fail("lb_step_spheres", e);
