@@ -45,7 +45,7 @@ def _deps():
 
 
 # the files that define the fused stream-collide kernel
-STREAM_COLLIDE_FILES = ("d3q19.cuh", "f32x2.cuh", "stream_collide.cuh", "sc_f32.cu", "sc_f16.cu", "sc_bf16.cu",
+STREAM_COLLIDE_FILES = ("chain.cuh", "d3q19.cuh", "f32x2.cuh", "stream_collide.cuh", "sc_f32.cu", "sc_f16.cu", "sc_bf16.cu",
                         "step_args.h")
 
 
