@@ -15,8 +15,11 @@
 //  - every block calls wait_for_previous() before it reads or writes any
 //    global memory (kernel parameters are free);
 //  - global loads are plain loads ordered after it: no __ldg and no const
-//    __restrict__ pointers, whose loads the compiler may move up (the ld_*
-//    functions below are volatile and stay where they stand);
+//    __restrict__ pointers, whose loads the compiler may move up.  The ld_*
+//    functions below are volatile, which keeps them behind the wait and in
+//    order among themselves, but not against ordinary stores: a kernel that
+//    stores to what it has read this way, with no branch on the loaded value
+//    in between, puts loads_done() before the store;
 //  - it lets its own successor start only after its wait, so at most two
 //    kernels of a stream are in flight and the buffers a step reads are never
 //    written by an earlier kernel still running.
@@ -31,6 +34,9 @@ __device__ __forceinline__ void wait_for_previous()
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
+
+// Every load above stands before every store below (for the compiler).
+__device__ __forceinline__ void loads_done() { asm volatile("" ::: "memory"); }
 
 __device__ __forceinline__ float ld_f32(const float *p)
 {

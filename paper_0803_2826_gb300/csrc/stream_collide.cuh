@@ -307,6 +307,7 @@ __global__ void __launch_bounds__(kBX) k_patch_impulse_nodes(const typename lbd:
             if (atomicMax(claim + node, tag) == tag) continue;  // another thread has it
             update_node<DT, NOISE, true, WALLS>(src, dst, ffield, facc, a, x, y, z);
             // the impulses are applied: clear them for the next coupling call
+            loads_done();
             facc[node] = 0.0f;
             facc[a.pitch + node] = 0.0f;
             facc[2 * a.pitch + node] = 0.0f;
