@@ -495,9 +495,12 @@ lb_status lb_adjoint_kinetic_coupled(lb_handle *h, const lb_particles *parts, co
  * per_replica[r]. */
 typedef struct lb_batch lb_batch;
 
-/* Launch shape of the persistent kernel: threads per block, nodes per tile
- * (a run of consecutive nodes of one replica), blocks per SM; grid is an
- * output (resident blocks).  Chosen by lb_batch_autotune or set directly. */
+/* Launch shape of the persistent kernel: threads per block (a multiple of 32
+ * from 32 to 1024; above 512 only if some replica has odd nx, where blocks of
+ * 512 run in their place, and LB_EUNSUPPORTED otherwise), nodes per tile (a run
+ * of consecutive nodes of one replica, at least 32), blocks per SM (at least 1;
+ * as many of them run as have room); grid is an output (resident blocks).
+ * Chosen by lb_batch_autotune or set directly. */
 typedef struct {
     int threads;
     int tile_nodes;
