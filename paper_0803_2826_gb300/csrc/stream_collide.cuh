@@ -267,6 +267,15 @@ __device__ __forceinline__ bool patch_node(int bx, int by, int bz, int k, int sp
     return z >= a.z0 && z < a.z1;
 }
 
+// Clears the impulses of a node patch_node refuses, where it is a solid one
+// (clear_solid; any number of threads may).
+__device__ __forceinline__ void clear_outside(float *facc, const StepArgs &a, int x, int y, int z)
+{
+    if (z < 0 || z >= a.nz) return;
+    const size_t node = ((size_t)z * a.ny + y) * a.nx + x;
+    facc[node] = facc[a.pitch + node] = facc[2 * a.pitch + node] = 0.0f;
+}
+
 // Re-update of the nodes that received particle impulses, after an update of
 // all nodes that left the impulses out (the coupling ran meanwhile): the
 // span^3 nodes of each record of particle p, records[s][p] (the linear index
@@ -302,7 +311,10 @@ __global__ void __launch_bounds__(kBX) k_patch_impulse_nodes(const typename lbd:
         const int bx = base - (int)(row * (uint32_t)a.nx), by = (int)(row - plane * (uint32_t)a.ny), bz = (int)plane;
         for (int e = q; e < nk; e += 8) {
             int x, y, z;
-            if (!patch_node<WALLS>(bx, by, bz, e, span, a, x, y, z)) continue;  // solid node
+            if (!patch_node<WALLS>(bx, by, bz, e, span, a, x, y, z)) {
+                clear_outside(facc, a, x, y, z);
+                continue;
+            }
             const size_t node = ((size_t)z * a.ny + y) * a.nx + x;
             if (atomicMax(claim + node, tag) == tag) continue;  // another thread has it
             update_node<DT, NOISE, true, WALLS>(src, dst, ffield, facc, a, x, y, z);
@@ -349,7 +361,10 @@ __global__ void __launch_bounds__(kBX, 8) k_patch_impulse_nodes_f32(float *dst, 
         const int bx = base - (int)(row * (uint32_t)a.nx), by = (int)(row - plane * (uint32_t)a.ny), bz = (int)plane;
         for (int e = q; e < nk; e += 8) {
             int x, y, z;
-            if (!patch_node<WALLS>(bx, by, bz, e, span, a, x, y, z)) continue;  // solid node
+            if (!patch_node<WALLS>(bx, by, bz, e, span, a, x, y, z)) {
+                clear_outside(facc, a, x, y, z);
+                continue;
+            }
             const size_t node = ((size_t)z * a.ny + y) * a.nx + x;
             // the claim, the impulse and the stored values are requested
             // together (one memory round trip instead of three); the values
@@ -518,6 +533,28 @@ __device__ __forceinline__ void pull_pair(const typename lbd::Store<DT>::T *__re
     }
 }
 
+// A particle that a narrow channel cannot keep inside its band spreads to the
+// solid planes too.  No update reads that; it is cleared, with the impulses
+// that are applied, by the threads of the fluid nodes next to it.
+__device__ __forceinline__ void clear_solid(float *facc, const StepArgs &a, int z, uint32_t self)
+{
+    const uint32_t plane = (uint32_t)a.nx * (uint32_t)a.ny;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        if (z == a.z0) facc[d * a.pitch + (self - plane)] = 0.0f;
+        if (z == a.z1 - 1) facc[d * a.pitch + (self + plane)] = 0.0f;
+    }
+}
+__device__ __forceinline__ void clear_solid_pair(float *facc, const StepArgs &a, int z, uint32_t self)  // even nx
+{
+    const uint32_t plane = (uint32_t)a.nx * (uint32_t)a.ny;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        if (z == a.z0) Pair<0>::store(facc + d * a.pitch + (self - plane), 0.0f, 0.0f, 1.0f);
+        if (z == a.z1 - 1) Pair<0>::store(facc + d * a.pitch + (self + plane), 0.0f, 0.0f, 1.0f);
+    }
+}
+
 template <int DT, bool FIELD, bool WALLS>
 __device__ __forceinline__ void load_pair(const typename lbd::Store<DT>::T *__restrict__ src,
                                           const float *__restrict__ ffield, float *facc,
@@ -528,8 +565,12 @@ __device__ __forceinline__ void load_pair(const typename lbd::Store<DT>::T *__re
     const uint32_t self = (uint32_t)((z * a.ny + y) * a.nx + x0);
     // only the planes next to a wall look at their links (z is the same for
     // a whole row, so a warp rarely takes both ways)
-    if (WALLS && (z == a.z0 || z == a.z1 - 1)) pull_pair<DT, true>(src, a, x0, y, z, self, n);
-    else pull_pair<DT, false>(src, a, x0, y, z, self, n);
+    if (WALLS && (z == a.z0 || z == a.z1 - 1)) {
+        if (FIELD && facc && a.consume && take) clear_solid_pair(facc, a, z, self);
+        pull_pair<DT, true>(src, a, x0, y, z, self, n);
+    } else {
+        pull_pair<DT, false>(src, a, x0, y, z, self, n);
+    }
     f0[0] = f1[0] = a.fx;
     f0[1] = f1[1] = a.fy;
     f0[2] = f1[2] = a.fz;
@@ -776,6 +817,10 @@ __device__ __forceinline__ void load_pair_any(const typename lbd::Store<DT>::T *
     second_node(a, at, xb, yb, zb);
     const PullAt pa = pull_at<WALLS>(a, at.x, at.y, at.z), pb = pull_at<WALLS>(a, xb, yb, zb);
     if (WALLS && (pa.lo || pa.hi || pb.lo || pb.hi)) {  // next to a wall (load_pair)
+        if (FIELD && facc && a.consume && take) {
+            clear_solid(facc, a, at.z, pa.self);
+            clear_solid(facc, a, zb, pb.self);
+        }
 #pragma unroll
         for (int i = 0; i < 19; ++i)
             n[i] = lbp::f2(pull_one<DT, true>(src, a, pa, i), pull_one<DT, true>(src, a, pb, i));
