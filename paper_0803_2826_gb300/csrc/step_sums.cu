@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(38 * kRows) k_reduce_rows(const float *in, siz
 
 size_t sc_block_count(const lb_handle *h)
 {
-    const dim3 g = sc_grid(h);
+    const dim3 g = sums_grid(h);
     return (size_t)g.x * g.y * g.z;
 }
 

@@ -712,21 +712,23 @@ struct PairAt {
     bool va, vb;
 };
 
-// Blocks of kLinBX threads that cover the fluid nodes (locate_pair).
-inline dim3 linear_grid(const StepArgs &a)
+// Blocks of bx threads that cover the fluid nodes of a box of nn nodes, or
+// those between its first and last plane (locate_pair).
+inline dim3 linear_grid(size_t nn, size_t plane, bool walls, int bx)
 {
-    const size_t first = a.z0 > 0 ? (size_t)a.nx * a.ny : 0;
-    const size_t pairs = (a.nn - first - (first & ~(size_t)1) + 1) / 2;
-    return dim3((unsigned)((pairs + kLinBX - 1) / kLinBX));
+    const size_t first = walls ? plane : 0;
+    const size_t pairs = (nn - first - (first & ~(size_t)1) + 1) / 2;
+    return dim3((unsigned)((pairs + bx - 1) / bx));
 }
+inline dim3 linear_grid(const StepArgs &a) { return linear_grid(a.nn, (size_t)a.nx * a.ny, a.z0 > 0, kLinBX); }
 
-template <bool WALLS>
+template <bool WALLS, int BX = kLinBX>
 __device__ __forceinline__ bool locate_pair(const StepArgs &a, PairAt &p)
 {
     const uint32_t plane = (uint32_t)a.nx * (uint32_t)a.ny;
     const uint32_t first = WALLS ? plane : 0u;
     const uint32_t end = (uint32_t)a.nn - first;
-    p.s = (first & ~1u) + 2u * (blockIdx.x * (uint32_t)kLinBX + threadIdx.x);
+    p.s = (first & ~1u) + 2u * (blockIdx.x * (uint32_t)BX + threadIdx.x);
     if (p.s >= end) return false;
     p.va = !WALLS || p.s >= first;
     p.vb = p.s + 1u < end;
@@ -954,10 +956,11 @@ auto linear_kernel()
 }
 
 // The step with moment sums on boxes whose pairs cannot move as one access
-// (rows of odd length, or more elements than 32-bit indices reach): rows mapped to blocks
-// as in k_stream_collide2, the pair's addresses and stores one node at a time,
-// the last node of an odd row alone.  The arithmetic is the pair's, so the
-// populations are those of k_stream_collide_linear bit for bit.
+// (rows of odd length, or more elements than 32-bit indices reach): pairs over
+// the linear index as in the ODD form of k_stream_collide_linear, whose
+// arithmetic and so whose populations these are bit for bit.  3 x 200 x 200
+// takes 15 us and 65^3 19 us a step; with a row to a block, which leaves most
+// of it idle, 199 and 34 us, and one node a thread 126 and 29 us.
 template <int DT, bool NOISE, bool FIELD, bool WALLS>
 __global__ void __launch_bounds__(kBX) k_stream_collide_sums_any(const typename lbd::Store<DT>::T *__restrict__ src,
                                                                  typename lbd::Store<DT>::T *__restrict__ dst,
@@ -965,15 +968,14 @@ __global__ void __launch_bounds__(kBX) k_stream_collide_sums_any(const typename 
                                                                  float *facc, const StepArgs a, float *partials)
 {
     __shared__ float part[kBX / 32][38];
-    const int x0 = 2 * (blockIdx.x * kBX + threadIdx.x);
-    const bool mine = x0 < a.nx;  // lanes past the row load its first nodes and store nothing
     PairAt at;
-    at.x = mine ? x0 : 0;
-    at.y = blockIdx.y;
-    at.z = blockIdx.z + a.z0;
-    at.s = (uint32_t)((at.z * a.ny + at.y) * a.nx + at.x);
-    at.va = true;
-    at.vb = at.x + 1 < a.nx;
+    const bool mine = locate_pair<WALLS, kBX>(a, at);
+    if (!mine) {  // lanes past the last pair load the first fluid node and store nothing
+        at.s = 0u;
+        at.x = at.y = 0;
+        at.z = a.z0;
+        at.va = at.vb = false;
+    }
     wait_for_previous();
     lbp::F2 n[19], m[19], out[19];
     float f0[3], f1[3];
@@ -983,14 +985,14 @@ __global__ void __launch_bounds__(kBX) k_stream_collide_sums_any(const typename 
 #pragma unroll
     for (int k = 0; k < 19; ++k) {
         lbp::split(m[k], m0[k], m1[k]);
+        if (!at.va) m0[k] = 0.0f;
         if (!at.vb) m1[k] = 0.0f;
     }
     warp_moment_sums(m0, m1, mine, part);
     if (mine) {
         lbp::collide_moments2<NOISE>(m, lbp::f2(f0[0], f1[0]), lbp::f2(f0[1], f1[1]), lbp::f2(f0[2], f1[2]), a, a.rk,
                                      at.s, a.replica, out);
-        store_one<DT>(dst, a, at.s, out, false);
-        if (at.vb) store_one<DT>(dst, a, at.s + 1u, out, true);
+        store_pair_any<DT>(dst, a, at, out);
     }
     block_moment_sums_out(part, partials + 38 * block_linear());
 }
@@ -1012,8 +1014,15 @@ inline dim3 sc_grid(const lb_handle *h)
     return dim3(((h->p.nx + 1) / 2 + kBX - 1) / kBX, h->p.ny, nzf);
 }
 
+// Grid of the launch with moment sums (a row of partial sums a block).
+inline dim3 sums_grid(const lb_handle *h)
+{
+    return sc_paired(h) ? sc_grid(h) : linear_grid(h->n_nodes, (size_t)h->p.nx * h->p.ny, h->p.walls != 0, kBX);
+}
+
 // partials != NULL: the launch also writes per-block moment sums
-// (partials[block][38], block = blockIdx.x + gridDim.x (blockIdx.y + gridDim.y blockIdx.z)).
+// (partials[block][38], block = blockIdx.x + gridDim.x (blockIdx.y + gridDim.y blockIdx.z)),
+// and src, dst are the handle's own buffers (256-byte aligned, so sc_paired decides).
 template <int DT>
 cudaError_t launch_stream_collide_dt(const lb_handle *h, const void *src, void *dst, float *facc,
                                      float *partials)
@@ -1035,10 +1044,11 @@ cudaError_t launch_stream_collide_dt(const lb_handle *h, const void *src, void *
     const bool odd = !paired;
     const dim3 linear = linear_grid(a);
 #define LBI_SC(NZ, FL, WL)                                                                                        \
-    (partials ? (paired ? launch_chained(k_stream_collide2<DT, NZ, FL, WL, true>, grid, block, h->stream, s, d,     \
-                                         h->force, facc, a, partials)                                             \
-                        : launch_chained(k_stream_collide_sums_any<DT, NZ, FL, WL>, grid, block, h->stream, s, d,   \
-                                         h->force, facc, a, partials))                                            \
+    (partials ? (sc_paired(h)                                                                                     \
+                     ? launch_chained(k_stream_collide2<DT, NZ, FL, WL, true>, grid, block, h->stream, s, d,        \
+                                      h->force, facc, a, partials)                                                \
+                     : launch_chained(k_stream_collide_sums_any<DT, NZ, FL, WL>, sums_grid(h), block, h->stream, s, \
+                                      d, h->force, facc, a, partials))                                            \
      : rows   ? launch_chained(rows_kernel<DT, NZ, FL, WL>(), grid, block, h->stream, s, d, h->force,    \
                                facc, a, nullptr)                                                                  \
      : odd    ? launch_chained(linear_kernel<DT, NZ, FL, WL, true>(), linear, dim3(kLinBX), h->stream, s, d, \
