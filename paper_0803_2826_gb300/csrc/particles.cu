@@ -2393,6 +2393,22 @@ const void *lanes_kernel(int kw, bool warp)
     return warp ? (const void *)k_couple_lanes<DT, 4, 32> : (const void *)k_couple_lanes<DT, 4, 8>;
 }
 
+// Whether eight lanes a particle pay for a call on `blocks` blocks.  In the
+// serial order always.  Beside the step's update of all nodes they take the
+// registers of the update's blocks (162 to 168 a thread: three blocks of 16
+// particles fill an SM, where one thread a particle needs one block of 128),
+// so they pay while the coupling is the longer of the two.  Ten phi_4 sub-steps
+// of 7296 particles beside 128^3 nodes: 269 against 293 us a step, 160^3
+// 311 / 324, 192^3 377 / 362, 256^3 583 / 472; of 2432 particles 192^3 339 / 346,
+// 208^3 377 / 373, 256^3 509 / 471; phi_3, 4864 particles, 192^3 261 / 277,
+// 208^3 305 / 300.
+bool lanes_beside(const lb_handle *h, int kw, int blocks)
+{
+    if (!h->aux || h->stream != h->aux) return true;
+    const int few = (kw == 3 ? 2 : 1) * device_sm_count();
+    return h->n_nodes <= ((size_t)1 << (blocks <= few ? 23 : 22));
+}
+
 template <int DT>
 cudaError_t run_substeps(lb_handle *h, const lb_particles *pp, const lb_couple_params *cp)
 {
@@ -2437,7 +2453,7 @@ cudaError_t run_substeps(lb_handle *h, const lb_particles *pp, const lb_couple_p
         if (le != cudaSuccess) return le;
         h->launches += 1;
         P->sub_counter += (uint32_t)cp->n_substeps;
-            return cudaGetLastError();
+        return cudaGetLastError();
     }
 
     // persistent path when every particle group can be resident at once
@@ -2447,12 +2463,16 @@ cudaError_t run_substeps(lb_handle *h, const lb_particles *pp, const lb_couple_p
         const int wblocks = (int)(((size_t)n * 32 + kPThreads - 1) / kPThreads);
         const int eblocks = (int)(((size_t)n * 8 + kPThreads - 1) / kPThreads);
         if (c.kw > 2) {
-            // several lanes a particle while they can all be resident (up to
-            // ~9700 particles), the stencil caches in shared memory beyond
+            // a warp a particle up to two blocks per SM (1216 particles on 152
+            // SMs: 81 us a phi_4 call of ten sub-steps and the step in a 64^3
+            // box, 134 us for 1280 particles with eight lanes), eight lanes
+            // while they are resident and may be (lanes_beside), the stencil
+            // caches in shared memory beyond
             const bool warp = wblocks <= 2 * sms;
             const int lblocks = warp ? wblocks : eblocks;
             const void *lfn = lanes_kernel<DT>(c.kw, warp);
-            if (lblocks <= resident_blocks(lfn, 0)) return launch_persistent(h, pp, cp, c, lfn, lblocks, 0);
+            if ((warp || lanes_beside(h, c.kw, lblocks)) && lblocks <= resident_blocks(lfn, 0))
+                return launch_persistent(h, pp, cp, c, lfn, lblocks, 0);
             const size_t smem = c.kw == 3 ? wide_smem_bytes<3>() : wide_smem_bytes<4>();
             const void *kfn = c.kw == 3 ? (const void *)k_couple_persistent_wide<DT, 3>
                                         : (const void *)k_couple_persistent_wide<DT, 4>;
