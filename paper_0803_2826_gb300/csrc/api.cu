@@ -83,14 +83,11 @@ StepArgs make_args(const lb_handle *h)
                                     : std::sqrt(1.0 - p.gamma_even * p.gamma_even);
         a.amp[k - 4] = (float)(phi * (double)lbd::sqrt_inv_w(k));
     }
-    const double gm[4] = {p.gamma_bulk, p.gamma_shear, p.gamma_odd, p.gamma_even};
-    for (int k = 4; k < 19; ++k)
-        a.rel[k - 4] = (float)(gm[k == 4 ? 0 : k < 10 ? 1 : k < 16 ? 2 : 3] * (double)lbd::inv_w(k));
-    for (int q = 0; q < 4; ++q) {
-        const double g = q == 0 ? p.gamma_bulk : p.gamma_shear, iw = (double)lbd::inv_w(4 + q);
-        a.eq[q] = (float)((1.0 - g) * iw);
-        a.frc[q] = (float)((1.0 + g) * iw * (q == 3 ? 0.5 : 1.0));
-    }
+    for (int k = 10; k < 19; ++k) a.rel[k - 10] = (float)((k < 16 ? p.gamma_odd : p.gamma_even) * (double)lbd::inv_w(k));
+    a.frc[0] = (float)(1.0 + p.gamma_bulk);
+    a.frc[1] = (float)(1.0 + p.gamma_shear);
+    a.frc[2] = (float)(0.5 * (1.0 + p.gamma_shear));
+    a.reserved[0] = a.reserved[1] = a.reserved[2] = 0.0f;
     a.forced = h->force || p.body_force[0] != 0.0 || p.body_force[1] != 0.0 || p.body_force[2] != 0.0;
     a.consume = 0;
     a.fx = (float)p.body_force[0];

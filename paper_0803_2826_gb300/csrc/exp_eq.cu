@@ -211,9 +211,9 @@ __device__ __forceinline__ void collide_exp2(const F2 m[19], F2 fx, F2 fy, F2 fz
                      hgs1 * (ux * fy + uy * fx),      hgs1 * (uy * fz + uz * fy),   hgs1 * (uz * fx + ux * fz)};
     F2 M[19];
     M[0] = m[0];
-    M[1] = (m[1] + fx) * three;
-    M[2] = (m[2] + fy) * three;
-    M[3] = (m[3] + fz) * three;
+    M[1] = m[1] + fx;  // (backward2 multiplies by 1 / w = 3)
+    M[2] = m[2] + fy;
+    M[3] = m[3] + fz;
     M[4] = lbp::fma2(lbp::f2s(a.g_bulk), m[4] - meq[4], meq[4] + F[0]) * lbd::inv_w(4);
 #pragma unroll
     for (int k = 5; k < 10; ++k) M[k] = lbp::fma2(lbp::f2s(a.g_shear), m[k] - meq[k], meq[k] + F[k - 4]) * lbd::inv_w(k);

@@ -139,11 +139,17 @@ __device__ __forceinline__ void forward2_conserved(const F2 n[19], F2 m[4])
     m[3] = (n[5] - n[6]) + ((pc - pd) + (pe - pg));
 }
 
-// Back transform n_i = a_i sum_k e_ki M_k (M_k = m_k / w_k) of both nodes:
-// lbd::backward in packed form.  WEIGHTED false leaves the a_i out, which is
-// the transpose of forward2 (the reverse mode's dL/dn_i = sum_k e_ki mu_k).
+// Back transform n_i = a_i sum_k e_ki M_k (M_k = m_k / w_k, but m_k itself for
+// k = 1..3) of both nodes: lbd::backward in packed form.  WEIGHTED false leaves
+// the a_i and that factor out, which is the transpose of forward2 (the reverse
+// mode's dL/dn_i = sum_k e_ki mu_k).
 template <bool WEIGHTED>
 __device__ __forceinline__ F2 weigh(float a, F2 v) { return WEIGHTED ? f2s(a) * v : v; }
+
+// M_k + v for k = 1..3.  WEIGHTED: M holds m_k, not yet over its norm 1/3, and
+// the momentum, the largest of the moments, is multiplied and added in one rounding.
+template <bool WEIGHTED>
+__device__ __forceinline__ F2 plus3(F2 j, F2 v) { return WEIGHTED ? fma2(j, f2s(3.0f), v) : j + v; }
 
 template <bool WEIGHTED = true>
 __device__ __forceinline__ void backward2(const F2 M[19], F2 n[19])
@@ -153,12 +159,12 @@ __device__ __forceinline__ void backward2(const F2 M[19], F2 n[19])
     {
         const F2 base = M[0] - M16x2;
         const F2 Ex = base + M5x2 - M17x2;
-        const F2 Ox = M[1] - (M[10] + M[10]);
+        const F2 Ox = plus3<WEIGHTED>(M[1], f2s(-2.0f) * M[10]);
         const F2 Eyz = base - M[5] + M[17];
         const F2 Ey = Eyz + M[6] - M[18];
         const F2 Ez = Eyz - M[6] + M[18];
-        const F2 Oy = M[2] - (M[11] + M[11]);
-        const F2 Oz = M[3] - (M[12] + M[12]);
+        const F2 Oy = plus3<WEIGHTED>(M[2], f2s(-2.0f) * M[11]);
+        const F2 Oz = plus3<WEIGHTED>(M[3], f2s(-2.0f) * M[12]);
         n[1] = weigh<WEIGHTED>(lbd::kA1, Ex + Ox);
         n[2] = weigh<WEIGHTED>(lbd::kA1, Ex - Ox);
         n[3] = weigh<WEIGHTED>(lbd::kA1, Ey + Oy);
@@ -170,8 +176,8 @@ __device__ __forceinline__ void backward2(const F2 M[19], F2 n[19])
         const F2 base = M[0] + M[4] + M[16];
         const F2 Exy = base + M[5] + M[6] + M[17] + M[18];
         const F2 E7 = Exy + M[7], E8 = Exy - M[7];
-        const F2 oxy1 = M[1] + M[10] + M[13];
-        const F2 oxy2 = M[2] + M[11] - M[14];
+        const F2 oxy1 = plus3<WEIGHTED>(M[1], M[10]) + M[13];
+        const F2 oxy2 = plus3<WEIGHTED>(M[2], M[11]) - M[14];
         const F2 O7 = oxy1 + oxy2, O8 = oxy1 - oxy2;
         n[7] = weigh<WEIGHTED>(lbd::kA2, E7 + O7);
         n[10] = weigh<WEIGHTED>(lbd::kA2, E7 - O7);
@@ -179,8 +185,8 @@ __device__ __forceinline__ void backward2(const F2 M[19], F2 n[19])
         n[9] = weigh<WEIGHTED>(lbd::kA2, E8 - O8);
         const F2 Eyz = base - M5x2 - M17x2;
         const F2 E11 = Eyz + M[8], E12 = Eyz - M[8];
-        const F2 oyz2 = M[2] + M[11] + M[14];
-        const F2 oyz3 = M[3] + M[12] - M[15];
+        const F2 oyz2 = plus3<WEIGHTED>(M[2], M[11]) + M[14];
+        const F2 oyz3 = plus3<WEIGHTED>(M[3], M[12]) - M[15];
         const F2 O11 = oyz2 + oyz3, O12 = oyz2 - oyz3;
         n[11] = weigh<WEIGHTED>(lbd::kA2, E11 + O11);
         n[14] = weigh<WEIGHTED>(lbd::kA2, E11 - O11);
@@ -188,8 +194,8 @@ __device__ __forceinline__ void backward2(const F2 M[19], F2 n[19])
         n[13] = weigh<WEIGHTED>(lbd::kA2, E12 - O12);
         const F2 Exz = base + M[5] - M[6] + M[17] - M[18];
         const F2 E15 = Exz + M[9], E16 = Exz - M[9];
-        const F2 oxz1 = M[1] + M[10] - M[13];
-        const F2 oxz3 = M[3] + M[12] + M[15];
+        const F2 oxz1 = plus3<WEIGHTED>(M[1], M[10]) - M[13];
+        const F2 oxz3 = plus3<WEIGHTED>(M[3], M[12]) + M[15];
         const F2 O15 = oxz1 + oxz3, O16 = oxz1 - oxz3;
         n[15] = weigh<WEIGHTED>(lbd::kA2, E15 + O15);
         n[18] = weigh<WEIGHTED>(lbd::kA2, E15 - O15);
@@ -277,9 +283,9 @@ struct RunningKeys {
 // The deterministic part of the collision of two nodes (Sec. 3.4, 3.7): from
 // their moments m and force densities (fx, fy, fz) to the post-collision
 // moments over w_k, M, and the densities.  The noisy update is bound by
-// instruction issue, so each mode's constants are multiplied on the host and
-// the forcing is passed over where nothing forces; with the shorter
-// Box-Muller map below, 256^3 FP16 373 us a step (396 before), 512 replicas
+// instruction issue, so constants are multiplied on the host where that costs
+// no accuracy and the forcing is passed over where nothing forces; with the
+// Box-Muller map above, 256^3 FP16 373 us a step (396 before), 512 replicas
 // 1.25 ms (1.29), 200^3 FP32 178 us (188), 256^3 FP32 364 us (382).
 __device__ __forceinline__ void relax2(const F2 m[19], F2 fx, F2 fy, F2 fz, const lbi::StepArgs &a, F2 M[19], F2 &rho)
 {
@@ -294,37 +300,38 @@ __device__ __forceinline__ void relax2(const F2 m[19], F2 fx, F2 fy, F2 fz, cons
 
     const F2 uxx = ux * ux, uyy = uy * uy, uzz = uz * uz;
     const F2 u2 = uxx + uyy + uzz;
-    const F2 meq4 = rho * u2;
-    const F2 meq5 = rho * (uxx * three - u2);
-    const F2 meq6 = rho * (uyy - uzz);
-    const F2 ruy = rho * uy;
-    const F2 meq7 = ruy * ux;
-    const F2 meq8 = ruy * uz;
-    const F2 meq9 = rho * uz * ux;
-    // M_k = (gamma_k m_k + (1 - gamma_k) m^eq_k + F_k) / w_k, with the constants of
-    // each mode multiplied beforehand
-    F2 S[6] = {meq4 * a.eq[0], meq5 * a.eq[1], meq6 * a.eq[2], meq7 * a.eq[3], meq8 * a.eq[3], meq9 * a.eq[3]};
+    // M_k = (gamma_k (m_k - m^eq_k) + m^eq_k + F_k) / w_k: the rounding of gamma_k
+    // only meets the difference, nothing cancels however small gamma_k is, and
+    // 1 / w_k is exact.  (gamma_k / w_k and (1 - gamma_k) / w_k from the host save
+    // a quarter of these operations, 1.2% of a batched step and 0.4% or less of
+    // others, but round to a factor of up to 1 + 1e-7 on a moment at equilibrium.)
+    const F2 ruy = rho * uy, nrho = f2s(-a.rho0) - m[0], nruy = nrho * uy;
+    const F2 t5 = uxx * three - u2, t6 = uyy - uzz;
+    F2 S[6] = {rho * u2, rho * t5, rho * t6, ruy * ux, ruy * uz, rho * uz * ux};  // m^eq
+    const F2 d[6] = {fma2(nrho, u2, m[4]), fma2(nrho, t5, m[5]),  fma2(nrho, t6, m[6]),
+                     fma2(nruy, ux, m[7]), fma2(nruy, uz, m[8]), fma2(nrho * uz, ux, m[9])};
+    F2 jx = m[1], jy = m[2], jz = m[3];
     M[0] = m[0];
     if (a.forced) {  // the same for the whole launch
         const F2 uf = ux * fx + uy * fy + uz * fz;
         S[0] = fma2(uf, a.frc[0], S[0]);
         S[1] = fma2(ux * fx * three - uf, a.frc[1], S[1]);
-        S[2] = fma2(uy * fy - uz * fz, a.frc[2], S[2]);
-        S[3] = fma2(ux * fy + uy * fx, a.frc[3], S[3]);
-        S[4] = fma2(uy * fz + uz * fy, a.frc[3], S[4]);
-        S[5] = fma2(uz * fx + ux * fz, a.frc[3], S[5]);
-        M[1] = (m[1] + fx) * three;
-        M[2] = (m[2] + fy) * three;
-        M[3] = (m[3] + fz) * three;
-    } else {
-        M[1] = m[1] * three;
-        M[2] = m[2] * three;
-        M[3] = m[3] * three;
+        S[2] = fma2(uy * fy - uz * fz, a.frc[1], S[2]);
+        S[3] = fma2(ux * fy + uy * fx, a.frc[2], S[3]);
+        S[4] = fma2(uy * fz + uz * fy, a.frc[2], S[4]);
+        S[5] = fma2(uz * fx + ux * fz, a.frc[2], S[5]);
+        jx = jx + fx;
+        jy = jy + fy;
+        jz = jz + fz;
     }
+    M[1] = jx;  // (backward2 multiplies by 1 / w = 3)
+    M[2] = jy;
+    M[3] = jz;
 #pragma unroll
-    for (int k = 4; k < 10; ++k) M[k] = fma2(m[k], a.rel[k - 4], S[k - 4]);
+    for (int k = 4; k < 10; ++k)
+        M[k] = fma2(d[k - 4], k == 4 ? a.g_bulk : a.g_shear, S[k - 4]) * lbd::inv_w(k);
 #pragma unroll
-    for (int k = 10; k < 19; ++k) M[k] = m[k] * a.rel[k - 4];
+    for (int k = 10; k < 19; ++k) M[k] = m[k] * a.rel[k - 10];
 }
 
 // The noise of nodes node0, node0 + 1 (Sec. 3.5) added to M:

@@ -48,9 +48,9 @@ struct StepArgs {
     float g_shear, g_bulk, g_odd, g_even;
     float phi_shear, phi_bulk, phi_odd, phi_even;  // sqrt(1 - gamma^2)
     float amp[15];         // noise of mode k = 4..18 per unit sqrt(mu rho): phi_k / sqrt(w_k)
-    float rel[15];         // gamma_k / w_k of mode k = 4..18
-    float eq[4];           // (1 - gamma_k) / w_k of modes 4, 5, 6 and 7..9
-    float frc[4];          // (1 + gamma_k) / w_k of modes 4, 5, 6, half of it of modes 7..9
+    float rel[9];          // gamma_k / w_k of mode k = 10..18
+    float frc[3];          // 1 + gamma_bulk, 1 + gamma_shear, half of that
+    float reserved[3];     // 0 (keeps the members below where they are read in fours)
     float fx, fy, fz;      // uniform body force
     int forced;            // a body force, a force field or particle impulses act
     float scale, inv_scale;  // storage scale of FP16/BF16 deviations
@@ -64,6 +64,8 @@ struct StepArgs {
     // in, and the 256^3 FP32 update goes from 72 registers and 365 us to 76 and 376)
     int consume;           // the impulses read are applied for good: clear them
 };
+static_assert(offsetof(StepArgs, amp) % 8 == 4 && offsetof(StepArgs, rk) % 16 == 0,
+              "the noise constants or the round keys moved against the groups they are read in");
 
 // Index checks of a library built with -DLB_DEBUG_BOUNDS: the element index i
 // of an access to an array of n elements is tested first; outside, the error
