@@ -103,7 +103,9 @@ __host__ __device__ constexpr int opposite(int i)
          : i == 15 ? 18 : i == 16 ? 17 : i == 17 ? 16 : 15;
 }
 
-// Forward transform m_k = sum_i e_ki n_i (Eq. (forward)).
+// Forward transform m_k = sum_i e_ki n_i (Eq. (forward)).  AS_PAIR: in the
+// order of additions of the packed transform (lbp::forward2).
+template <bool AS_PAIR = false>
 __device__ __forceinline__ void forward(const float n[19], float m[19])
 {
     // even (pair sums) and odd (pair differences) parts
@@ -119,7 +121,7 @@ __device__ __forceinline__ void forward(const float n[19], float m[19])
     const float A = sx + sy + sz;
     const float Dxy = sa + sb, Dyz = sc + sd, Dxz = se + sg;
     const float D = Dxy + Dyz + Dxz;
-    const float t5 = Dxy - 2.0f * Dyz + Dxz;
+    const float t5 = AS_PAIR ? (Dxy + Dxz) - 2.0f * Dyz : Dxy - 2.0f * Dyz + Dxz;
     const float t6 = Dxy - Dxz;
     const float syz = sy + sz;
     m[0] = n[0] + A + D;
@@ -149,20 +151,24 @@ __device__ __forceinline__ void forward(const float n[19], float m[19])
 }
 
 // Back transform n_i = a_i sum_k e_ki M_k with M_k = m_k / w_k already scaled.
+// AS_PAIR: M_1..3 are m_1..3 themselves, multiplied by 1 / w = 3 and added in
+// one rounding, as in the packed transform (lbp::backward2).
+template <bool AS_PAIR = false>
 __device__ __forceinline__ void backward(const float M[19], float n[19])
 {
+    const auto plus = [](float m, float v) { return AS_PAIR ? fmaf(m, 3.0f, v) : m + v; };
     // rest
     n[0] = kA0 * (M[0] - M[4] + M[16]);
     // axes: even part E, odd part O; n_+ = a (E + O), n_- = a (E - O)
     {
         const float base = M[0] - 2.0f * M[16];
         const float Ex = base + 2.0f * M[5] - 2.0f * M[17];
-        const float Ox = M[1] - 2.0f * M[10];
+        const float Ox = plus(M[1], -2.0f * M[10]);
         const float Eyz = base - M[5] + M[17];
         const float Ey = Eyz + M[6] - M[18];
         const float Ez = Eyz - M[6] + M[18];
-        const float Oy = M[2] - 2.0f * M[11];
-        const float Oz = M[3] - 2.0f * M[12];
+        const float Oy = plus(M[2], -2.0f * M[11]);
+        const float Oz = plus(M[3], -2.0f * M[12]);
         n[1] = kA1 * (Ex + Ox);
         n[2] = kA1 * (Ex - Ox);
         n[3] = kA1 * (Ey + Oy);
@@ -176,8 +182,8 @@ __device__ __forceinline__ void backward(const float M[19], float n[19])
         // xy plane
         const float Exy = base + M[5] + M[6] + M[17] + M[18];
         const float E7 = Exy + M[7], E8 = Exy - M[7];
-        const float oxy1 = M[1] + M[10] + M[13];  // x-odd part seen from the xy plane
-        const float oxy2 = M[2] + M[11] - M[14];  // y-odd part seen from the xy plane
+        const float oxy1 = plus(M[1], M[10]) + M[13];  // x-odd part seen from the xy plane
+        const float oxy2 = plus(M[2], M[11]) - M[14];  // y-odd part seen from the xy plane
         const float O7 = oxy1 + oxy2, O8 = oxy1 - oxy2;
         n[7] = kA2 * (E7 + O7);
         n[10] = kA2 * (E7 - O7);
@@ -186,8 +192,8 @@ __device__ __forceinline__ void backward(const float M[19], float n[19])
         // yz plane
         const float Eyz = base - 2.0f * M[5] - 2.0f * M[17];
         const float E11 = Eyz + M[8], E12 = Eyz - M[8];
-        const float oyz2 = M[2] + M[11] + M[14];  // y-odd part seen from the yz plane
-        const float oyz3 = M[3] + M[12] - M[15];  // z-odd part seen from the yz plane
+        const float oyz2 = plus(M[2], M[11]) + M[14];  // y-odd part seen from the yz plane
+        const float oyz3 = plus(M[3], M[12]) - M[15];  // z-odd part seen from the yz plane
         const float O11 = oyz2 + oyz3, O12 = oyz2 - oyz3;
         n[11] = kA2 * (E11 + O11);
         n[14] = kA2 * (E11 - O11);
@@ -196,8 +202,8 @@ __device__ __forceinline__ void backward(const float M[19], float n[19])
         // xz plane
         const float Exz = base + M[5] - M[6] + M[17] - M[18];
         const float E15 = Exz + M[9], E16 = Exz - M[9];
-        const float oxz1 = M[1] + M[10] - M[13];  // x-odd part seen from the xz plane
-        const float oxz3 = M[3] + M[12] + M[15];  // z-odd part seen from the xz plane
+        const float oxz1 = plus(M[1], M[10]) - M[13];  // x-odd part seen from the xz plane
+        const float oxz3 = plus(M[3], M[12]) + M[15];  // z-odd part seen from the xz plane
         const float O15 = oxz1 + oxz3, O16 = oxz1 - oxz3;
         n[15] = kA2 * (E15 + O15);
         n[18] = kA2 * (E15 - O15);
@@ -314,33 +320,17 @@ __device__ __forceinline__ float neg2log(float v, float d)
 // The angle is centred, 2 pi v2 = pi + 2 pi (v2 - 1/2) with v2 - 1/2 exact,
 // so the hardware sine / cosine see an argument in (-pi, pi), where their
 // absolute error is below 2^-21; cos and sin of the shifted angle change sign.
-// The pair has standard deviation sd (a factor of the radius: -2 ln v1 alone
-// goes through the reciprocal square root, so the amplitude of a node is one
-// square root however small it is).
-__device__ __forceinline__ void box_muller(uint32_t a, uint32_t b, float &g0, float &g1, float sd = 1.0f)
+__device__ __forceinline__ void box_muller(uint32_t a, uint32_t b, float &g0, float &g1)
 {
     const float v1 = uniform01(a);
     const float d1 = 1.0f - v1;  // exact for v1 >= 1/2, the only range where it is used
     const float w = uniform01(b) - 0.5f;
     const float L = neg2log(v1, d1);  // >= 2^-23
-    const float r = L * rsqrt_normal(L) * sd;
+    const float r = L * rsqrt_normal(L);
     float s, c;
     __sincosf(6.283185307179586f * w, &s, &c);
     g0 = -r * c;
     g1 = -r * s;
-}
-
-// Sixteen Gaussians of standard deviation sd for counter word 0, step, domain,
-// replica: Philox blocks b = 0..3 with counter (w0, step, domain<<8 | b, replica).
-__device__ __forceinline__ void gaussians16(const RoundKeys &rk, uint32_t w0, uint32_t step, uint32_t domain,
-                                            uint32_t replica, float sd, float g[16])
-{
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-        const U4 r = philox10(U4{w0, step, (domain << 8) | (uint32_t)b, replica}, rk);
-        box_muller(r.x, r.y, g[4 * b + 0], g[4 * b + 1], sd);
-        box_muller(r.z, r.w, g[4 * b + 2], g[4 * b + 3], sd);
-    }
 }
 
 // ---------------------------------------------------------------------------

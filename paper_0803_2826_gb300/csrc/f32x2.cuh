@@ -13,8 +13,9 @@
 // a packed form (reciprocal, log2, rsqrt, sine / cosine, the Philox integer
 // rounds, compares) run per half.  Every packed operation rounds each half
 // exactly as the scalar operation would, so the results are those of
-// d3q19.cuh / stream_collide.cuh's scalar code up to which multiply-adds the
-// compiler fuses there.
+// collide_node (stream_collide.cuh) up to which multiplications the assembler
+// joins with an addition behind them: with noise to the bit, without it but for
+// the last bit of some values where gamma_odd or gamma_even is not 0.
 #pragma once
 
 #include <cstdint>
@@ -214,8 +215,10 @@ constexpr float kLog3 = 0.666670024f, kLog4 = 0.499496400f, kLog5 = 0.423335731f
 // from the mantissa bits, -2 ln v1 from the hardware log2 or the series near
 // 1, the radius sqrt(-2 ln v1) as L rsqrt(L), the centred angle -- to FP32
 // rounding, with the arithmetic packed and the special functions per half.
-// nsd is minus the standard deviation: the sign of the centred angle's sine
-// and cosine costs nothing there, and a negation per half elsewhere.
+// nsd is minus the standard deviation (a factor of the radius: -2 ln v1 alone
+// goes through the reciprocal square root, so the amplitude of a node is one
+// square root however small it is; the sign of the centred angle's sine and
+// cosine costs nothing there, and a negation per half elsewhere).
 __device__ __forceinline__ void box_muller2(uint32_t a0, uint32_t b0, uint32_t a1, uint32_t b1, F2 &g0, F2 &g1,
                                             F2 nsd)
 {
@@ -244,6 +247,25 @@ __device__ __forceinline__ void box_muller2(uint32_t a0, uint32_t b0, uint32_t a
     __sincosf(ah, &s1, &c1);
     g0 = nr * f2(c0, c1);
     g1 = nr * f2(s0, s1);
+}
+
+// The same for one node.
+__device__ __forceinline__ void box_muller1(uint32_t a, uint32_t b, float &g0, float &g1, float nsd)
+{
+    const float v1 = lbd::one_to_two(a) - 0.99999994039535522f;
+    const float d1 = 1.0f - v1;
+    const float ang = fmaf(lbd::one_to_two(b) - 1.5f, 6.283185307179586f, 3.7450704e-07f);
+    const float lg = __fmul_rn(lbd::log2_normal(v1), -1.3862943611198906f);
+    float t = fmaf(d1, kLog5, kLog4);
+    t = fmaf(d1, t, kLog3);
+    t = fmaf(d1, t, 1.0f);
+    t = fmaf(d1, t, 2.0f);
+    const float L = d1 < 0.03125f ? __fmul_rn(d1, t) : lg;
+    const float nr = __fmul_rn(__fmul_rn(L, lbd::rsqrt_normal(L)), nsd);
+    float s, c;
+    __sincosf(ang, &s, &c);
+    g0 = __fmul_rn(nr, c);
+    g1 = __fmul_rn(nr, s);
 }
 
 // -sqrt(mu rho) of both nodes (mu rho0 where the amplitude is the reference's).
@@ -363,7 +385,7 @@ __device__ __forceinline__ void add_noise2(F2 M[19], F2 rho, const lbi::StepArgs
 }
 
 // Collision of nodes node0, node0 + 1 from their moments m and force densities
-// to the post-collision deviations out: lbi::collide_moments of each node, paired.
+// to the post-collision deviations out: lbi::collide_node of each node, paired.
 template <bool NOISE>
 __device__ __forceinline__ void collide_moments2(const F2 m[19], F2 fx, F2 fy, F2 fz, const lbi::StepArgs &a,
                                                  const lbd::RoundKeys &rk, uint32_t node0, uint32_t replica,

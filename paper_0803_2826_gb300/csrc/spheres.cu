@@ -579,9 +579,8 @@ __device__ __forceinline__ void sphere_node(const float *src, float *dst,
         fy += ld_f32(ffield + a.nn + self);
         fz += ld_f32(ffield + 2 * a.nn + self);
     }
-    float m[19], out[19];
-    lbd::forward(n, m);
-    collide_moments<NOISE>(m, fx, fy, fz, a, a.rk, (uint32_t)self, a.replica, out);
+    float out[19];
+    collide_node<NOISE>(n, fx, fy, fz, a, a.rk, (uint32_t)self, a.replica, out);
 #pragma unroll
     for (int i = 0; i < 19; ++i) dst[(size_t)i * P + self] = out[i];
 }

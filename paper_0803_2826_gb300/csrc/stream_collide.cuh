@@ -37,75 +37,71 @@ constexpr int kLinBX = 64;
 
 // Collision of one node (Sec. 3.4, 3.5, 3.7) from its pulled populations n
 // (deviations n_i - a_i rho0) and the force density (fx, fy, fz) to the
-// post-collision deviations out.  Physics constants come from a; the noise
-// stream is Philox with round keys rk and counter (node, a.step, b, replica).
-template <bool NOISE>
-__device__ __forceinline__ void collide_moments(const float m[19], float fx, float fy, float fz, const StepArgs &a,
-                                                const lbd::RoundKeys &rk, uint32_t node, uint32_t replica,
-                                                float out[19])
-{
-    const float rho = a.rho0 + m[0];
-    const float inv_rho = 1.0f / rho;
-    const float ux = (m[1] + 0.5f * fx) * inv_rho;
-    const float uy = (m[2] + 0.5f * fy) * inv_rho;
-    const float uz = (m[3] + 0.5f * fz) * inv_rho;
-
-    // ---- relaxation in moment space ----------------------------------------
-    const float uxx = ux * ux, uyy = uy * uy, uzz = uz * uz;
-    const float u2 = uxx + uyy + uzz;
-    const float meq4 = rho * u2;
-    const float meq5 = rho * (3.0f * uxx - u2);
-    const float meq6 = rho * (uyy - uzz);
-    const float meq7 = rho * ux * uy;
-    const float meq8 = rho * uy * uz;
-    const float meq9 = rho * uz * ux;
-    // forcing moments of Delta'' (Sigma of Eq. (moment_two_external_force))
-    const float uf = ux * fx + uy * fy + uz * fz;
-    const float gs1 = 1.0f + a.g_shear;
-    const float F4 = (1.0f + a.g_bulk) * uf;
-    const float F5 = gs1 * (3.0f * ux * fx - uf);
-    const float F6 = gs1 * (uy * fy - uz * fz);
-    const float F7 = 0.5f * gs1 * (ux * fy + uy * fx);
-    const float F8 = 0.5f * gs1 * (uy * fz + uz * fy);
-    const float F9 = 0.5f * gs1 * (uz * fx + ux * fz);
-
-    float M[19];  // post-collision moments divided by w_k
-    M[0] = m[0];
-    M[1] = 3.0f * (m[1] + fx);
-    M[2] = 3.0f * (m[2] + fy);
-    M[3] = 3.0f * (m[3] + fz);
-    M[4] = lbd::inv_w(4) * (meq4 + a.g_bulk * (m[4] - meq4) + F4);
-    M[5] = lbd::inv_w(5) * (meq5 + a.g_shear * (m[5] - meq5) + F5);
-    M[6] = lbd::inv_w(6) * (meq6 + a.g_shear * (m[6] - meq6) + F6);
-    M[7] = lbd::inv_w(7) * (meq7 + a.g_shear * (m[7] - meq7) + F7);
-    M[8] = lbd::inv_w(8) * (meq8 + a.g_shear * (m[8] - meq8) + F8);
-    M[9] = lbd::inv_w(9) * (meq9 + a.g_shear * (m[9] - meq9) + F9);
-#pragma unroll
-    for (int k = 10; k < 16; ++k) M[k] = lbd::inv_w(k) * (a.g_odd * m[k]);
-#pragma unroll
-    for (int k = 16; k < 19; ++k) M[k] = lbd::inv_w(k) * (a.g_even * m[k]);
-
-    if (NOISE) {
-        // sqrt(mu rho w_k) phi_k r_k, divided by w_k: (phi_k / sqrt(w_k)) times a
-        // Gaussian of variance mu rho (the factor rides in the Box-Muller radius)
-        float g[16];
-        lbd::gaussians16(rk, node, a.step, 0u, replica, sqrtf(a.mu * (a.noise_rho0 ? a.rho0 : rho)), g);
-#pragma unroll
-        for (int k = 4; k < 19; ++k) M[k] = fmaf(a.amp[k - 4], g[k - 4], M[k]);
-    }
-
-    lbd::backward(M, out);
-}
-
-// The same from the pulled populations n (deviations n_i - a_i rho0).
+// post-collision deviations out: lbp::relax2, add_noise2 and backward2 for one
+// node, operation by operation, so that a node that is updated again by itself
+// (impulse nodes, nodes next to spheres) rounds as its neighbours in the packed
+// update do.  (What multiplications the assembler joins with an addition behind
+// them can still differ.)  The noise stream is Philox with round keys rk and
+// counter (node, a.step, b, replica).
 template <bool NOISE>
 __device__ __forceinline__ void collide_node(const float n[19], float fx, float fy, float fz, const StepArgs &a,
                                              const lbd::RoundKeys &rk, uint32_t node, uint32_t replica,
                                              float out[19])
 {
     float m[19];
-    lbd::forward(n, m);
-    collide_moments<NOISE>(m, fx, fy, fz, a, rk, node, replica, out);
+    lbd::forward<true>(n, m);
+    const float rho = a.rho0 + m[0];
+    const float inv_rho = __frcp_rn(rho);
+    const float ux = __fmul_rn(fmaf(0.5f, fx, m[1]), inv_rho);
+    const float uy = __fmul_rn(fmaf(0.5f, fy, m[2]), inv_rho);
+    const float uz = __fmul_rn(fmaf(0.5f, fz, m[3]), inv_rho);
+    const float uxx = __fmul_rn(ux, ux), uyy = __fmul_rn(uy, uy), uzz = __fmul_rn(uz, uz);
+    const float u2 = uxx + uyy + uzz;
+    const float ruy = __fmul_rn(rho, uy), nrho = -a.rho0 - m[0], nruy = __fmul_rn(nrho, uy);
+    const float t5 = __fmul_rn(uxx, 3.0f) - u2, t6 = uyy - uzz;
+    float S[6] = {__fmul_rn(rho, u2), __fmul_rn(rho, t5), __fmul_rn(rho, t6),
+                  __fmul_rn(ruy, ux), __fmul_rn(ruy, uz), __fmul_rn(__fmul_rn(rho, uz), ux)};
+    const float d[6] = {fmaf(nrho, u2, m[4]), fmaf(nrho, t5, m[5]), fmaf(nrho, t6, m[6]),
+                        fmaf(nruy, ux, m[7]), fmaf(nruy, uz, m[8]), fmaf(__fmul_rn(nrho, uz), ux, m[9])};
+    float M[19];
+    M[0] = m[0];
+    M[1] = m[1];
+    M[2] = m[2];
+    M[3] = m[3];
+    if (a.forced) {
+        const float xx = __fmul_rn(ux, fx), yy = __fmul_rn(uy, fy), zz = __fmul_rn(uz, fz);
+        const float uf = xx + yy + zz;
+        S[0] = fmaf(uf, a.frc[0], S[0]);
+        S[1] = fmaf(__fmul_rn(xx, 3.0f) - uf, a.frc[1], S[1]);
+        S[2] = fmaf(yy - zz, a.frc[1], S[2]);
+        S[3] = fmaf(__fmul_rn(ux, fy) + __fmul_rn(uy, fx), a.frc[2], S[3]);
+        S[4] = fmaf(__fmul_rn(uy, fz) + __fmul_rn(uz, fy), a.frc[2], S[4]);
+        S[5] = fmaf(__fmul_rn(uz, fx) + __fmul_rn(ux, fz), a.frc[2], S[5]);
+        M[1] += fx;
+        M[2] += fy;
+        M[3] += fz;
+    }
+#pragma unroll
+    for (int k = 4; k < 10; ++k)
+        M[k] = __fmul_rn(fmaf(d[k - 4], k == 4 ? a.g_bulk : a.g_shear, S[k - 4]), lbd::inv_w(k));
+#pragma unroll
+    for (int k = 10; k < 19; ++k) M[k] = __fmul_rn(m[k], a.rel[k - 10]);
+    if (NOISE) {
+        const float nsd = -sqrtf(a.noise_rho0 ? a.mu * a.rho0 : __fmul_rn(rho, a.mu));
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            const lbd::U4 r = lbd::philox10(lbd::U4{node, a.step, (uint32_t)b, replica}, rk);
+            float g[4];
+            lbp::box_muller1(r.x, r.y, g[0], g[1], nsd);
+            lbp::box_muller1(r.z, r.w, g[2], g[3], nsd);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int k = 4 + 4 * b + j;
+                if (k < 19) M[k] = fmaf(g[j], a.amp[k - 4], M[k]);
+            }
+        }
+    }
+    lbd::backward<true>(M, out);
 }
 
 // One step of a butterfly reduce-scatter over the warp: each lane keeps one
@@ -230,9 +226,8 @@ __device__ __forceinline__ void update_node(const typename lbd::Store<DT>::T *__
             fz += ld_f32(facc + 2 * P + self);
         }
     }
-    float m[19], out[19];
-    lbd::forward(n, m);
-    collide_moments<NOISE>(m, fx, fy, fz, a, a.rk, self, a.replica, out);
+    float out[19];
+    collide_node<NOISE>(n, fx, fy, fz, a, a.rk, self, a.replica, out);
 #pragma unroll
     for (int i = 0; i < 19; ++i)
         if (in_bounds((size_t)i * P + self, 19 * P, a.err)) dst[(size_t)i * P + self] = S::pack(out[i], a.scale);
@@ -283,7 +278,7 @@ __device__ __forceinline__ void clear_outside(float *facc, const StepArgs &a, in
 // updated again from the same pre-step state
 // with the impulses added.  The update of a node depends only on that state, the
 // forces at the node and the counter-based noise, so the result is the one a
-// single update with the impulses would give.  Thread (p, q) walks p's
+// single update with the impulses would give (collide_node).  Thread (p, q) walks p's
 // distinct cells and takes nodes q, q + 8, ... of each; a node shared by several
 // particles is updated once, by the thread that raises its tag to `tag`
 // first (tags grow by one per patch, so the array is never cleared).
@@ -1069,7 +1064,8 @@ cudaError_t launch_patch_dt(const lb_handle *h, const void *src, void *dst, floa
                             int n, int nsub, int span, unsigned int *claim, unsigned int tag)
 {
     using T = typename lbd::Store<DT>::T;
-    const StepArgs a = make_args(h);
+    StepArgs a = make_args(h);
+    a.forced = 1;
     if (n <= 0 || nsub <= 0) return cudaSuccess;
     const unsigned int blocks = (unsigned int)(((size_t)n * 8 + kBX - 1) / kBX);
     const T *s = static_cast<const T *>(src);
