@@ -88,9 +88,11 @@ __device__ __forceinline__ void push_pair(float *lam_out, const StepArgs &a, con
             if (in_bounds(k + 1, 19 * P, a.err)) Pair<0>::store(lam_out + k, v0, v1, 1.0f);
             continue;
         }
-        float *row = lam_out + ((size_t)i * P + p.z[1 - lbd::cz(i)] + p.y[1 - lbd::cy(i)]);
-        row[lbd::cx(i) == 1 ? xm : at.x + 1] = v0;
-        row[lbd::cx(i) == 1 ? at.x : xp] = v1;
+        const size_t row = (size_t)i * P + p.z[1 - lbd::cz(i)] + p.y[1 - lbd::cy(i)];
+        const size_t k0 = row + (uint32_t)(lbd::cx(i) == 1 ? xm : at.x + 1);
+        const size_t k1 = row + (uint32_t)(lbd::cx(i) == 1 ? at.x : xp);
+        if (in_bounds(k0, 19 * P, a.err)) lam_out[k0] = v0;
+        if (in_bounds(k1, 19 * P, a.err)) lam_out[k1] = v1;
     }
 }
 
