@@ -591,8 +591,10 @@ lb_status lb_adjoint_forward(lb_handle *h, int nsteps, int checkpoint_every, con
     // Each step writes its result where it is needed: a checkpoint at the end
     // of a segment, the segment states themselves in the last segment (the
     // reverse pass then has nothing to recompute there), the handle's buffers
-    // otherwise and at the end.
+    // otherwise and at the end: the one lb_step would have ended in, so that a
+    // captured call with an even number of steps can be replayed on its result.
     const int last0 = (nsteps - 1) / K * K;  // first step of the last segment
+    void *const end = h->pops[(h->cur + nsteps) & 1];
     void *src = h->pops[h->cur];
     e = cudaMemcpyAsync(b.ckpt[0], src, 19 * h->pitch * h->elem, cudaMemcpyDeviceToDevice, h->stream);
     for (int t = 0; t < nsteps && e == cudaSuccess; ++t) {
@@ -600,6 +602,7 @@ lb_status lb_adjoint_forward(lb_handle *h, int nsteps, int checkpoint_every, con
         void *dst = h->pops[other];
         if (t + 1 < nsteps && (t + 1) % K == 0) dst = b.ckpt[(t + 1) / K];
         else if (t + 1 < nsteps && t >= last0) dst = b.seg[t + 1 - last0];
+        else if (t + 1 == nsteps) dst = end;  // (src is a checkpoint or a segment state, or nsteps is 1)
         timer_mark(h, 0, 0, h->stream);
         e = step_from(h, src, dst, step0 + (uint32_t)t);
         timer_mark(h, 0, 1, h->stream);
@@ -607,7 +610,7 @@ lb_status lb_adjoint_forward(lb_handle *h, int nsteps, int checkpoint_every, con
         src = dst;
     }
     if (e != cudaSuccess) return cuda_fail("lb_adjoint_forward", e);
-    h->cur = src == h->pops[0] ? 0 : 1;
+    h->cur = (h->cur + nsteps) & 1;
     h->step = step0 + (uint32_t)nsteps;
     // the loss and its seed lambda_T = dL/dstate at the final state (first
     // adjoint buffer) with its own dL/df (gseed), for lb_adjoint_backward.
