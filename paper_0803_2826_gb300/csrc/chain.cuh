@@ -75,7 +75,9 @@ cudaError_t launch_chained(void (*kernel)(K...), dim3 grid, dim3 block, cudaStre
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = attr;
     lc.numAttrs = 1;
-    return cudaLaunchKernelEx(&lc, kernel, static_cast<K>(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&lc, kernel, static_cast<K>(args)...);
+    if (e != cudaSuccess) (void)cudaGetLastError();  // reported here, not again by the next call that looks
+    return e;
 }
 
 }  // namespace lbi
