@@ -311,8 +311,8 @@ struct RunningKeys {
 // moments over w_k, M, and the densities.  The noisy update is bound by
 // instruction issue, so constants are multiplied on the host where that costs
 // no accuracy and the forcing is passed over where nothing forces; with the
-// Box-Muller map above, 256^3 FP16 373 us a step (396 before), 512 replicas
-// 1.25 ms (1.29), 200^3 FP32 178 us (188), 256^3 FP32 364 us (382).
+// Box-Muller map above, 256^3 FP16 376 us a step (396 before), 512 replicas
+// 1.26 ms (1.29), 200^3 FP32 180 us (188), 256^3 FP32 365 us (382).
 __device__ __forceinline__ void relax2(const F2 m[19], F2 fx, F2 fy, F2 fz, const lbi::StepArgs &a, F2 M[19], F2 &rho)
 {
     const F2 half = f2s(0.5f), three = f2s(3.0f);

@@ -399,9 +399,8 @@ __device__ __forceinline__ void stencil_coords(const int o[3], int q, const Step
     else z = wrap_node(z, g.nz);
 }
 
-// The record of a particle's sub-step, which the overlapped step's
-// re-update and the clearing of applied impulses expand to a block of
-// record_span^3 nodes: for phi_2 and phi_4 the linear index of the
+// The record of a particle's sub-step (overlapped calls), which the step's
+// re-update of impulse nodes expands to a block of record_span^3 nodes: for phi_2 and phi_4 the linear index of the
 // particle's cell (the block is the cell's corners, resp. one node further
 // on each side: the stencil), for phi_3 the wrapped stencil origin (the
 // block is the 27-node stencil itself, not the 64 nodes around the cell).
@@ -1364,12 +1363,11 @@ __device__ __forceinline__ void couple_persistent_run(const PersistArgs &a)
 }
 
 // The phi_2 persistent coupling.  168 registers, no spills: beside the
-// stream-collide launch of a 256^3 box (80 registers) it leaves four of that
-// kernel's six blocks on the SMs it shares, and ends in 0.22 ms; capped at
-// 112 registers it left five but spilled and took 0.40 ms, for the same
-// stream-collide time (0.41 ms) and a longer step (0.4289 against 0.4257 ms).
-// Blocks of 256 or 512 particles on fewer SMs slowed the launch beside them
-// more (0.418 ms).
+// stream-collide launch of a 256^3 box (72 registers) it leaves four of that
+// kernel's seven blocks on the SMs it shares.  Capped at 112 registers it would
+// leave five, but it spills and takes longer: 16384 monomers with ten
+// sub-steps, 433 to 436 us a step against 428 us.  Blocks of 256 or 512
+// particles on fewer SMs slowed the launch beside them more.
 template <int DT>
 __global__ void __launch_bounds__(kPThreads) k_couple_persistent(PersistArgs a)
 {

@@ -674,13 +674,14 @@ __global__ void __launch_bounds__(kBX)
 }
 
 // The same where a force field is read: room for seven blocks of 128 threads
-// per SM (FP32) or eight (FP16 / BF16).  The update wants warps more than
-// registers, and these kernels carry a few more registers than six blocks
-// leave room for (256^3 FP32 between walls with a field 412 us against 443 us a
-// step, 512 x 512 x 256 FP16 1576 us against 1612 us, for 24 to 88 bytes of
-// spills).  Without a field the compiler's own choice, 72 registers, is the
-// best (256^3 FP32 365 us; 371 us with room for six or seven blocks, 383 us for
-// eight).
+// per SM in FP32 (72 registers, no spills) and for eight in FP16 / BF16 (64
+// registers, 24 to 72 bytes of spills), where the update wants warps more than
+// registers: 512^3 FP16 between walls with the impulses of 1e5 tracers 3.43 ms a
+// step against 3.49 ms with the compiler's own 72 to 74 registers.  Elsewhere
+// the two are close: 512 x 512 x 256 FP16 1597 against 1590 us, 256^3 FP32
+// between walls 407 against 412 us, 200^3 FP32 204 against 201 us.  Without a
+// field the compiler's own choice, 72 registers, is the best (256^3 FP32 365 us;
+// 371 us with room for six or seven blocks, 383 us for eight).
 template <int DT>
 constexpr int field_blocks() { return DT == 0 ? 7 : 8; }
 
