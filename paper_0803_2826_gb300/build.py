@@ -18,8 +18,9 @@ INCLUDE = os.path.join(ROOT, "include")
 OUT = os.path.join(PKG, "liblbfluct.so")
 BUILD = os.path.join(ROOT, "_build")
 # the index-checking variant (-DLB_DEBUG_BOUNDS): every population pull and
-# store and every particle spread index is tested against its array first; a
-# violation sets LB_DERR_BOUNDS in the handle's error word and skips the access
+# store of the update, batch and field kernels, every store of the reverse step
+# and every particle spread index is tested against its array first; a violation
+# sets LB_DERR_BOUNDS in the handle's error word and skips the access
 OUT_BOUNDS = os.path.join(PKG, "liblbfluct_bounds.so")
 BUILD_BOUNDS = os.path.join(ROOT, "_build", "bounds")
 
